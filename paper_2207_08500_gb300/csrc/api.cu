@@ -39,6 +39,7 @@ struct neno6_handle {
   double* d_vjp_rhs = nullptr;     // dU/dt of that forward pass (lazily)
   double* d_vjp_contrib = nullptr; // per-face adjoint contributions (lazily)
   float* d_params32 = nullptr;     // FP32 parameters, weights-file order
+  double* d_net64 = nullptr;       // classifier blob of the FP64 kernels (kNetBlobBytes)
   void* d_bwd_scratch = nullptr;   // per-CTA partial gradients (lazily)
   unsigned long long* d_guard_count = nullptr;
   cudaStream_t copy_stream = nullptr;  // neno6_step_host: band copies in and out (lazily)
@@ -46,7 +47,7 @@ struct neno6_handle {
   cudaEvent_t band_done[9] = {};       // band of the last stage done; [8]: all copied out
   FacesMixedArgs faces_args;
   size_t state_elems = 0;
-  RhsParamsF64 rhs_params;        // launch parameter blocks (copied at launch)
+  RhsArgs rhs_args;               // launch parameter blocks (copied at launch)
   ClassifyParamsF64 cls_params;
   ScalarParams scalar_params;
   std::string err;
@@ -300,6 +301,8 @@ void fill_rhs_args(const neno6_handle* h, RhsArgs& a) {
   a.two_thirds = 2.0 / 3.0;
   a.mask_mode = h->cfg.mask_mode;
   a.status = h->d_status;
+  a.net64 = h->d_net64;
+  a.filter = reinterpret_cast<const float*>(h->d_net64 + kNetParams);
   std::memcpy(a.cand, h->cand, sizeof a.cand);
   std::memcpy(a.wtab, h->wtab, sizeof a.wtab);
   if (a.mask_mode == kMaskTeno) teno_tables(a.teno);
@@ -579,6 +582,10 @@ int neno6_create(const neno6_config* cfg, const char* weights_path, neno6_handle
     e = cudaMalloc(&h->d_params32, kNetParams * sizeof(float));
     if (e == cudaSuccess) e = cudaMemcpy(h->d_params32, p32.data(), kNetParams * sizeof(float), cudaMemcpyHostToDevice);
   }
+  if (e == cudaSuccess && !h->narrow) {
+    e = cudaMalloc(&h->d_net64, kNetBlobBytes);
+    if (e == cudaSuccess) e = launch_net_blob(h->net, h->d_net64, nullptr);
+  }
   if (e == cudaSuccess && c.precision != NENO6_FP64) {
     std::vector<uint8_t> img(kNetImageBytes);
     if (h->narrow)
@@ -630,6 +637,7 @@ int neno6_destroy(neno6_handle* h) {
   cudaFree(h->d_vjp_rhs);
   cudaFree(h->d_vjp_contrib);
   cudaFree(h->d_params32);
+  cudaFree(h->d_net64);
   cudaFree(h->d_bwd_scratch);
   for (cudaEvent_t ev : h->band_in)
     if (ev) cudaEventDestroy(ev);
@@ -661,16 +669,15 @@ int neno6_rhs(neno6_handle* h, const double* U, double* dUdt, const uint8_t* mas
   }
   if (!aligned(U, 16) || !aligned(dUdt, 16)) return fail(h, NENO6_ERR_ALIGN, "rhs: U/dUdt must be 16-byte aligned");
   if ((const void*)U == (const void*)dUdt) return fail(h, NENO6_ERR_ARG, "rhs: dUdt must not alias U");
-  RhsParamsF64& p = h->rhs_params;
-  fill_rhs_args(h, p.a);
-  p.a.U = U;
-  p.a.out = dUdt;
-  p.a.mask_in = mask_in;
-  p.a.mask_out = mask_out;
-  if (mask_in) p.a.mask_mode = kMaskGiven;
-  p.a.stage = 0;
-  p.net = h->net;
-  cudaError_t e = launch_rhs_fp64(h->cfg.ndim, p, (cudaStream_t)stream);
+  RhsArgs& a = h->rhs_args;
+  fill_rhs_args(h, a);
+  a.U = U;
+  a.out = dUdt;
+  a.mask_in = mask_in;
+  a.mask_out = mask_out;
+  if (mask_in) a.mask_mode = kMaskGiven;
+  a.stage = 0;
+  cudaError_t e = launch_rhs_fp64(h->cfg.ndim, a, (cudaStream_t)stream);
   if (e != cudaSuccess) return cuda_fail(h, e, "rhs launch");
   return NENO6_OK;
 }
@@ -691,23 +698,22 @@ int neno6_step(neno6_handle* h, double* U, double cfl, double t_end, double* t_d
   double* S2 = h->d_stage + h->state_elems;
   cudaError_t e = launch_cfl_reduce(h->cfg.ndim, U, h->cfg.nx, h->cfg.ny, h->cfg.gamma, h->d_smax, h->d_status, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "step: cfl reduction");
-  RhsParamsF64& p = h->rhs_params;
-  fill_rhs_args(h, p.a);
-  p.a.smax = h->d_smax;
-  p.a.dt_dev = h->d_dt;
-  p.a.t_dev = t_dev ? t_dev : h->d_t;
-  p.a.dt_user = dt_dev;
-  p.a.cfl = cfl;
-  p.a.t_end = t_end;
-  p.a.U0 = U;
-  p.net = h->net;
+  RhsArgs& a = h->rhs_args;
+  fill_rhs_args(h, a);
+  a.smax = h->d_smax;
+  a.dt_dev = h->d_dt;
+  a.t_dev = t_dev ? t_dev : h->d_t;
+  a.dt_user = dt_dev;
+  a.cfl = cfl;
+  a.t_end = t_end;
+  a.U0 = U;
   const double* in[3] = {U, S1, S2};
   double* outp[3] = {S1, S2, U};
   for (int st = 1; st <= 3; ++st) {
-    p.a.stage = st;
-    p.a.U = in[st - 1];
-    p.a.out = outp[st - 1];
-    e = launch_rhs_fp64(h->cfg.ndim, p, s);
+    a.stage = st;
+    a.U = in[st - 1];
+    a.out = outp[st - 1];
+    e = launch_rhs_fp64(h->cfg.ndim, a, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "step: stage launch");
   }
   return NENO6_OK;
@@ -800,7 +806,7 @@ int neno6_rhs_vjp(neno6_handle* h, const double* U, const double* lambda, const 
     return fail(h, NENO6_ERR_ALIGN, "rhs_vjp: arrays must be 16-byte aligned");
   if (grad_U == U || grad_U == lambda) return fail(h, NENO6_ERR_ARG, "rhs_vjp: grad_U must not alias an input");
   cudaStream_t s = (cudaStream_t)stream;
-  RhsParamsF64& p = h->rhs_params;
+  RhsArgs& a = h->rhs_args;
   if (!mask) {
     // recompute the classifier mask of U with the FP64 path (bit-identical
     // to the forward FP64 right-hand side)
@@ -808,13 +814,12 @@ int neno6_rhs_vjp(neno6_handle* h, const double* U, const double* lambda, const 
     if (!h->d_mask) e = cudaMalloc(&h->d_mask, (size_t)neno6_mask_bytes(h));
     if (e == cudaSuccess && !h->d_vjp_rhs) e = cudaMalloc(&h->d_vjp_rhs, h->state_elems * sizeof(double));
     if (e != cudaSuccess) return cuda_fail(h, e, "rhs_vjp: mask buffers");
-    fill_rhs_args(h, p.a);
-    p.a.U = U;
-    p.a.out = h->d_vjp_rhs;
-    p.a.mask_out = h->d_mask;
-    p.a.stage = 0;
-    p.net = h->net;
-    e = launch_rhs_fp64(h->cfg.ndim, p, s);
+    fill_rhs_args(h, a);
+    a.U = U;
+    a.out = h->d_vjp_rhs;
+    a.mask_out = h->d_mask;
+    a.stage = 0;
+      e = launch_rhs_fp64(h->cfg.ndim, a, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "rhs_vjp: forward");
     mask = h->d_mask;
   }
@@ -825,10 +830,10 @@ int neno6_rhs_vjp(neno6_handle* h, const double* U, const double* lambda, const 
       return cuda_fail(h, e, "rhs_vjp: contribution buffer");
     }
   }
-  fill_rhs_args(h, p.a);
-  p.a.U = U;
-  p.a.mask_in = mask;
-  cudaError_t e = launch_rhs_vjp(h->cfg.ndim, p.a, lambda, grad_U, h->d_vjp_contrib, s);
+  fill_rhs_args(h, a);
+  a.U = U;
+  a.mask_in = mask;
+  cudaError_t e = launch_rhs_vjp(h->cfg.ndim, a, lambda, grad_U, h->d_vjp_contrib, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "rhs_vjp launch");
   return NENO6_OK;
 }

@@ -9,177 +9,152 @@
 // nor reorder it; the classifier masks are therefore a deterministic function
 // of the state, identical on any IEEE-754 implementation of that order.
 //
-// Design (GB300): binary64 arithmetic runs on the SM's FP64 pipe, and the
-// classifier (3104 multiply-adds per call, 16 calls per cell and RHS) is ~97 %
-// of the work, so this kernel is bound by that pipe.  Each CTA owns a tile of
-// cells, stages the tile plus a 3-cell halo (periodic wrap or zero-gradient
-// copy done in the load) and every per-cell quantity in shared memory once,
-// then runs one work item per (face, characteristic field) with four lanes
-// per face.  Classifier weights live in the kernel's parameter block
-// (constant bank), so the multiply-adds take the weight as a constant operand
-// and the warp reads it by broadcast.  Cheap comparisons (ReLU, max, |x|) are
-// done on the integer pipe on the bit patterns to keep the FP64 pipe for the
-// arithmetic.
+// Design (GB300): the binary64 pipe issues two lanes per clock and SM, 1/61 of
+// the FP32 pipe's rate, so the classifier (3104 multiply-adds per stencil, 16
+// stencils per cell and RHS) is evaluated in FP32 with a certified bound and in
+// binary64 only where the bound does not settle a logit's sign
+// (mlp_filter.cuh).  What stays on the FP64 pipe is the reconstruction itself,
+// ~1150 operations per cell, and each is done once: a thread takes a face
+// with all its characteristic fields, so the Roe state is formed once per face.
+// Persistent CTAs take tiles of cells: the tile plus a 3-cell halo (periodic
+// wrap or zero-gradient copy done in the load) and the per-cell quantities are
+// staged in shared memory, the faces' fluxes written back there and
+// differenced, with no scratch in global memory.  Comparisons (ReLU, max, |x|)
+// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 14.4 ms,
+// against 437 ms with every classifier row in binary64 and four lanes per
+// face; the FP64 operations alone would take 7.8 ms of a full FP64 pipe.
+#include <cmath>
+
 #include "fp64_ops.cuh"
 #include "internal.h"
-#include "tc.cuh"
+#include "mlp_filter.cuh"
 
 namespace neno6 {
 namespace {
 
 using namespace f64ops;
 
-constexpr int kThreads = 256;
-
-template <int NDIM>
-struct Geom;
-// Staged tile: TX x TY cells and a 3-cell halo; staged column bx holds
-// global column i0 - X0 + bx.  In 2D the tile's rows are 40 cells wide
-// (i0-4 .. i0+35) so that a TMA copy of the box can start on a 16-byte
-// boundary (an even float64 column); the outer two columns are staged but
-// never read.
-template <>
-struct Geom<2> {
-  static constexpr int TX = 32, TY = 16, HY = 3, NV = 4;
-  static constexpr int X0 = 4, SX = TX + 8, SY = TY + 6;
-  static constexpr int NXF = TY * (TX + 1);  // x faces of a tile
-  static constexpr int NYF = (TY + 1) * TX;  // y faces of a tile
-};
-template <>
-struct Geom<1> {
-  static constexpr int TX = 63, TY = 1, HY = 0, NV = 3;
-  static constexpr int X0 = 3, SX = TX + 6, SY = 1;
-  static constexpr int NXF = TX + 1;
-  static constexpr int NYF = 0;
-};
-
-// Per-cell arrays staged in shared memory (structure of arrays).
-template <int NV>
-struct CellArrays {
-  static constexpr int U = 0;                // NV conserved variables
-  static constexpr int u = NV, v = NV + 1, c = NV + 2, H = NV + 3, s = NV + 4;
-  static constexpr int Fx = NV + 5;          // NV x-fluxes
-  static constexpr int Fy = Fx + NV;         // NV y-fluxes (2D)
-  static constexpr int N = Fy + NV;
+// Tile of TX x TY cells (TY = 1 in 1D) worked on by NT threads, OCC CTAs per
+// SM.  Faces are dealt to warps in runs of 32 of one direction.  SPLIT: a
+// warp's item is one characteristic field of 32 faces instead of all of them
+// (the Roe state is then formed NV times over).
+template <int NDIM_, int TX_, int TY_, int NT_, int OCC_, bool SPLIT_>
+struct Tile {
+  static constexpr int NDIM = NDIM_, TX = TX_, TY = TY_, NT = NT_, OCC = OCC_;
+  static constexpr bool SPLIT = SPLIT_;
+  static constexpr int NV = NDIM == 2 ? 4 : 3;
+  static constexpr int HY = NDIM == 2 ? 3 : 0;
+  static constexpr int SX = TX + 6, SY = TY + 2 * HY, NC = SX * SY;
+  static constexpr int NXF = TY * (TX + 1);                   // x faces
+  static constexpr int NYF = NDIM == 2 ? (TY + 1) * TX : 0;   // y faces
+  static constexpr int WX = (NXF + 31) / 32, WY = (NYF + 31) / 32;  // runs of 32 faces
+  // staged planes of NC values: U[NV], u, (v,) c, H, sqrt(rho), then the
+  // fluxes but the mass flux (which is a momentum): x, then y
+  static constexpr int P_U = 0, P_u = NV, P_v = NV + 1, P_c = NV + NDIM, P_H = P_c + 1, P_s = P_c + 2;
+  static constexpr int P_F = P_c + 3;
+  static constexpr int NPLANES = P_F + NDIM * (NV - 1);
+  static constexpr int kPark = 12;  // per thread: the "+" stencil, the mirrored "-" stencil
+  static constexpr int kScratch = 128;  // per warp (binary64 classifier)
+  // doubles: planes, face fluxes, parked stencils, warp scratch, and for
+  // SPLIT the faces' field fluxes and Roe states; then the FP32 table
+  static constexpr int O_F = NPLANES * NC;
+  static constexpr int O_P = O_F + NV * (NXF + NYF);
+  static constexpr int O_W = O_P + kPark * NT;
+  static constexpr int O_G = O_W + kScratch * (NT / 32);
+  static constexpr int O_T = (O_G + (SPLIT ? (NV + 5) * (NXF + NYF) : 0) + 1) / 2 * 2;
+  static constexpr size_t SMEM = sizeof(double) * O_T + sizeof(float) * kFiltFloats;
+  static_assert(NT % 32 == 0 && OCC * (SMEM + 1024) <= 228 * 1024, "resident CTAs");
 };
 
-// Per-thread slot parked in shared memory while the classifier runs (keeps
-// the stencils and the R row out of registers): "+" stencil, mirrored "-"
-// stencil, R row.
-constexpr int kPark = 16;
-
-template <int NDIM>
-constexpr size_t rhs_smem_bytes() {
-  using G = Geom<NDIM>;
-  // ... then one mbarrier (the tile's TMA copy)
-  return sizeof(double) * (size_t(CellArrays<G::NV>::N) * G::SX * G::SY +
-                           size_t(G::NV) * G::TY * (G::TX + 1) +
-                           size_t(G::NV) * (G::TY + 1) * G::TX + size_t(kPark) * kThreads + 1);
+// x is 0 or its magnitude lies in [2^-60, 2^60).
+__device__ __forceinline__ bool moderate(double x) {
+  const unsigned long long b = (unsigned long long)dbits(x) & 0x7fffffffffffffffULL;
+  return b == 0ull || (unsigned)(b >> 32) - (963u << 20) < (120u << 20);
+}
+// x / 2 for x = 0 or 2^-1021 <= |x| < inf, on the integer pipe.
+__device__ __forceinline__ double half_exact(double x) {
+  const int hi = __double2hiint(x);
+  return __hiloint2double((hi & 0x7ff00000) ? hi - 0x00100000 : hi, __double2loint(x));
 }
 
-// The 2D tile at (i0, j0) is copied by TMA: U described by the tensor map
-// (in the parameter space, 64-byte aligned) and the whole staged box inside
-// the grid (no periodic wrap, no clamp).  The box's first column i0 - 4 is
-// even, hence 16-byte aligned.
-__device__ __forceinline__ bool tile_by_tma(const RhsArgs& a, int i0, int j0) {
-  using G = Geom<2>;
-  return a.use_tma && (reinterpret_cast<uintptr_t>(&a.tmap) & 63u) == 0 && i0 - G::X0 >= 0 &&
-         i0 - G::X0 + G::SX <= a.nx && j0 - G::HY >= 0 && j0 - G::HY + G::SY <= a.ny;
+// Roe-averaged state of a face (Sec. 4.4).
+struct Roe {
+  double ut, vt, Ht, ct, ic, b1, b2, qt;
+};
+
+// Row m of R applied to the field fluxes g: component n of the face flux.
+template <int NDIM>
+__device__ __forceinline__ double back_project(const Roe& r, int dir, int n, const double (&g)[4]) {
+  constexpr int NV = NDIM == 2 ? 4 : 3;
+  double R[4];
+  const double ntc = __dmul_rn(dir == 0 ? r.ut : r.vt, r.ct);
+  if (NDIM == 1) {
+    if (n == 0) { R[0] = 1.0; R[1] = 1.0; R[2] = 1.0; }
+    else if (n == 1) { R[0] = __dsub_rn(r.ut, r.ct); R[1] = r.ut; R[2] = __dadd_rn(r.ut, r.ct); }
+    else { R[0] = __dsub_rn(r.Ht, ntc); R[1] = __dmul_rn(0.5, r.qt); R[2] = __dadd_rn(r.Ht, ntc); }
+    R[3] = 0.0;
+  } else if (n == 0) {
+    R[0] = 1.0; R[1] = 1.0; R[2] = 0.0; R[3] = 1.0;
+  } else if (n == 1) {
+    if (dir == 0) { R[0] = __dsub_rn(r.ut, r.ct); R[1] = r.ut; R[2] = 0.0; R[3] = __dadd_rn(r.ut, r.ct); }
+    else { R[0] = r.ut; R[1] = r.ut; R[2] = 1.0; R[3] = r.ut; }
+  } else if (n == 2) {
+    if (dir == 0) { R[0] = r.vt; R[1] = r.vt; R[2] = 1.0; R[3] = r.vt; }
+    else { R[0] = __dsub_rn(r.vt, r.ct); R[1] = r.vt; R[2] = 0.0; R[3] = __dadd_rn(r.vt, r.ct); }
+  } else {
+    R[0] = __dsub_rn(r.Ht, ntc); R[1] = __dmul_rn(0.5, r.qt); R[2] = dir == 0 ? r.vt : r.ut;
+    R[3] = __dadd_rn(r.Ht, ntc);
+  }
+  double F = __dmul_rn(R[0], g[0]);
+#pragma unroll
+  for (int q = 1; q < NV; ++q) F = __fma_rn(R[q], g[q], F);
+  return F;
 }
 
+// Row m of L in the Roe/Toro scaling.
 template <int NDIM>
-__global__ void __launch_bounds__(kThreads, 1) rhs_fp64_kernel(const __grid_constant__ RhsParamsF64 P) {
-  using G = Geom<NDIM>;
-  using CA = CellArrays<G::NV>;
-  constexpr int NV = G::NV, SX = G::SX, SY = G::SY, NC = SX * SY;
-  constexpr int TX = G::TX, TY = G::TY;
-  extern __shared__ __align__(1024) double smem[];
-  double* C = smem;                        // [CA::N][NC]
-  double* sFx = smem + CA::N * NC;         // [NV][TY][TX+1]
-  double* sFy = sFx + NV * TY * (TX + 1);  // [NV][TY+1][TX]
-  double* park = sFy + NV * (TY + 1) * TX + threadIdx.x;  // [kPark][kThreads]
-  uint64_t* tbar = reinterpret_cast<uint64_t*>(sFy + NV * (TY + 1) * TX + kPark * kThreads);
-  const RhsArgs& a = P.a;
-  const double* __restrict__ net = P.net.p;
+__device__ __forceinline__ void left_row(const Roe& r, int dir, int m, double (&L)[4]) {
+  const double nt = dir == 0 ? r.ut : r.vt;
+  const double nc = __dmul_rn(nt, r.ic);
+  const double b1u = __dmul_rn(r.b1, r.ut), hb1 = __dmul_rn(0.5, r.b1);
+  L[3] = 0.0;
+  if (NDIM == 1) {
+    if (m == 0) { L[0] = __dmul_rn(0.5, __dadd_rn(r.b2, nc)); L[1] = __dmul_rn(0.5, __dsub_rn(-b1u, r.ic)); L[2] = hb1; }
+    else if (m == 1) { L[0] = __dsub_rn(1.0, r.b2); L[1] = b1u; L[2] = -r.b1; }
+    else { L[0] = __dmul_rn(0.5, __dsub_rn(r.b2, nc)); L[1] = __dmul_rn(0.5, __dadd_rn(-b1u, r.ic)); L[2] = hb1; }
+    return;
+  }
+  const double b1v = __dmul_rn(r.b1, r.vt);
+  if (m == 1) {
+    L[0] = __dsub_rn(1.0, r.b2); L[1] = b1u; L[2] = b1v; L[3] = -r.b1;
+  } else if (m == 2) {
+    L[0] = dir == 0 ? -r.vt : -r.ut; L[1] = dir == 0 ? 0.0 : 1.0; L[2] = dir == 0 ? 1.0 : 0.0;
+  } else {
+    // the normal velocity's entry carries -+1/c, the tangential one does not
+    const double nb = dir == 0 ? -b1u : -b1v, tb = dir == 0 ? -b1v : -b1u;
+    const double ln = __dmul_rn(0.5, m == 0 ? __dsub_rn(nb, r.ic) : __dadd_rn(nb, r.ic));
+    const double lt = __dmul_rn(0.5, tb);
+    L[0] = __dmul_rn(0.5, m == 0 ? __dadd_rn(r.b2, nc) : __dsub_rn(r.b2, nc));
+    L[1] = dir == 0 ? ln : lt; L[2] = dir == 0 ? lt : ln; L[3] = hb1;
+  }
+}
+
+template <class G>
+__global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_constant__ RhsArgs a) {
+  constexpr int NDIM = G::NDIM, NV = G::NV, TX = G::TX, TY = G::TY, SX = G::SX, NC = G::NC, NT = G::NT;
+  extern __shared__ __align__(16) double smem[];
+  double* C = smem;
+  double* sF = smem + G::O_F;            // x faces [NV][TY][TX+1], then y faces [NV][TY+1][TX]
+  double* park0 = smem + G::O_P;         // [kPark][NT]
+  float* T = reinterpret_cast<float*>(smem + G::O_T);
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  double* park = park0 + t;
+  double* ws = smem + G::O_W + warp * G::kScratch;
   const int nx = a.nx, ny = a.ny;
   const size_t plane = (size_t)nx * ny;
-  const int i0 = blockIdx.x * TX, j0 = blockIdx.y * TY;
   const double gm1 = a.gm1, gamma = a.gamma;
-
-  // ---- 1. tile + halo and per-cell quantities.  An interior 2D tile's
-  // conserved variables arrive by one TMA copy of the box [NV][SY][SX]
-  // straight into the CA::U planes; edge tiles (ghost cells by periodic wrap
-  // or zero-gradient clamp) and 1D tiles are loaded cell by cell.
-  bool by_tma = false;
-  if (NDIM == 2) {
-    by_tma = tile_by_tma(a, i0, j0);
-    if (by_tma) {
-      if (threadIdx.x == 0) {
-        tc::mbar_init(tbar, 1);
-        tc::fence_mbar_init();
-        tc::mbar_arrive_expect_tx(tbar, (uint32_t)(NV * NC * sizeof(double)));
-        tc::tma_load_3d(C + CA::U * NC, &a.tmap, tbar, i0 - G::X0, j0 - G::HY, 0);
-      }
-      __syncthreads();  // the barrier is initialised before anyone waits on it
-      const bool timed_out = !tc::mbar_wait(tbar, 0);
-      if (__syncthreads_or(timed_out)) {
-        // the copy may still be in flight: wait once more (bounded) before
-        // the CTA's shared memory is released
-        tc::mbar_wait(tbar, 0);
-        if (threadIdx.x == 0) atomicOr(a.status, 4);
-        return;
-      }
-    }
-  }
-  for (int e = threadIdx.x; e < NC; e += kThreads) {
-    const int bx = e % SX, by = e / SX;
-    double U[NV];
-    if (by_tma) {
-#pragma unroll
-      for (int n = 0; n < NV; ++n) U[n] = C[(CA::U + n) * NC + e];
-    } else {
-      const int gi = wrap_index(i0 - G::X0 + bx, nx, a.bcx);
-      const int gj = NDIM == 2 ? wrap_index(j0 - G::HY + by, ny, a.bcy) : 0;
-      const size_t g = (size_t)gj * nx + gi;
-#pragma unroll
-      for (int n = 0; n < NV; ++n) {
-        U[n] = a.U[n * plane + g];
-        C[(CA::U + n) * NC + e] = U[n];
-      }
-    }
-    const double rho = U[0], E = U[NV - 1];
-    const double u = __ddiv_rn(U[1], rho);
-    double v = 0.0, q;
-    if (NDIM == 2) {
-      v = __ddiv_rn(U[2], rho);
-      q = __fma_rn(v, v, __dmul_rn(u, u));
-    } else {
-      q = __dmul_rn(u, u);
-    }
-    const double p = __dmul_rn(gm1, __dsub_rn(E, __dmul_rn(0.5, __dmul_rn(rho, q))));
-    const double c = __dsqrt_rn(__ddiv_rn(__dmul_rn(gamma, p), rho));
-    const double Ep = __dadd_rn(E, p);
-    if (!(rho > 0.0) || !(p > 0.0)) atomicOr(a.status, 1);
-    C[CA::u * NC + e] = u;
-    C[CA::v * NC + e] = v;
-    C[CA::c * NC + e] = c;
-    C[CA::H * NC + e] = __ddiv_rn(Ep, rho);
-    C[CA::s * NC + e] = __dsqrt_rn(rho);
-    if (NDIM == 2) {
-      C[(CA::Fx + 0) * NC + e] = U[1];
-      C[(CA::Fx + 1) * NC + e] = __fma_rn(U[1], u, p);
-      C[(CA::Fx + 2) * NC + e] = __dmul_rn(U[2], u);
-      C[(CA::Fx + 3) * NC + e] = __dmul_rn(Ep, u);
-      C[(CA::Fy + 0) * NC + e] = U[2];
-      C[(CA::Fy + 1) * NC + e] = __dmul_rn(U[1], v);
-      C[(CA::Fy + 2) * NC + e] = __fma_rn(U[2], v, p);
-      C[(CA::Fy + 3) * NC + e] = __dmul_rn(Ep, v);
-    } else {
-      C[(CA::Fx + 0) * NC + e] = U[1];
-      C[(CA::Fx + 1) * NC + e] = __fma_rn(U[1], u, p);
-      C[(CA::Fx + 2) * NC + e] = __dmul_rn(Ep, u);
-    }
-  }
+  const double* __restrict__ Wt = a.net64;
+  if (a.mask_mode == kMaskMLP) filt::load_filter(T, a.filter, t, NT);
 
   // dt of an RK3 step (stage 1 computes it from max(|u|+c), max(|v|+c)).
   double dt = 0.0;
@@ -188,253 +163,322 @@ __global__ void __launch_bounds__(kThreads, 1) rhs_fp64_kernel(const __grid_cons
     double s = __ddiv_rn(sx, a.dx);
     if (NDIM == 2) s = __dadd_rn(s, __ddiv_rn(__longlong_as_double((long long)a.smax[1]), a.dy));
     dt = __ddiv_rn(a.cfl, s);
-    const double t = *a.t_dev;
-    if (a.t_end > 0.0 && __dadd_rn(t, dt) > a.t_end) dt = __dsub_rn(a.t_end, t);
-    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
+    const double tm = *a.t_dev;
+    if (a.t_end > 0.0 && __dadd_rn(tm, dt) > a.t_end) dt = __dsub_rn(a.t_end, tm);
+    if (blockIdx.x == 0 && t == 0) {
       *a.dt_dev = dt;
       if (a.dt_user) *a.dt_user = dt;
     }
   } else if (a.stage >= 2) {
     dt = *a.dt_dev;
-    if (a.stage == 3 && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
-      *a.t_dev = __dadd_rn(*a.t_dev, dt);
+    if (a.stage == 3 && blockIdx.x == 0 && t == 0) *a.t_dev = __dadd_rn(*a.t_dev, dt);
   }
-  __syncthreads();
 
-  // ---- 2. faces: one item per (face, field), four lanes per face
-  constexpr int NITEMS = 4 * (G::NXF + G::NYF);
-  static_assert((4 * G::NXF) % 32 == 0, "x/y items must not share a warp");
-  const int lane = threadIdx.x & 31;
-#pragma unroll 1
-  for (int base = 0; base < NITEMS; base += kThreads) {
-    const int w = base + threadIdx.x;
-    if (base + (threadIdx.x & ~31) >= NITEMS) break;  // whole warp past the end
-    const int face = w >> 2;
-    const int m = min(w & 3, NV - 1);
-    const int dir = face < G::NXF ? 0 : 1;  // warp-uniform
-    int cb0, stride, gf, gline;
-    if (dir == 0) {
-      const int r = face / (TX + 1), f = face % (TX + 1);
-      cb0 = (G::HY + r) * SX + (G::X0 - 3) + f;
-      stride = 1;
-      gf = i0 + f;      // global face index along x, 0..nx
-      gline = j0 + r;   // row
-    } else {
-      const int fl = face - G::NXF;
-      const int f = fl / TX, c = fl % TX;
-      cb0 = f * SX + G::X0 + c;
-      stride = SX;
-      gf = j0 + f;
-      gline = i0 + c;   // column
-    }
-    const bool valid = (w & 3) < NV &&
-                       (dir == 0 ? (gf <= nx && gline < ny) : (gf <= ny && gline < nx));
-    const double* Fl = C + (dir == 0 ? CA::Fx : CA::Fy) * NC;
-    const double* Un = C + (dir == 0 ? CA::u : CA::v) * NC;  // normal velocity
-    const int ca = cb0 + 2 * stride, cbb = cb0 + 3 * stride;
-
-    // Roe average of cells i and i+1 (Sec. 4.4).
-    const double sa = C[CA::s * NC + ca], sb = C[CA::s * NC + cbb];
-    const double den = __dadd_rn(sa, sb);
-    const double ut = __ddiv_rn(__fma_rn(sb, C[CA::u * NC + cbb], __dmul_rn(sa, C[CA::u * NC + ca])), den);
-    const double Ht = __ddiv_rn(__fma_rn(sb, C[CA::H * NC + cbb], __dmul_rn(sa, C[CA::H * NC + ca])), den);
-    double vt = 0.0, qt;
-    if (NDIM == 2) {
-      vt = __ddiv_rn(__fma_rn(sb, C[CA::v * NC + cbb], __dmul_rn(sa, C[CA::v * NC + ca])), den);
-      qt = __fma_rn(vt, vt, __dmul_rn(ut, ut));
-    } else {
-      qt = __dmul_rn(ut, ut);
-    }
-    const double c2 = __dmul_rn(gm1, __dsub_rn(Ht, __dmul_rn(0.5, qt)));
-    if (valid && !(c2 > 0.0)) atomicOr(a.status, 2);
-    const double ct = __dsqrt_rn(c2);
-    const double ic = __ddiv_rn(1.0, ct);
-    const double b1 = __ddiv_rn(gm1, c2);
-    const double b2 = __dmul_rn(0.5, __dmul_rn(b1, qt));
-    const double nt = dir == 0 ? ut : vt;
-    const double nc = __dmul_rn(nt, ic);
-    const double b1u = __dmul_rn(b1, ut), b1v = __dmul_rn(b1, vt);
-    const double hb1 = __dmul_rn(0.5, b1), ntc = __dmul_rn(nt, ct);
-
-    // Left eigenvector (row m of L) and right-eigenvector components (row m
-    // of R, i.e. component m of every column) in the Roe/Toro scaling.
-    double L[4], R[4];
-    {
-      const double am = __dmul_rn(0.5, __dadd_rn(b2, nc));   // acoustic "-" first entry
-      const double ap = __dmul_rn(0.5, __dsub_rn(b2, nc));   // acoustic "+" first entry
-      const double nb1u = -b1u, nb1v = -b1v;
-      const double hm_u = __dmul_rn(0.5, __dsub_rn(nb1u, ic)), hp_u = __dmul_rn(0.5, __dadd_rn(nb1u, ic));
-      if (NDIM == 1) {
-        if (m == 0) { L[0] = am; L[1] = hm_u; L[2] = hb1; }
-        else if (m == 1) { L[0] = __dsub_rn(1.0, b2); L[1] = b1u; L[2] = -b1; }
-        else { L[0] = ap; L[1] = hp_u; L[2] = hb1; }
-        L[3] = 0.0;
-        if (m == 0) { R[0] = 1.0; R[1] = 1.0; R[2] = 1.0; }
-        else if (m == 1) { R[0] = __dsub_rn(ut, ct); R[1] = ut; R[2] = __dadd_rn(ut, ct); }
-        else { R[0] = __dsub_rn(Ht, ntc); R[1] = __dmul_rn(0.5, qt); R[2] = __dadd_rn(Ht, ntc); }
-        R[3] = 0.0;
+  const long long ntx = (nx + TX - 1) / TX, ntiles = ntx * ((ny + TY - 1) / TY);
+  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int i0 = (int)(tile % ntx) * TX, j0 = (int)(tile / ntx) * TY;
+    // ---- 1. tile + halo (without its corners) and per-cell quantities.
+    // `odd`: some value is not 0 or in [2^-60, 2^60), or a cell is not
+    // physical; the tile's faces then take every operation of the
+    // specification literally (below).
+    bool odd = false;
+    for (int e = t; e < NC; e += NT) {
+      const int bx = e % SX, by = e / SX;
+      if (NDIM == 2 && (bx < 3 || bx >= TX + 3) && (by < 3 || by >= TY + 3)) continue;
+      const int gi = wrap_index(i0 - 3 + bx, nx, a.bcx);
+      const int gj = NDIM == 2 ? wrap_index(j0 - 3 + by, ny, a.bcy) : 0;
+      const size_t g = (size_t)gj * nx + gi;
+      double U[NV];
+#pragma unroll
+      for (int n = 0; n < NV; ++n) {
+        U[n] = a.U[n * plane + g];
+        C[(G::P_U + n) * NC + e] = U[n];
+        odd |= !moderate(U[n]);
+      }
+      const double rho = U[0], E = U[NV - 1];
+      const double u = __ddiv_rn(U[1], rho);
+      double v = 0.0, q;
+      if (NDIM == 2) {
+        v = __ddiv_rn(U[2], rho);
+        q = __fma_rn(v, v, __dmul_rn(u, u));
       } else {
-        const double hnb1v = __dmul_rn(0.5, nb1v), hnb1u = __dmul_rn(0.5, nb1u);
-        const double hm_v = __dmul_rn(0.5, __dsub_rn(nb1v, ic)), hp_v = __dmul_rn(0.5, __dadd_rn(nb1v, ic));
-        if (m == 0) {
-          L[0] = am; L[1] = dir == 0 ? hm_u : hnb1u; L[2] = dir == 0 ? hnb1v : hm_v; L[3] = hb1;
-        } else if (m == 1) {
-          L[0] = __dsub_rn(1.0, b2); L[1] = b1u; L[2] = b1v; L[3] = -b1;
-        } else if (m == 2) {
-          L[0] = dir == 0 ? -vt : -ut; L[1] = dir == 0 ? 0.0 : 1.0; L[2] = dir == 0 ? 1.0 : 0.0; L[3] = 0.0;
-        } else {
-          L[0] = ap; L[1] = dir == 0 ? hp_u : hnb1u; L[2] = dir == 0 ? hnb1v : hp_v; L[3] = hb1;
+        q = __dmul_rn(u, u);
+      }
+      const double p = __dmul_rn(gm1, __dsub_rn(E, __dmul_rn(0.5, __dmul_rn(rho, q))));
+      const double c = __dsqrt_rn(__ddiv_rn(__dmul_rn(gamma, p), rho));
+      const double Ep = __dadd_rn(E, p);
+      if (!(rho > 0.0) || !(p > 0.0)) {
+        atomicOr(a.status, 1);
+        odd = true;
+      }
+      odd |= !moderate(p);
+      C[G::P_u * NC + e] = u;
+      C[G::P_c * NC + e] = c;
+      C[G::P_H * NC + e] = __ddiv_rn(Ep, rho);
+      C[G::P_s * NC + e] = __dsqrt_rn(rho);
+      double* F = C + G::P_F * NC + e;
+      if (NDIM == 2) {
+        C[G::P_v * NC + e] = v;
+        if (by >= 3 && by < TY + 3) {
+          F[0] = __fma_rn(U[1], u, p);
+          F[NC] = __dmul_rn(U[2], u);
+          F[2 * NC] = __dmul_rn(Ep, u);
         }
-        if (m == 0) { R[0] = 1.0; R[1] = 1.0; R[2] = 0.0; R[3] = 1.0; }
-        else if (m == 1) {
-          if (dir == 0) { R[0] = __dsub_rn(ut, ct); R[1] = ut; R[2] = 0.0; R[3] = __dadd_rn(ut, ct); }
-          else { R[0] = ut; R[1] = ut; R[2] = 1.0; R[3] = ut; }
-        } else if (m == 2) {
-          if (dir == 0) { R[0] = vt; R[1] = vt; R[2] = 1.0; R[3] = vt; }
-          else { R[0] = __dsub_rn(vt, ct); R[1] = vt; R[2] = 0.0; R[3] = __dadd_rn(vt, ct); }
-        } else {
-          R[0] = __dsub_rn(Ht, ntc); R[1] = __dmul_rn(0.5, qt); R[2] = dir == 0 ? vt : ut;
-          R[3] = __dadd_rn(Ht, ntc);
+        if (bx >= 3 && bx < TX + 3) {
+          F[3 * NC] = __dmul_rn(U[1], v);
+          F[4 * NC] = __fma_rn(U[2], v, p);
+          F[5 * NC] = __dmul_rn(Ep, v);
         }
+      } else {
+        F[0] = __fma_rn(U[1], u, p);
+        F[NC] = __dmul_rn(Ep, u);
       }
     }
+    odd |= !moderate(gm1);
+    odd = __syncthreads_or(odd);
 
-    // LLF alpha_m: max over the six stencil cells of |lambda_m|.
-    double alpha = 0.0;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      const int cj = cb0 + j * stride;
-      const double un = Un[cj], cs = C[CA::c * NC + cj];
-      const double lam = m == 0 ? __dsub_rn(un, cs) : (m == NV - 1 ? __dadd_rn(un, cs) : un);
-      alpha = j == 0 ? dabs(lam) : dmax_nn(alpha, dabs(lam));
-    }
-
-    // Characteristic projection and LLF split of the six stencil cells.
-    double sp[6], sm[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      const int cj = cb0 + j * stride;
-      double vv = __dmul_rn(L[0], C[(CA::U + 0) * NC + cj]);
-      double gg = __dmul_rn(L[0], Fl[0 * NC + cj]);
-#pragma unroll
-      for (int n = 1; n < NV; ++n) {
-        vv = __fma_rn(L[n], C[(CA::U + n) * NC + cj], vv);
-        gg = __fma_rn(L[n], Fl[n * NC + cj], gg);
-      }
-      sp[j] = __dmul_rn(0.5, __fma_rn(alpha, vv, gg));
-      sm[j] = __dmul_rn(0.5, __fma_rn(-alpha, vv, gg));
-    }
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      park[j * kThreads] = sp[j];
-      park[(6 + j) * kThreads] = sm[5 - j];  // the "-" side is the mirror image
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) park[(12 + q) * kThreads] = R[q];
-
-    // Classifier bits of both sides ("-" side = mirror image).
-    // Compiler-level barrier: the parked values must be re-read from shared
-    // memory, not kept live in registers across the classifier.
-    asm volatile("" ::: "memory");
-    unsigned eta_side[2];
-    if (a.mask_mode == kMaskMLP) {
+    // ---- 2. faces
+    constexpr int kItems = (G::WX + G::WY) * (G::SPLIT ? NV : 1);
 #pragma unroll 1
-      for (int side = 0; side < 2; ++side) {
-        double st[6], x[6], z[4];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) st[j] = park[(side * 6 + j) * kThreads];
-        normalise6(st, x);
-        eta_side[side] = mlp64(net, x, z);
-      }
-    } else if (a.mask_mode == kMaskTeno) {
-      // TENO6-opt selection on the split fluxes themselves (its indicator
-      // ratios do not depend on the scale)
-#pragma unroll 1
-      for (int side = 0; side < 2; ++side) {
-        double st[6];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) st[j] = park[(side * 6 + j) * kThreads];
-        eta_side[side] = teno6_eta(a.teno, st);
-      }
-    } else if (a.mask_mode == kMaskGiven) {
-      size_t idx;
-      if (dir == 0) idx = ((size_t)m * ny + gline) * (nx + 1) + gf;
-      else idx = (size_t)NV * ny * (nx + 1) + ((size_t)m * (ny + 1) + gf) * nx + gline;
-      const unsigned b = valid ? a.mask_in[idx] : 0u;
-      eta_side[0] = b & 15u;
-      eta_side[1] = b >> 4;
-    } else {
-      eta_side[0] = eta_side[1] = a.mask_mode == kMaskRough ? 15u : 0u;
-    }
-    asm volatile("" ::: "memory");
-    double spl[6], smir[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      spl[j] = park[j * kThreads];
-      smir[j] = park[(6 + j) * kThreads];
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) R[q] = park[(12 + q) * kThreads];
-    const double gp = combine64(a, spl, eta_side[0]);
-    const double gmn = combine64(a, smir, eta_side[1]);
-    const double gh = __dadd_rn(gp, gmn);
-
-    // Back-projection F_n = sum_m R[n][m] gh_m; lane m of the face holds gh_m
-    // and computes component n = m.
-    const int fbase = lane & ~3;
-    double ghm[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) ghm[q] = __shfl_sync(0xffffffffu, gh, fbase + q);
-    double Fh = __dmul_rn(R[0], ghm[0]);
-#pragma unroll
-    for (int q = 1; q < NV; ++q) Fh = __fma_rn(R[q], ghm[q], Fh);
-
-    if (valid) {
+    for (int it = warp; it < kItems; it += NT / 32) {
+      const int run = G::SPLIT ? it / NV : it;
+      const int dir = NDIM == 2 && run >= G::WX ? 1 : 0;  // warp-uniform
+      const int nf = dir == 0 ? G::NXF : G::NYF;
+      const int fraw = (run - (dir ? G::WX : 0)) * 32 + lane;
+      const int face = min(fraw, nf - 1);
+      int cb0, gf, gline;
+      const int stride = dir == 0 ? 1 : SX;
       if (dir == 0) {
         const int r = face / (TX + 1), f = face % (TX + 1);
-        sFx[(m * TY + r) * (TX + 1) + f] = Fh;
+        cb0 = (G::HY + r) * SX + f;
+        gf = i0 + f;      // global face index along x, 0..nx
+        gline = j0 + r;   // row
       } else {
-        const int fl = face - G::NXF;
-        sFy[(m * (TY + 1) + fl / TX) * TX + fl % TX] = Fh;
+        const int f = face / TX, c = face % TX;
+        cb0 = f * SX + 3 + c;
+        gf = j0 + f;
+        gline = i0 + c;   // column
       }
-      if (a.mask_out) {
-        size_t idx;
-        if (dir == 0) idx = ((size_t)m * ny + gline) * (nx + 1) + gf;
-        else idx = (size_t)NV * ny * (nx + 1) + ((size_t)m * (ny + 1) + gf) * nx + gline;
-        a.mask_out[idx] = (uint8_t)(eta_side[0] | (eta_side[1] << 4));
-      }
-    }
-  }
-  __syncthreads();
+      const bool valid = fraw < nf && (dir == 0 ? (gf <= nx && gline < ny) : (gf <= ny && gline < nx));
+      if (__ballot_sync(0xffffffffu, valid) == 0u) continue;
+      const double* Un = C + (dir == 0 ? G::P_u : G::P_v) * NC;  // normal velocity
+      const double* F0 = C + (G::P_U + 1 + dir) * NC;            // mass flux
+      const double* F1 = C + (G::P_F + dir * 3) * NC;            // the other fluxes
+      const int ca = cb0 + 2 * stride, cb = cb0 + 3 * stride;
 
-  // ---- 3. conservative difference and (optionally) the RK3 stage update
-  for (int e = threadIdx.x; e < TX * TY; e += kThreads) {
-    const int c = e % TX, r = e / TX;
-    const int gi = i0 + c, gj = j0 + r;
-    if (gi >= nx || gj >= ny) continue;
-    const size_t g = (size_t)gj * nx + gi;
-    const int bc = (G::HY + r) * SX + G::X0 + c;
+      // Roe average of cells i and i+1 (Sec. 4.4).
+      Roe r;
+      {
+        const double sa = C[G::P_s * NC + ca], sb = C[G::P_s * NC + cb];
+        const double den = __dadd_rn(sa, sb);
+        r.ut = __ddiv_rn(__fma_rn(sb, C[G::P_u * NC + cb], __dmul_rn(sa, C[G::P_u * NC + ca])), den);
+        r.Ht = __ddiv_rn(__fma_rn(sb, C[G::P_H * NC + cb], __dmul_rn(sa, C[G::P_H * NC + ca])), den);
+        r.vt = 0.0;
+        if (NDIM == 2) {
+          r.vt = __ddiv_rn(__fma_rn(sb, C[G::P_v * NC + cb], __dmul_rn(sa, C[G::P_v * NC + ca])), den);
+          r.qt = __fma_rn(r.vt, r.vt, __dmul_rn(r.ut, r.ut));
+        } else {
+          r.qt = __dmul_rn(r.ut, r.ut);
+        }
+        const double c2 = __dmul_rn(gm1, __dsub_rn(r.Ht, __dmul_rn(0.5, r.qt)));
+        if (valid && !(c2 > 0.0)) atomicOr(a.status, 2);
+        r.ct = __dsqrt_rn(c2);
+        r.ic = __ddiv_rn(1.0, r.ct);
+        r.b1 = __ddiv_rn(gm1, c2);
+        r.b2 = __dmul_rn(0.5, __dmul_rn(r.b1, r.qt));
+      }
+
+      double gh[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
+      for (int m = G::SPLIT ? it % NV : 0; m < (G::SPLIT ? it % NV + 1 : NV); ++m) {
+        // LLF alpha_m: max over the six stencil cells of |lambda_m|.
+        double alpha = 0.0;
 #pragma unroll
-    for (int n = 0; n < NV; ++n) {
-      const double Fp = sFx[(n * TY + r) * (TX + 1) + c + 1];
-      const double Fm = sFx[(n * TY + r) * (TX + 1) + c];
-      double rr = -__ddiv_rn(__dsub_rn(Fp, Fm), a.dx);
-      if (NDIM == 2) {
-        const double Gp = sFy[(n * (TY + 1) + r + 1) * TX + c];
-        const double Gm = sFy[(n * (TY + 1) + r) * TX + c];
-        rr = __dsub_rn(rr, __ddiv_rn(__dsub_rn(Gp, Gm), a.dy));
+        for (int j = 0; j < 6; ++j) {
+          double lam = Un[cb0 + j * stride];
+          if (m == 0) lam = __dsub_rn(lam, C[G::P_c * NC + cb0 + j * stride]);
+          else if (m == NV - 1) lam = __dadd_rn(lam, C[G::P_c * NC + cb0 + j * stride]);
+          alpha = j == 0 ? dabs(lam) : dmax_nn(alpha, dabs(lam));
+        }
+        // Characteristic projection and LLF split of the six stencil cells,
+        // (L F +- alpha L U) / 2 with the "-" side mirrored.  On a moderate
+        // tile every intermediate is 0 or far above the subnormal range, so
+        // halving the row of L halves every following value exactly and saves
+        // the twelve products by 1/2; and the shear row's entries 0 and 1 need
+        // no products.
+        double L[4], sp[6], sm[6];
+        left_row<NDIM>(r, dir, m, L);
+        if (!odd) {
+          if (NDIM == 2 && m == 2) {
+            const double l0 = half_exact(L[0]);
+            const double* Ut = C + (G::P_U + 2 - dir) * NC;  // tangential momentum
+            const double* Ft = F1 + (1 - dir) * NC;          // and its flux
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+              const int cj = cb0 + j * stride;
+              const double vv = __fma_rn(0.5, Ut[cj], __dmul_rn(l0, C[G::P_U * NC + cj]));
+              const double gg = __fma_rn(0.5, Ft[cj], __dmul_rn(l0, F0[cj]));
+              sp[j] = __fma_rn(alpha, vv, gg);
+              sm[j] = __fma_rn(-alpha, vv, gg);
+            }
+          } else {
+#pragma unroll
+            for (int n = 0; n < NV; ++n) L[n] = half_exact(L[n]);
+#pragma unroll
+            for (int j = 0; j < 6; ++j) {
+              const int cj = cb0 + j * stride;
+              double vv = __dmul_rn(L[0], C[G::P_U * NC + cj]);
+              double gg = __dmul_rn(L[0], F0[cj]);
+#pragma unroll
+              for (int n = 1; n < NV; ++n) {
+                vv = __fma_rn(L[n], C[(G::P_U + n) * NC + cj], vv);
+                gg = __fma_rn(L[n], F1[(n - 1) * NC + cj], gg);
+              }
+              sp[j] = __fma_rn(alpha, vv, gg);
+              sm[j] = __fma_rn(-alpha, vv, gg);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 6; ++j) {
+            const int cj = cb0 + j * stride;
+            double vv = __dmul_rn(L[0], C[G::P_U * NC + cj]);
+            double gg = __dmul_rn(L[0], F0[cj]);
+#pragma unroll
+            for (int n = 1; n < NV; ++n) {
+              vv = __fma_rn(L[n], C[(G::P_U + n) * NC + cj], vv);
+              gg = __fma_rn(L[n], F1[(n - 1) * NC + cj], gg);
+            }
+            sp[j] = __dmul_rn(0.5, __fma_rn(alpha, vv, gg));
+            sm[j] = __dmul_rn(0.5, __fma_rn(-alpha, vv, gg));
+          }
+        }
+        double smir[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+          smir[j] = sm[5 - j];  // the "-" side is the mirror image
+          park[j * NT] = sp[j];
+          park[(6 + j) * NT] = smir[j];
+        }
+
+        // Classifier bits of both sides.
+        unsigned eta_side[2];
+        if (a.mask_mode == kMaskMLP) {
+          float x[2][6];
+          const bool ok0 = filt::filter_input(sp, x[0]);
+          const bool ok1 = filt::filter_input(smir, x[1]);
+          // the stencils are re-read from shared memory after the classifier
+          // rather than kept in registers across it
+          asm volatile("" ::: "memory");
+          unsigned res[2];
+          filt::filter_rows<2>(T, x, res);
+          eta_side[0] = res[0] & 15u;
+          eta_side[1] = res[1] & 15u;
+          filt::settle_rows(Wt, park0 + warp * 32, NT, ws, valid && !(ok0 && (res[0] & 16u)), eta_side[0]);
+          filt::settle_rows(Wt, park0 + 6 * NT + warp * 32, NT, ws, valid && !(ok1 && (res[1] & 16u)),
+                            eta_side[1]);
+          asm volatile("" ::: "memory");
+        } else if (a.mask_mode == kMaskTeno) {
+          // TENO6-opt selection on the split fluxes themselves (its indicator
+          // ratios do not depend on the scale)
+          eta_side[0] = teno6_eta(a.teno, sp);
+          eta_side[1] = teno6_eta(a.teno, smir);
+        } else if (a.mask_mode == kMaskGiven) {
+          size_t idx;
+          if (dir == 0) idx = ((size_t)m * ny + gline) * (nx + 1) + gf;
+          else idx = (size_t)NV * ny * (nx + 1) + ((size_t)m * (ny + 1) + gf) * nx + gline;
+          const unsigned b = valid ? a.mask_in[idx] : 0u;
+          eta_side[0] = b & 15u;
+          eta_side[1] = b >> 4;
+        } else {
+          eta_side[0] = eta_side[1] = a.mask_mode == kMaskRough ? 15u : 0u;
+        }
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+          sp[j] = park[j * NT];
+          smir[j] = park[(6 + j) * NT];
+        }
+        const double g = __dadd_rn(combine64(a, sp, eta_side[0]), combine64(a, smir, eta_side[1]));
+#pragma unroll
+        for (int q = 0; q < NV; ++q)
+          if (q == m) gh[q] = g;
+        if (valid && a.mask_out) {
+          size_t idx;
+          if (dir == 0) idx = ((size_t)m * ny + gline) * (nx + 1) + gf;
+          else idx = (size_t)NV * ny * (nx + 1) + ((size_t)m * (ny + 1) + gf) * nx + gline;
+          a.mask_out[idx] = (uint8_t)(eta_side[0] | (eta_side[1] << 4));
+        }
+        if (G::SPLIT) {
+          const int fi = (dir == 0 ? 0 : G::NXF) + face;
+          double* sG = smem + G::O_G;
+          if (fraw < nf) {
+            sG[m * (G::NXF + G::NYF) + fi] = g;
+            if (m == 0) {
+              double* sR = sG + NV * (G::NXF + G::NYF) + fi;
+              const double rv[5] = {r.ut, r.vt, r.Ht, r.ct, r.qt};
+#pragma unroll
+              for (int q = 0; q < 5; ++q) sR[q * (G::NXF + G::NYF)] = rv[q];
+            }
+          }
+        }
       }
-      double val = rr;
-      const double Ucur = C[(CA::U + n) * NC + bc];
-      if (a.stage == 1) {
-        val = __fma_rn(dt, rr, Ucur);
-      } else if (a.stage == 2) {
-        val = __fma_rn(0.75, a.U0[n * plane + g], __dmul_rn(0.25, __fma_rn(dt, rr, Ucur)));
-      } else if (a.stage == 3) {
-        val = __fma_rn(a.third, a.U0[n * plane + g], __dmul_rn(a.two_thirds, __fma_rn(dt, rr, Ucur)));
+      // Back-projection F_n = sum_m R[n][m] gh_m.
+      if (!G::SPLIT && fraw < nf) {
+        double* dst = sF + (dir == 0 ? 0 : NV * G::NXF) + face;
+#pragma unroll
+        for (int n = 0; n < NV; ++n) dst[n * nf] = back_project<NDIM>(r, dir, n, gh);
       }
-      a.out[n * plane + g] = val;
     }
+    __syncthreads();
+    if (G::SPLIT) {
+      const double* sG = smem + G::O_G;
+      for (int e = t; e < NV * (G::NXF + G::NYF); e += NT) {
+        const int n = e / (G::NXF + G::NYF), fi = e % (G::NXF + G::NYF);
+        const int dir = fi < G::NXF ? 0 : 1;
+        double gq[4] = {0.0, 0.0, 0.0, 0.0}, rv[5];
+#pragma unroll
+        for (int q = 0; q < NV; ++q) gq[q] = sG[q * (G::NXF + G::NYF) + fi];
+#pragma unroll
+        for (int q = 0; q < 5; ++q) rv[q] = sG[(NV + q) * (G::NXF + G::NYF) + fi];
+        Roe r;
+        r.ut = rv[0]; r.vt = rv[1]; r.Ht = rv[2]; r.ct = rv[3]; r.qt = rv[4];
+        const double F = back_project<NDIM>(r, dir, n, gq);
+        if (dir == 0) sF[n * G::NXF + fi] = F;
+        else sF[NV * G::NXF + n * G::NYF + fi - G::NXF] = F;
+      }
+      __syncthreads();
+    }
+
+    // ---- 3. conservative difference and (optionally) the RK3 stage update.
+    // A division by a power of two is the exact product with its reciprocal.
+    const double* sFy = sF + NV * G::NXF;
+    for (int e = t; e < TX * TY; e += NT) {
+      const int c = e % TX, rw = e / TX;
+      const int gi = i0 + c, gj = j0 + rw;
+      if (gi >= nx || gj >= ny) continue;
+      const size_t g = (size_t)gj * nx + gi;
+      const int bc = (G::HY + rw) * SX + 3 + c;
+#pragma unroll
+      for (int n = 0; n < NV; ++n) {
+        const double dF = __dsub_rn(sF[(n * TY + rw) * (TX + 1) + c + 1], sF[(n * TY + rw) * (TX + 1) + c]);
+        double rr = -(a.inv_dx != 0.0 ? __dmul_rn(dF, a.inv_dx) : __ddiv_rn(dF, a.dx));
+        if (NDIM == 2) {
+          const double dG = __dsub_rn(sFy[(n * (TY + 1) + rw + 1) * TX + c], sFy[(n * (TY + 1) + rw) * TX + c]);
+          rr = __dsub_rn(rr, a.inv_dy != 0.0 ? __dmul_rn(dG, a.inv_dy) : __ddiv_rn(dG, a.dy));
+        }
+        double val = rr;
+        const double Ucur = C[(G::P_U + n) * NC + bc];
+        if (a.stage == 1) {
+          val = __fma_rn(dt, rr, Ucur);
+        } else if (a.stage == 2) {
+          val = __fma_rn(0.75, a.U0[n * plane + g], __dmul_rn(0.25, __fma_rn(dt, rr, Ucur)));
+        } else if (a.stage == 3) {
+          val = __fma_rn(a.third, a.U0[n * plane + g], __dmul_rn(a.two_thirds, __fma_rn(dt, rr, Ucur)));
+        }
+        a.out[n * plane + g] = val;
+      }
+    }
+    __syncthreads();  // the next tile's cells overwrite what the difference reads
   }
 }
 
@@ -467,6 +511,41 @@ __global__ void __launch_bounds__(256) classify_fp64_narrow_kernel(const __grid_
 #pragma unroll
     for (int k = 0; k < 4; ++k) P.logits[r * 4 + k] = z[k];
   }
+}
+
+// The classifier parameters as the FP64 kernels read them: the binary64
+// weights transposed, then the FP32 table of the certified filter.
+__global__ void net_blob_kernel(const __grid_constant__ NetF64 net, const __grid_constant__ FilterKappa k,
+                                double* __restrict__ Wt, float* __restrict__ T) {
+  constexpr int W[6] = {6, 64, 32, 16, 8, 4};
+  const int kW[5] = {kFiltW1, kFiltW2, kFiltW3, kFiltW4, kFiltW5};
+  const int kB[5] = {0, kFiltB2, kFiltB3, kFiltB4, kFiltB5};
+  for (int i = threadIdx.x; i < kFiltFloats; i += blockDim.x) T[i] = 0.0f;
+  __syncthreads();
+  int p = 0;
+  for (int l = 0; l < 5; ++l) {
+    const int nin = W[l], nout = W[l + 1];
+    for (int e = threadIdx.x; e < nin * nout; e += blockDim.x) {
+      const int o = e / nin, i = e % nin;
+      const double w = net.p[p + e];
+      Wt[p + i * nout + o] = w;
+      if (l == 0) T[kFiltW1 + 8 * o + i] = (float)w;
+      else T[kW[l] + i * nout + o] = (float)(l == 4 ? w * k.scale[o] : w);
+    }
+    p += nin * nout;
+    for (int o = threadIdx.x; o < nout; o += blockDim.x) {
+      const double b = net.p[p + o];
+      Wt[p + o] = b;
+      if (l == 0) T[kFiltW1 + 8 * o + 6] = (float)b;
+      else T[kB[l] + o] = (float)(l == 4 ? b * k.scale[o] : b);
+    }
+    p += nout;
+  }
+  for (int i = threadIdx.x; i < 7; i += blockDim.x) T[kFiltIn + i] = i == 0 ? k.k0 : k.in[i - 1];
+  for (int i = threadIdx.x; i < 64; i += blockDim.x) T[kFiltW1 + 8 * i + 7] = k.h1[i];
+  for (int i = threadIdx.x; i < 32; i += blockDim.x) T[kFiltK2 + i] = k.h2[i];
+  for (int i = threadIdx.x; i < 16; i += blockDim.x) T[kFiltK3 + i] = k.h3[i];
+  for (int i = threadIdx.x; i < 8; i += blockDim.x) T[kFiltK4 + i] = k.h4[i];
 }
 
 __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
@@ -524,62 +603,106 @@ __global__ void __launch_bounds__(256) cfl_reduce_kernel(const double* __restric
 
 }  // namespace
 
-namespace {
-
-// cuTensorMapEncodeTiled, reached through the runtime's driver entry-point
-// query (the library links no driver library); null if unavailable.
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn encode_tiled() {
-  static EncodeTiledFn fn = [] {
-    void* f = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) !=
-            cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      return (EncodeTiledFn) nullptr;
-    return reinterpret_cast<EncodeTiledFn>(f);
-  }();
-  return fn;
+// Coefficients of the filter's bound (mlp_filter.cuh).
+static void build_filter_kappa(const NetF64& net, FilterKappa& out) {
+  constexpr int W[6] = {6, 64, 32, 16, 8, 4};
+  constexpr int off[5] = {0, 448, 2528, 3056, 3192};
+  const double u = 1.0 / 16777216.0, tiny = std::ldexp(1.0, -125);
+  auto aw = [&](int l, int o, int i) { return std::fmax(std::fabs(net.p[off[l] + o * W[l] + i]), tiny); };
+  auto ab = [&](int l, int o) { return std::fmax(std::fabs(net.p[off[l] + W[l] * W[l + 1] + o]), tiny); };
+  // static bound per logit over |x| <= 1: the logits' relative scales
+  double M[64], e[64], Mn[64], en[64];
+  for (int i = 0; i < 6; ++i) {
+    M[i] = 1.0;
+    e[i] = 8.0 * u;
+  }
+  for (int l = 0; l < 5; ++l) {
+    for (int o = 0; o < W[l + 1]; ++o) {
+      double s = ab(l, o), d = 0.0;
+      for (int i = 0; i < W[l]; ++i) {
+        s += aw(l, o, i) * M[i];
+        d += aw(l, o, i) * e[i];
+      }
+      Mn[o] = s;
+      en[o] = d + (W[l] + 2) * u * s;
+    }
+    for (int o = 0; o < W[l + 1]; ++o) {
+      M[o] = Mn[o];
+      e[o] = en[o];
+    }
+  }
+  double G[4][64], Gn[4][64];
+  for (int k = 0; k < 4; ++k) {
+    const double s = e[0] / e[k];
+    out.scale[k] = s > 1e-30 && s < 1e30 ? s : 1.0;
+    for (int o = 0; o < 4; ++o) G[k][o] = k == o ? out.scale[k] : 0.0;
+  }
+  auto up = [](double x) { return std::nextafter((float)(1.01 * x), INFINITY); };
+  double k0[4] = {0.0, 0.0, 0.0, 0.0};
+  float* dst[5] = {out.in, out.h1, out.h2, out.h3, out.h4};
+  for (int l = 4; l >= 0; --l) {
+    const int n = W[l], m = W[l + 1];
+    for (int i = 0; i < n; ++i) {
+      double worst = 0.0;
+      for (int k = 0; k < 4; ++k) {
+        double g = 0.0;
+        for (int o = 0; o < m; ++o) g += G[k][o] * aw(l, o, i);
+        Gn[k][i] = g;
+        // the i-th FMA of the chain and those after it, and the weight's rounding
+        double c = (n - i + 1) * u * g;
+        if (l == 0) {
+          c += 8.0 * u * g;
+          k0[k] += g * tiny;
+        }
+        worst = std::fmax(worst, c);
+        if (!(c == c)) worst = c;  // a NaN weight: nothing is certified
+      }
+      dst[l][i] = up(worst);
+    }
+    for (int k = 0; k < 4; ++k)
+      for (int o = 0; o < m; ++o) k0[k] += (n + 1) * u * G[k][o] * ab(l, o);
+    for (int k = 0; k < 4; ++k)
+      for (int i = 0; i < n; ++i) G[k][i] = Gn[k][i];
+  }
+  double worst = 0.0;
+  for (int k = 0; k < 4; ++k) worst = k0[k] == k0[k] ? std::fmax(worst, k0[k]) : k0[k];
+  out.k0 = up(worst);
 }
 
-// Tensor map of the 2D state U ([4][ny][nx] float64) with the box of one
-// staged FP64 tile ([4][SY][SX]).  False when U cannot be described: the
-// row stride nx * 8 and the base must be multiples of 16 bytes.
-bool encode_tile_map(RhsArgs& a) {
-  using G = Geom<2>;
-  EncodeTiledFn enc = encode_tiled();
-  if (!enc || a.nx % 2 != 0 || (reinterpret_cast<uintptr_t>(a.U) & 15u) != 0) return false;
-  const cuuint64_t dims[3] = {(cuuint64_t)a.nx, (cuuint64_t)a.ny, (cuuint64_t)G::NV};
-  const cuuint64_t strides[2] = {(cuuint64_t)a.nx * 8, (cuuint64_t)a.nx * a.ny * 8};
-  const cuuint32_t box[3] = {(cuuint32_t)G::SX, (cuuint32_t)G::SY, (cuuint32_t)G::NV};
-  const cuuint32_t unit[3] = {1, 1, 1};
-  return enc(&a.tmap, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 3, const_cast<double*>(a.U), dims, strides, box, unit,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+cudaError_t launch_net_blob(const NetF64& net, void* blob, cudaStream_t s) {
+  FilterKappa k;
+  build_filter_kappa(net, k);
+  double* Wt = static_cast<double*>(blob);
+  net_blob_kernel<<<1, 256, 0, s>>>(net, k, Wt, reinterpret_cast<float*>(Wt + kNetParams));
+  return cudaGetLastError();
+}
+
+namespace {
+
+template <class G>
+cudaError_t launch_tiles(const RhsArgs& a, cudaStream_t s) {
+  cudaError_t e =
+      cudaFuncSetAttribute(rhs_fp64_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
+  if (e != cudaSuccess) return e;
+  const long long tiles = (long long)((a.nx + G::TX - 1) / G::TX) * ((a.ny + G::TY - 1) / G::TY);
+  const long long most = 152ll * G::OCC;
+  rhs_fp64_kernel<G><<<(unsigned)(tiles < most ? tiles : most), G::NT, G::SMEM, s>>>(a);
+  return cudaGetLastError();
+}
+
+// 1/d when d is a power of two whose reciprocal is normal, else 0.
+double exact_reciprocal(double d) {
+  int e;
+  return std::frexp(d, &e) == 0.5 && e > -1000 && e < 1000 ? 1.0 / d : 0.0;
 }
 
 }  // namespace
 
-cudaError_t launch_rhs_fp64(int ndim, RhsParamsF64& p, cudaStream_t s) {
-  p.a.use_tma = ndim == 2 && encode_tile_map(p.a) ? 1 : 0;
-  if (ndim == 2) {
-    using G = Geom<2>;
-    constexpr size_t sm = rhs_smem_bytes<2>();
-    cudaError_t e = cudaFuncSetAttribute(rhs_fp64_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    dim3 grid((p.a.nx + G::TX - 1) / G::TX, (p.a.ny + G::TY - 1) / G::TY);
-    rhs_fp64_kernel<2><<<grid, kThreads, sm, s>>>(p);
-  } else {
-    using G = Geom<1>;
-    constexpr size_t sm = rhs_smem_bytes<1>();
-    cudaError_t e = cudaFuncSetAttribute(rhs_fp64_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    if (e != cudaSuccess) return e;
-    dim3 grid((p.a.nx + G::TX - 1) / G::TX, 1);
-    rhs_fp64_kernel<1><<<grid, kThreads, sm, s>>>(p);
-  }
-  return cudaGetLastError();
+cudaError_t launch_rhs_fp64(int ndim, RhsArgs& a, cudaStream_t s) {
+  a.inv_dx = exact_reciprocal(a.dx);
+  a.inv_dy = ndim == 2 ? exact_reciprocal(a.dy) : 0.0;
+  if (ndim == 2) return launch_tiles<Tile<2, 16, 16, 192, 2, false>>(a, s);
+  return launch_tiles<Tile<1, 191, 1, 192, 2, false>>(a, s);
 }
 
 cudaError_t launch_classify_fp64(const ClassifyParamsF64& p, bool narrow, cudaStream_t s) {

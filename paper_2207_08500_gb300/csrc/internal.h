@@ -29,13 +29,31 @@ enum MaskMode { kMaskMLP = 0, kMaskSmooth = 1, kMaskRough = 2, kMaskTeno = 3, kM
 constexpr int kTenoTable = 79;
 void teno_tables(double out[kTenoTable]);
 
-// Arguments of one RHS / RK3-stage launch.  The tensor map (filled by
-// launch_rhs_fp64) describes U as a [nv][ny][nx] float64 tensor with the box
-// of one FP64 tile and its halo; use_tma = 0 when U cannot be described (odd
-// nx, 1D) and every tile is loaded with plain loads.
+// FP32 table of the certified classifier filter (mlp_filter.cuh), in floats:
+// k0 and the six input coefficients, then per unit of layer 1 its six weights,
+// bias and kappa, and for the layers after it W transposed ([in][out]), bias
+// and kappa of the outputs (none for layer 5).
+constexpr int kFiltIn = 0, kFiltW1 = 8;
+constexpr int kFiltW2 = kFiltW1 + 64 * 8, kFiltB2 = kFiltW2 + 64 * 32, kFiltK2 = kFiltB2 + 32;
+constexpr int kFiltW3 = kFiltK2 + 32, kFiltB3 = kFiltW3 + 32 * 16, kFiltK3 = kFiltB3 + 16;
+constexpr int kFiltW4 = kFiltK3 + 16, kFiltB4 = kFiltW4 + 16 * 8, kFiltK4 = kFiltB4 + 8;
+constexpr int kFiltW5 = kFiltK4 + 8, kFiltB5 = kFiltW5 + 8 * 4, kFiltFloats = kFiltB5 + 4;
+static_assert(kFiltFloats % 4 == 0, "copied in 16-byte chunks");
+struct FilterKappa {
+  double scale[4];  // logit k's row of W5 and b5 is multiplied by this
+  float k0, in[6], h1[64], h2[32], h3[16], h4[8];
+};
+// Device blob of a network: the binary64 parameters with every W transposed,
+// then the filter table.  Written by a one-CTA kernel from launch parameters,
+// so it can be launched under stream capture.
+constexpr size_t kNetBlobBytes = kNetParams * sizeof(double) + kFiltFloats * sizeof(float);
+static_assert(kNetParams * sizeof(double) % 16 == 0, "the table is 16-byte aligned");
+cudaError_t launch_net_blob(const NetF64& net, void* blob, cudaStream_t s);
+
+// Arguments of one RHS / RK3-stage launch.
 struct RhsArgs {
-  CUtensorMap tmap;
-  int use_tma;
+  const double* net64;  // blob: transposed binary64 parameters
+  const float* filter;  // blob: filter table
   const double* U;   // state the right-hand side is evaluated on
   const double* U0;  // state at the start of the RK3 step (stages 2, 3)
   double* out;       // dU/dt (stage 0) or the next stage state
@@ -50,16 +68,12 @@ struct RhsArgs {
   int mask_mode;
   int stage;  // 0 = dU/dt; 1, 2, 3 = SSP-RK3 stages
   double dx, dy, gamma, gm1;
+  double inv_dx, inv_dy;  // exact reciprocals, 0 where there is none (launch_rhs_fp64)
   double cfl, t_end;
   double third, two_thirds;
   double cand[4][4];   // candidate coefficients, stencil order
   double wtab[16][4];  // renormalised weights d_k / sum(kept d) per mask
   double teno[kTenoTable];  // TENO6-opt indicator matrices (mask_mode kMaskTeno)
-};
-
-struct RhsParamsF64 {
-  RhsArgs a;
-  NetF64 net;
 };
 
 struct ClassifyParamsF64 {
@@ -190,7 +204,7 @@ cudaError_t launch_cfl_mixed(int ndim, const double* U, int nx, int ny, double g
 cudaError_t launch_dt(const unsigned long long* smax, int ndim, double dx, double dy, double cfl, double t_end,
                       const double* t_dev, double* dt_dev, double* dt_user, cudaStream_t s);
 
-cudaError_t launch_rhs_fp64(int ndim, RhsParamsF64& p, cudaStream_t s);
+cudaError_t launch_rhs_fp64(int ndim, RhsArgs& a, cudaStream_t s);
 cudaError_t launch_classify_mixed(const double* X, long long n, uint8_t* eta, double* logits,
                                   const uint8_t* net_image, bool bf16, bool narrow, int* status,
                                   cudaStream_t s);

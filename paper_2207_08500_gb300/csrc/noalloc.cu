@@ -18,9 +18,11 @@ namespace {
 // Largest state (nv * nx * ny float64 values) one call may advance.
 constexpr size_t kMaxElems = NENO6_NOALLOC_MAX_STATE_ELEMS;
 // Layout of the static array, in float64 slots: stage 1, stage 2, then the
-// small words (CFL maxima x2, dt, t, status).
+// small words (CFL maxima x2, dt, t, status)
 constexpr size_t kSmall = 8;
-static __device__ __align__(256) double g_noalloc_scratch[2 * kMaxElems + kSmall];
+// ... and the classifier blob of the call's network.
+constexpr size_t kBlob = (kNetBlobBytes + sizeof(double) - 1) / sizeof(double);
+static __device__ __align__(256) double g_noalloc_scratch[2 * kMaxElems + kSmall + kBlob];
 
 constexpr int kMaxDevices = 64;
 // Per device: the array's device address and the id of the context it was
@@ -116,6 +118,7 @@ extern "C" int neno6_step_noalloc(const neno6_config* cfg, const double* net_par
   double* S1 = base;
   double* S2 = base + kMaxElems;
   double* small = base + 2 * kMaxElems;
+  double* blob = small + kSmall;
   unsigned long long* smax = reinterpret_cast<unsigned long long*>(small);
   double* dt_s = small + 2;
   double* t_s = small + 3;
@@ -133,42 +136,50 @@ extern "C" int neno6_step_noalloc(const neno6_config* cfg, const double* net_par
     if (e != cudaSuccess) return NENO6_ERR_CUDA;
   }
 
-  // Launch parameters (26 KB; on the stack, no heap allocation).
-  RhsParamsF64 p;
-  std::memset(&p.a, 0, sizeof p.a);
-  std::memcpy(p.net.p, net_params, sizeof p.net.p);
+  // Launch parameters (on the stack, no heap allocation): the network, laid
+  // out in the static array by a one-CTA kernel, and the right-hand side's.
+  if (c.mask_mode == NENO6_MASK_MLP) {
+    NetF64 net;
+    std::memcpy(net.p, net_params, sizeof net.p);
+    e = launch_net_blob(net, blob, s);
+    if (e != cudaSuccess) return NENO6_ERR_CUDA;
+  }
+  RhsArgs a;
+  std::memset(&a, 0, sizeof a);
+  a.net64 = blob;
+  a.filter = reinterpret_cast<const float*>(blob + kNetParams);
   double d[4];
-  scheme_tables(c.linear_weights, d, p.a.cand, p.a.wtab);
-  p.a.nx = c.nx;
-  p.a.ny = c.ny;
-  p.a.bcx = c.bc[0];
-  p.a.bcy = c.bc[1];
-  p.a.dx = c.dx;
-  p.a.dy = c.dy;
-  p.a.gamma = c.gamma;
-  p.a.gm1 = c.gamma - 1.0;
-  p.a.third = 1.0 / 3.0;
-  p.a.two_thirds = 2.0 / 3.0;
-  p.a.mask_mode = c.mask_mode;
-  if (c.mask_mode == kMaskTeno) teno_tables(p.a.teno);
-  p.a.status = status;
-  p.a.smax = smax;
-  p.a.dt_dev = dt_s;
-  p.a.t_dev = t_dev ? t_dev : t_s;
-  p.a.dt_user = dt_dev;
-  p.a.cfl = cfl;
-  p.a.t_end = t_end;
-  p.a.U0 = U;
+  scheme_tables(c.linear_weights, d, a.cand, a.wtab);
+  a.nx = c.nx;
+  a.ny = c.ny;
+  a.bcx = c.bc[0];
+  a.bcy = c.bc[1];
+  a.dx = c.dx;
+  a.dy = c.dy;
+  a.gamma = c.gamma;
+  a.gm1 = c.gamma - 1.0;
+  a.third = 1.0 / 3.0;
+  a.two_thirds = 2.0 / 3.0;
+  a.mask_mode = c.mask_mode;
+  if (c.mask_mode == kMaskTeno) teno_tables(a.teno);
+  a.status = status;
+  a.smax = smax;
+  a.dt_dev = dt_s;
+  a.t_dev = t_dev ? t_dev : t_s;
+  a.dt_user = dt_dev;
+  a.cfl = cfl;
+  a.t_end = t_end;
+  a.U0 = U;
 
   e = launch_cfl_reduce(c.ndim, U, c.nx, c.ny, c.gamma, smax, status, s);
   if (e != cudaSuccess) return NENO6_ERR_CUDA;
   const double* in[3] = {U, S1, S2};
   double* outp[3] = {S1, S2, U};
   for (int st = 1; st <= 3; ++st) {
-    p.a.stage = st;
-    p.a.U = in[st - 1];
-    p.a.out = outp[st - 1];
-    e = launch_rhs_fp64(c.ndim, p, s);
+    a.stage = st;
+    a.U = in[st - 1];
+    a.out = outp[st - 1];
+    e = launch_rhs_fp64(c.ndim, a, s);
     if (e != cudaSuccess) return NENO6_ERR_CUDA;
   }
   return NENO6_OK;
