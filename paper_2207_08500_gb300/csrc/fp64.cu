@@ -20,9 +20,9 @@
 // wrap or zero-gradient copy done in the load) and the per-cell quantities are
 // staged in shared memory, the faces' fluxes written back there and
 // differenced, with no scratch in global memory.  Comparisons (ReLU, max, |x|)
-// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 14.4 ms,
+// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 13.6 ms,
 // against 437 ms with every classifier row in binary64 and four lanes per
-// face; the FP64 operations alone would take 7.8 ms of a full FP64 pipe.
+// face; the FP64 operations alone would take 7.9 ms of a full FP64 pipe.
 #include <cmath>
 
 #include "fp64_ops.cuh"
@@ -45,6 +45,7 @@ struct Tile {
   static constexpr int NV = NDIM == 2 ? 4 : 3;
   static constexpr int HY = NDIM == 2 ? 3 : 0;
   static constexpr int SX = TX + 6, SY = TY + 2 * HY, NC = SX * SY;
+  static constexpr int NCELLS = TY * SX + 2 * HY * TX;        // staged cells: no corners
   static constexpr int NXF = TY * (TX + 1);                   // x faces
   static constexpr int NYF = NDIM == 2 ? (TY + 1) * TX : 0;   // y faces
   static constexpr int WX = (NXF + 31) / 32, WY = (NYF + 31) / 32;  // runs of 32 faces
@@ -182,9 +183,15 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
     // physical; the tile's faces then take every operation of the
     // specification literally (below).
     bool odd = false;
-    for (int e = t; e < NC; e += NT) {
-      const int bx = e % SX, by = e / SX;
-      if (NDIM == 2 && (bx < 3 || bx >= TX + 3) && (by < 3 || by >= TY + 3)) continue;
+    for (int k = t; k < G::NCELLS; k += NT) {
+      // the rows of the tile with their x halo, then the y halo
+      int bx = k % SX, by = G::HY + k / SX;
+      if (NDIM == 2 && k >= TY * SX) {
+        const int h = k - TY * SX, row = h / TX;
+        bx = 3 + h % TX;
+        by = row < 3 ? row : TY + row;
+      }
+      const int e = by * SX + bx;
       const int gi = wrap_index(i0 - 3 + bx, nx, a.bcx);
       const int gj = NDIM == 2 ? wrap_index(j0 - 3 + by, ny, a.bcy) : 0;
       const size_t g = (size_t)gj * nx + gi;
@@ -701,8 +708,32 @@ double exact_reciprocal(double d) {
 cudaError_t launch_rhs_fp64(int ndim, RhsArgs& a, cudaStream_t s) {
   a.inv_dx = exact_reciprocal(a.dx);
   a.inv_dy = ndim == 2 ? exact_reciprocal(a.dy) : 0.0;
-  if (ndim == 2) return launch_tiles<Tile<2, 16, 16, 192, 2, false>>(a, s);
-  return launch_tiles<Tile<1, 191, 1, 192, 2, false>>(a, s);
+  // Tiles whose (TX + 1) TY x faces and (TY + 1) TX y faces fill whole runs of
+  // 32 (the FP64 pipe takes 64 clocks per warp instruction and SM quarter
+  // however few lanes are active): 2.13 face slots per cell for 15 x 16, 2.29
+  // for 7 x 16 and 7 x 8.  The smaller the grid, the smaller the tile, so that
+  // every SM has warps; the smallest grids give a warp a single field.
+  // Measured in us per RHS, periodic quadrants:
+  //             24x16   64x64  130x97 200x136 300x300   512^2   1024^2   2048^2
+  //   15 x 16    242     179     187     187     420     974     3533    13621
+  //   7 x 16     144      98     104     139     362     907     3535    13920
+  //   7 x 8       95      56      77     145     364     919     3609    14298
+  //   7 x 3 SPLIT 70      48     110     203     561    1454     5669    22704
+  // (16 x 16 with 192 threads: 2048^2 in 14109.)
+  // 1D, n =                    400    4096   16384  131072
+  //   31 SPLIT                22.7    20.8    37.5   195
+  //   127                     43.2    41.4    43.4   181
+  const auto tiles = [&](int tx, int ty) {
+    return (long long)((a.nx + tx - 1) / tx) * ((a.ny + ty - 1) / ty);
+  };
+  if (ndim == 1) {
+    if (tiles(31, 1) <= 152 * 4) return launch_tiles<Tile<1, 31, 1, 96, 4, true>>(a, s);
+    return launch_tiles<Tile<1, 127, 1, 128, 3, false>>(a, s);
+  }
+  if (tiles(7, 3) <= 152 * 2) return launch_tiles<Tile<2, 7, 3, 256, 2, true>>(a, s);
+  if (tiles(7, 8) <= 152 * 3) return launch_tiles<Tile<2, 7, 8, 128, 3, false>>(a, s);
+  if (tiles(15, 16) < 152 * 2 * 12) return launch_tiles<Tile<2, 7, 16, 128, 3, false>>(a, s);
+  return launch_tiles<Tile<2, 15, 16, 192, 2, false>>(a, s);
 }
 
 cudaError_t launch_classify_fp64(const ClassifyParamsF64& p, bool narrow, cudaStream_t s) {

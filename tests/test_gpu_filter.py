@@ -78,12 +78,31 @@ def test_tiles_with_extreme_values(oracle_mod, tmp_path, kind, nx, ny):
     check(tmp_path, balanced_net(33), U, bc="transmissive")
 
 
-@pytest.mark.parametrize("nx,ny", [(1, 1), (15, 16), (16, 15), (17, 33), (48, 16), (31, 3), (3, 31), (130, 65)])
+# the last four lie on both sides of the sizes at which the tile changes
+@pytest.mark.parametrize("nx,ny", [(1, 1), (15, 16), (16, 15), (17, 33), (48, 16), (31, 3), (3, 31), (130, 65),
+                                   (133, 48), (134, 48), (168, 152), (169, 152)])
 @pytest.mark.parametrize("bc", ["periodic", "transmissive"])
 def test_tile_edges_2d(oracle_mod, tmp_path, nx, ny, bc):
     check(tmp_path, balanced_net(34), synth.noisy(synth.quadrants_2d(nx, ny, seed=7), 8), bc)
 
 
-@pytest.mark.parametrize("nx", [1, 5, 30, 31, 32, 63, 190, 191, 192, 383])
+@pytest.mark.parametrize("nx", [1, 5, 30, 31, 32, 63, 127, 383, 18848, 18849])
 def test_tile_edges_1d(oracle_mod, tmp_path, nx):
     check(tmp_path, balanced_net(35), synth.riemann_1d(nx, seed=9), "transmissive")
+
+
+def test_large_grid_tile(oracle_mod, tmp_path):
+    """The tile of large grids (from 3648 tiles of 15 x 16) on a ragged grid:
+    equal to the oracle on a band of rows cut out with its halo."""
+    import oracle
+    import paper_2207_08500_gb300 as p
+    nx, ny, r0, r1 = 15 * 61 - 4, 16 * 60 - 7, 300, 340
+    U = synth.noisy(synth.quadrants_2d(nx, ny, seed=10), 11)
+    net = balanced_net(36)
+    path = str(tmp_path / "net.bin")
+    net.save(path)
+    g = p.Neno6(ndim=2, nx=nx, ny=ny, weights=path)
+    d = g.rhs(torch.from_numpy(U).cuda()).cpu().numpy()
+    cut = np.ascontiguousarray(U[:, r0 - 3:r1 + 3])
+    o = oracle.Oracle(ndim=2, nx=nx, ny=r1 - r0 + 6, net=net, dx=1.0 / nx, dy=1.0 / ny)
+    assert np.array_equal(d[:, r0:r1], o.rhs(cut)[:, 3:-3])
