@@ -36,7 +36,6 @@ struct neno6_handle {
   float* d_guard_w = nullptr;      // FP32 transposed parameters (guard band)
   double* d_faces = nullptr;       // x- and y-face fluxes (mixed precision, lazily)
   uint8_t* d_mask = nullptr;       // classifier mask of the adjoint's forward pass (lazily)
-  double* d_vjp_rhs = nullptr;     // dU/dt of that forward pass (lazily)
   double* d_vjp_contrib = nullptr; // per-face adjoint contributions (lazily)
   float* d_params32 = nullptr;     // FP32 parameters, weights-file order
   double* d_net64 = nullptr;       // classifier blob of the FP64 kernels (kNetBlobBytes)
@@ -634,7 +633,6 @@ int neno6_destroy(neno6_handle* h) {
   cudaFree(h->d_faces);
   cudaFree(h->d_guard_count);
   cudaFree(h->d_mask);
-  cudaFree(h->d_vjp_rhs);
   cudaFree(h->d_vjp_contrib);
   cudaFree(h->d_params32);
   cudaFree(h->d_net64);
@@ -812,11 +810,12 @@ int neno6_rhs_vjp(neno6_handle* h, const double* U, const double* lambda, const 
     // to the forward FP64 right-hand side)
     cudaError_t e = cudaSuccess;
     if (!h->d_mask) e = cudaMalloc(&h->d_mask, (size_t)neno6_mask_bytes(h));
-    if (e == cudaSuccess && !h->d_vjp_rhs) e = cudaMalloc(&h->d_vjp_rhs, h->state_elems * sizeof(double));
-    if (e != cudaSuccess) return cuda_fail(h, e, "rhs_vjp: mask buffers");
+    if (e != cudaSuccess) {
+      h->d_mask = nullptr;
+      return cuda_fail(h, e, "rhs_vjp: mask buffer");
+    }
     fill_rhs_args(h, a);
     a.U = U;
-    a.out = h->d_vjp_rhs;
     a.mask_out = h->d_mask;
     a.stage = 0;
       e = launch_rhs_fp64(h->cfg.ndim, a, s);

@@ -400,6 +400,13 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
         } else {
           eta_side[0] = eta_side[1] = a.mask_mode == kMaskRough ? 15u : 0u;
         }
+        if (valid && a.mask_out) {
+          size_t idx;
+          if (dir == 0) idx = ((size_t)m * ny + gline) * (nx + 1) + gf;
+          else idx = (size_t)NV * ny * (nx + 1) + ((size_t)m * (ny + 1) + gf) * nx + gline;
+          a.mask_out[idx] = (uint8_t)(eta_side[0] | (eta_side[1] << 4));
+        }
+        if (!a.out) continue;  // the masks alone
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
           sp[j] = park[j * NT];
@@ -409,12 +416,6 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
 #pragma unroll
         for (int q = 0; q < NV; ++q)
           if (q == m) gh[q] = g;
-        if (valid && a.mask_out) {
-          size_t idx;
-          if (dir == 0) idx = ((size_t)m * ny + gline) * (nx + 1) + gf;
-          else idx = (size_t)NV * ny * (nx + 1) + ((size_t)m * (ny + 1) + gf) * nx + gline;
-          a.mask_out[idx] = (uint8_t)(eta_side[0] | (eta_side[1] << 4));
-        }
         if (G::SPLIT) {
           const int fi = (dir == 0 ? 0 : G::NXF) + face;
           double* sG = smem + G::O_G;
@@ -430,13 +431,14 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
         }
       }
       // Back-projection F_n = sum_m R[n][m] gh_m.
-      if (!G::SPLIT && fraw < nf) {
+      if (!G::SPLIT && a.out && fraw < nf) {
         double* dst = sF + (dir == 0 ? 0 : NV * G::NXF) + face;
 #pragma unroll
         for (int n = 0; n < NV; ++n) dst[n * nf] = back_project<NDIM>(r, dir, n, gh);
       }
     }
     __syncthreads();
+    if (!a.out) continue;
     if (G::SPLIT) {
       const double* sG = smem + G::O_G;
       for (int e = t; e < NV * (G::NXF + G::NYF); e += NT) {

@@ -56,7 +56,7 @@ struct RhsArgs {
   const float* filter;  // blob: filter table
   const double* U;   // state the right-hand side is evaluated on
   const double* U0;  // state at the start of the RK3 step (stages 2, 3)
-  double* out;       // dU/dt (stage 0) or the next stage state
+  double* out;       // dU/dt (stage 0) or the next stage state; null: mask_out alone
   const uint8_t* mask_in;
   uint8_t* mask_out;
   int* status;
