@@ -37,8 +37,8 @@ struct neno6_handle {
   double* d_faces = nullptr;       // x- and y-face fluxes (mixed precision, lazily)
   uint8_t* d_mask = nullptr;       // classifier mask of the adjoint's forward pass (lazily)
   double* d_vjp_contrib = nullptr; // per-face adjoint contributions (lazily)
+  double* d_net64 = nullptr;       // classifier blob of the FP64 kernels (kNetBlobBytes), then:
   float* d_params32 = nullptr;     // FP32 parameters, weights-file order
-  double* d_net64 = nullptr;       // classifier blob of the FP64 kernels (kNetBlobBytes)
   void* d_bwd_scratch = nullptr;   // per-CTA partial gradients (lazily)
   unsigned long long* d_guard_count = nullptr;
   cudaStream_t copy_stream = nullptr;  // neno6_step_host: band copies in and out (lazily)
@@ -576,14 +576,14 @@ int neno6_create(const neno6_config* cfg, const char* weights_path, neno6_handle
   if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMemset(h->d_t, 0, sizeof(double));
   if (e == cudaSuccess) {
-    std::vector<float> p32(kNetParams);
+    // one allocation and one copy: the FP64 kernels' blob, then the FP32 parameters
+    std::vector<double> img((kNetBlobBytes + kNetParams * sizeof(float) + 7) / 8);
+    float* p32 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(img.data()) + kNetBlobBytes);
+    if (!h->narrow) build_net_blob(h->net, img.data());
     for (int i = 0; i < kNetParams; ++i) p32[i] = (float)h->net.p[i];
-    e = cudaMalloc(&h->d_params32, kNetParams * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_params32, p32.data(), kNetParams * sizeof(float), cudaMemcpyHostToDevice);
-  }
-  if (e == cudaSuccess && !h->narrow) {
-    e = cudaMalloc(&h->d_net64, kNetBlobBytes);
-    if (e == cudaSuccess) e = launch_net_blob(h->net, h->d_net64, nullptr);
+    e = cudaMalloc(&h->d_net64, img.size() * sizeof(double));
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_net64, img.data(), img.size() * sizeof(double), cudaMemcpyHostToDevice);
+    h->d_params32 = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(h->d_net64) + kNetBlobBytes);
   }
   if (e == cudaSuccess && c.precision != NENO6_FP64) {
     std::vector<uint8_t> img(kNetImageBytes);
@@ -634,7 +634,6 @@ int neno6_destroy(neno6_handle* h) {
   cudaFree(h->d_guard_count);
   cudaFree(h->d_mask);
   cudaFree(h->d_vjp_contrib);
-  cudaFree(h->d_params32);
   cudaFree(h->d_net64);
   cudaFree(h->d_bwd_scratch);
   for (cudaEvent_t ev : h->band_in)

@@ -522,41 +522,6 @@ __global__ void __launch_bounds__(256) classify_fp64_narrow_kernel(const __grid_
   }
 }
 
-// The classifier parameters as the FP64 kernels read them: the binary64
-// weights transposed, then the FP32 table of the certified filter.
-__global__ void net_blob_kernel(const __grid_constant__ NetF64 net, const __grid_constant__ FilterKappa k,
-                                double* __restrict__ Wt, float* __restrict__ T) {
-  constexpr int W[6] = {6, 64, 32, 16, 8, 4};
-  const int kW[5] = {kFiltW1, kFiltW2, kFiltW3, kFiltW4, kFiltW5};
-  const int kB[5] = {0, kFiltB2, kFiltB3, kFiltB4, kFiltB5};
-  for (int i = threadIdx.x; i < kFiltFloats; i += blockDim.x) T[i] = 0.0f;
-  __syncthreads();
-  int p = 0;
-  for (int l = 0; l < 5; ++l) {
-    const int nin = W[l], nout = W[l + 1];
-    for (int e = threadIdx.x; e < nin * nout; e += blockDim.x) {
-      const int o = e / nin, i = e % nin;
-      const double w = net.p[p + e];
-      Wt[p + i * nout + o] = w;
-      if (l == 0) T[kFiltW1 + 8 * o + i] = (float)w;
-      else T[kW[l] + i * nout + o] = (float)(l == 4 ? w * k.scale[o] : w);
-    }
-    p += nin * nout;
-    for (int o = threadIdx.x; o < nout; o += blockDim.x) {
-      const double b = net.p[p + o];
-      Wt[p + o] = b;
-      if (l == 0) T[kFiltW1 + 8 * o + 6] = (float)b;
-      else T[kB[l] + o] = (float)(l == 4 ? b * k.scale[o] : b);
-    }
-    p += nout;
-  }
-  for (int i = threadIdx.x; i < 7; i += blockDim.x) T[kFiltIn + i] = i == 0 ? k.k0 : k.in[i - 1];
-  for (int i = threadIdx.x; i < 64; i += blockDim.x) T[kFiltW1 + 8 * i + 7] = k.h1[i];
-  for (int i = threadIdx.x; i < 32; i += blockDim.x) T[kFiltK2 + i] = k.h2[i];
-  for (int i = threadIdx.x; i < 16; i += blockDim.x) T[kFiltK3 + i] = k.h3[i];
-  for (int i = threadIdx.x; i < 8; i += blockDim.x) T[kFiltK4 + i] = k.h4[i];
-}
-
 __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
   return a > b ? a : b;
 }
@@ -678,12 +643,36 @@ static void build_filter_kappa(const NetF64& net, FilterKappa& out) {
   out.k0 = up(worst);
 }
 
-cudaError_t launch_net_blob(const NetF64& net, void* blob, cudaStream_t s) {
+void build_net_blob(const NetF64& net, void* blob) {
+  constexpr int W[6] = {6, 64, 32, 16, 8, 4};
+  constexpr int kW[5] = {kFiltW1, kFiltW2, kFiltW3, kFiltW4, kFiltW5}, kB[5] = {0, kFiltB2, kFiltB3, kFiltB4, kFiltB5};
   FilterKappa k;
   build_filter_kappa(net, k);
   double* Wt = static_cast<double*>(blob);
-  net_blob_kernel<<<1, 256, 0, s>>>(net, k, Wt, reinterpret_cast<float*>(Wt + kNetParams));
-  return cudaGetLastError();
+  float* T = reinterpret_cast<float*>(Wt + kNetParams);
+  for (int i = 0; i < kFiltFloats; ++i) T[i] = 0.0f;
+  int p = 0;
+  for (int l = 0; l < 5; ++l) {
+    const int nin = W[l], nout = W[l + 1];
+    for (int o = 0; o < nout; ++o) {
+      const double scale = l == 4 ? k.scale[o] : 1.0;
+      for (int i = 0; i < nin; ++i) {
+        const double w = net.p[p + o * nin + i];
+        Wt[p + i * nout + o] = w;
+        T[l == 0 ? kFiltW1 + 8 * o + i : kW[l] + i * nout + o] = (float)(w * scale);
+      }
+      const double b = net.p[p + nin * nout + o];
+      Wt[p + nin * nout + o] = b;
+      T[l == 0 ? kFiltW1 + 8 * o + 6 : kB[l] + o] = (float)(b * scale);
+    }
+    p += nin * nout + nout;
+  }
+  T[kFiltIn] = k.k0;
+  for (int i = 0; i < 6; ++i) T[kFiltIn + 1 + i] = k.in[i];
+  for (int i = 0; i < 64; ++i) T[kFiltW1 + 8 * i + 7] = k.h1[i];
+  for (int i = 0; i < 32; ++i) T[kFiltK2 + i] = k.h2[i];
+  for (int i = 0; i < 16; ++i) T[kFiltK3 + i] = k.h3[i];
+  for (int i = 0; i < 8; ++i) T[kFiltK4 + i] = k.h4[i];
 }
 
 namespace {

@@ -43,12 +43,11 @@ struct FilterKappa {
   double scale[4];  // logit k's row of W5 and b5 is multiplied by this
   float k0, in[6], h1[64], h2[32], h3[16], h4[8];
 };
-// Device blob of a network: the binary64 parameters with every W transposed,
-// then the filter table.  Written by a one-CTA kernel from launch parameters,
-// so it can be launched under stream capture.
+// Blob of a network as the FP64 kernels read it: the binary64 parameters with
+// every W transposed, then the filter table.
 constexpr size_t kNetBlobBytes = kNetParams * sizeof(double) + kFiltFloats * sizeof(float);
 static_assert(kNetParams * sizeof(double) % 16 == 0, "the table is 16-byte aligned");
-cudaError_t launch_net_blob(const NetF64& net, void* blob, cudaStream_t s);
+void build_net_blob(const NetF64& net, void* blob);
 
 // Arguments of one RHS / RK3-stage launch.
 struct RhsArgs {

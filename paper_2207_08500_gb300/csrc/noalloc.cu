@@ -84,6 +84,16 @@ cudaError_t scratch_address(int dev, double** out) {
   return cudaSuccess;
 }
 
+// A piece of the blob as launch parameters (at most 32 KB of them).
+constexpr size_t kChunk = (kBlob + 1) / 2;
+struct Chunk {
+  double v[kChunk];
+};
+static_assert(sizeof(Chunk) <= 30 * 1024, "launch parameters");
+__global__ void put_chunk_kernel(const __grid_constant__ Chunk c, double* dst, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = c.v[i];
+}
+
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 }  // namespace
@@ -136,12 +146,21 @@ extern "C" int neno6_step_noalloc(const neno6_config* cfg, const double* net_par
     if (e != cudaSuccess) return NENO6_ERR_CUDA;
   }
 
-  // Launch parameters (on the stack, no heap allocation): the network, laid
-  // out in the static array by a one-CTA kernel, and the right-hand side's.
+  // The network's blob, laid out on the host stack and written by kernels that
+  // carry it in their launch parameters (no pageable copy: a captured call
+  // stays valid after the caller's arrays are gone).
   if (c.mask_mode == NENO6_MASK_MLP) {
     NetF64 net;
     std::memcpy(net.p, net_params, sizeof net.p);
-    e = launch_net_blob(net, blob, s);
+    double img[kBlob];
+    build_net_blob(net, img);
+    for (size_t at = 0; at < kBlob; at += kChunk) {
+      Chunk ch;
+      const int n = (int)(kBlob - at < kChunk ? kBlob - at : kChunk);
+      std::memcpy(ch.v, img + at, n * sizeof(double));
+      put_chunk_kernel<<<1, 256, 0, s>>>(ch, blob + at, n);
+    }
+    e = cudaGetLastError();
     if (e != cudaSuccess) return NENO6_ERR_CUDA;
   }
   RhsArgs a;
