@@ -1,13 +1,13 @@
-// Per-sample forward and backward pass of the classifier's training loss,
-// shared by the gradient kernel (mlp_bwd.cu) and the training kernel
-// (mlp_train.cu).  The network is the 6-64-32-16-8-4 ReLU MLP of Sec. 3.1,
+// Forward and backward pass of the classifier's training loss for the training
+// kernel (mlp_train.cu), and the parameter layout it shares with the gradient
+// kernel (mlp_bwd.cu).  The network is the 6-64-32-16-8-4 ReLU MLP of Sec. 3.1,
 // the loss the mean binary cross entropy of Eq. (Crossentropy) over the S = 4
 // sigmoid outputs, all in FP32.
 //
-// One thread per sample.  The weights W (weights-file order: per layer
-// W[out][in] then b[out]) are broadcast from shared memory; every layer's
-// input and every delta are staged feature-major in shared memory, column
-// `col` of rows of length PITCH, for the parameter-gradient sums that follow.
+// The weights W (weights-file order: per layer W[out][in] then b[out]) are
+// broadcast from shared memory; every layer's input and every delta are
+// staged feature-major in shared memory, column `col` of rows of length PITCH,
+// for the parameter-gradient sums that follow.
 #pragma once
 
 #include <cmath>
@@ -28,124 +28,16 @@ __device__ __forceinline__ float softplus(float z) {  // log(1 + e^z), stable
   return fmaxf(z, 0.0f) + log1pf(__expf(-fabsf(z)));
 }
 
-// Forward and backward pass of one sample (raw stencil x, label bits lab;
-// `live` false stages zeros).  inv_nS = 1 / (4 n) for a batch of n samples.
-// Adds the sample's BCE sum over the four outputs to `loss`.
-template <int PITCH>
-__device__ __forceinline__ void sample_fwd_bwd(const float* W, float* st, int col, bool live, const float (&xr)[6],
-                                               unsigned lab, float inv_nS, double& loss) {
-  // ---- forward (Eq. (normalizainput), (reconstuction), (activationfunction))
-  float x0[6], m = 1.0f;
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    x0[j] = live ? xr[j] : 0.0f;
-    m = fmaxf(m, fabsf(x0[j]));
-  }
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    x0[j] = x0[j] / m;
-    st[(kX0 + j) * PITCH + col] = x0[j];
-  }
-  float h1[64];
-#pragma unroll
-  for (int o = 0; o < 64; ++o) {
-    float a = W[wofs(0) + 384 + o];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) a = fmaf(W[wofs(0) + o * 6 + i], x0[i], a);
-    h1[o] = fmaxf(a, 0.0f);
-    st[(kX1 + o) * PITCH + col] = h1[o];
-  }
-  float h2[32];
-#pragma unroll
-  for (int o = 0; o < 32; ++o) {
-    float a = W[wofs(1) + 2048 + o];
-#pragma unroll
-    for (int i = 0; i < 64; ++i) a = fmaf(W[wofs(1) + o * 64 + i], h1[i], a);
-    h2[o] = fmaxf(a, 0.0f);
-    st[(kX2 + o) * PITCH + col] = h2[o];
-  }
-  float h3[16];
-#pragma unroll
-  for (int o = 0; o < 16; ++o) {
-    float a = W[wofs(2) + 512 + o];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) a = fmaf(W[wofs(2) + o * 32 + i], h2[i], a);
-    h3[o] = fmaxf(a, 0.0f);
-    st[(kX3 + o) * PITCH + col] = h3[o];
-  }
-  float h4[8];
-#pragma unroll
-  for (int o = 0; o < 8; ++o) {
-    float a = W[wofs(3) + 128 + o];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) a = fmaf(W[wofs(3) + o * 16 + i], h3[i], a);
-    h4[o] = fmaxf(a, 0.0f);
-    st[(kX4 + o) * PITCH + col] = h4[o];
-  }
-  // ---- output: loss and dL/dz = (sigma(z) - y) / (n S); ReLU masks of the
-  // backward pass are re-read from the staged activations (fewer live
-  // registers)
-  asm volatile("" ::: "memory");
-  float d5[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    float z = W[wofs(4) + 32 + k];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) z = fmaf(W[wofs(4) + k * 8 + i], h4[i], z);
-    const float yk = (float)((lab >> k) & 1u);
-    const float sig = 1.0f / (1.0f + __expf(-z));
-    // -[y log s + (1-y) log(1-s)] = softplus(z) - y z
-    if (live) loss += (double)(softplus(z) - yk * z);
-    d5[k] = live ? (sig - yk) * inv_nS : 0.0f;
-    st[(kD5 + k) * PITCH + col] = d5[k];
-  }
-  // ---- backward: delta_l = (W_{l+1}^T delta_{l+1}) * relu'(pre-activation)
-  float d4[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    float a = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) a = fmaf(W[wofs(4) + k * 8 + i], d5[k], a);
-    d4[i] = st[(kX4 + i) * PITCH + col] > 0.0f ? a : 0.0f;
-    st[(kD4 + i) * PITCH + col] = d4[i];
-  }
-  float d3[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    float a = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) a = fmaf(W[wofs(3) + k * 16 + i], d4[k], a);
-    d3[i] = st[(kX3 + i) * PITCH + col] > 0.0f ? a : 0.0f;
-    st[(kD3 + i) * PITCH + col] = d3[i];
-  }
-  float d2[32];
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    float a = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 16; ++k) a = fmaf(W[wofs(2) + k * 32 + i], d3[k], a);
-    d2[i] = st[(kX2 + i) * PITCH + col] > 0.0f ? a : 0.0f;
-    st[(kD2 + i) * PITCH + col] = d2[i];
-  }
-#pragma unroll
-  for (int i = 0; i < 64; ++i) {
-    float a = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 32; ++k) a = fmaf(W[wofs(1) + k * 64 + i], d2[k], a);
-    st[(kD1 + i) * PITCH + col] = st[(kX1 + i) * PITCH + col] > 0.0f ? a : 0.0f;
-  }
-}
-
-// The same forward and backward pass, the CTA's NW warps cooperating on up
-// to 32 samples (lane = sample = staged column `col`): every layer's outputs
-// are split among the warps (output o to warp o % NW), each output computed
-// exactly as above -- its bias (or 0), then an fma chain over its inputs in
-// ascending order, the inputs read back from the staged rows -- with a CTA
-// barrier between layers; warp 0 forms the outputs, the loss and dL/dz.  The
-// staged rows are therefore bit for bit those of sample_fwd_bwd, in a
-// quarter of its latency with four warps.  Every thread of the CTA must call
-// it: lanes with `active` false (no staged column) only meet the barriers,
-// active lanes past the batch pass `live` false.
+// Forward and backward pass of up to 32 samples (raw stencil x, label bits
+// lab; `live` false stages zeros), the CTA's NW warps cooperating (lane =
+// sample = staged column `col`): every layer's outputs are split among the
+// warps (output o to warp o % NW), each output its bias (or 0), then an fma
+// chain over its inputs in ascending order, the inputs read back from the
+// staged rows, with a CTA barrier between layers; warp 0 forms the outputs,
+// the loss and dL/dz (inv_nS = 1 / (4 n) for a batch of n samples) and adds
+// the sample's BCE sum over the four outputs to `loss`.  Every thread of the
+// CTA must call it: lanes with `active` false (no staged column) only meet
+// the barriers, active lanes past the batch pass `live` false.
 template <int PITCH, int NW, int kG = 8>
 __device__ __forceinline__ void sample_fwd_bwd_coop(const float* W, float* st, int col, int warp, bool active,
                                                     bool live, const float (&xr)[6], unsigned lab, float inv_nS,
