@@ -378,7 +378,7 @@ const char* neno6_last_error(const neno6_handle* h);
  *
  * Scratch: one file-scope static device array holding two stage states of at
  * most NENO6_NOALLOC_MAX_STATE_ELEMS float64 values each (4 MiB each) plus
- * the call's network (39 KB) and a few words; every GPU that loads the library holds it (8 MiB) until the
+ * the call's network (39 KB), wave-speed maxima (19 KB) and a few words; every GPU that loads the library holds it (8 MiB) until the
  * process exits.  Every call shares it and it keeps the previous call's
  * contents; the call clears what must start at zero.  Calls whose work
  * overlaps on the GPU (different streams, or different host threads) race on

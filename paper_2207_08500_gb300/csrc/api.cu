@@ -26,7 +26,7 @@ struct neno6_handle {
   double cand[4][4];          // candidate coefficients
   double wtab[16][4];         // renormalised weights per mask pattern
   int* d_status = nullptr;    // device status word
-  unsigned long long* d_smax = nullptr;  // [2] CFL maxima
+  unsigned long long* d_smax = nullptr;  // CFL maxima (FP64: kCflBlocks per direction; mixed: two)
   double* d_dt = nullptr;     // dt of the current step
   double* d_t = nullptr;      // internal time (neno6_step with t_dev == NULL)
   double* d_stage = nullptr;  // two RK3 stage states (lazily allocated)
@@ -570,7 +570,7 @@ int neno6_create(const neno6_config* cfg, const char* weights_path, neno6_handle
   h->state_elems = (size_t)h->nv * c.nx * c.ny;
   cudaError_t e = cudaGetDevice(&h->device);
   if (e == cudaSuccess) e = cudaMalloc(&h->d_status, sizeof(int));
-  if (e == cudaSuccess) e = cudaMalloc(&h->d_smax, 2 * sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMalloc(&h->d_smax, 2 * kCflBlocks * sizeof(unsigned long long));
   if (e == cudaSuccess) e = cudaMalloc(&h->d_dt, sizeof(double));
   if (e == cudaSuccess) e = cudaMalloc(&h->d_t, sizeof(double));
   if (e == cudaSuccess) e = cudaMemset(h->d_status, 0, sizeof(int));
@@ -693,11 +693,13 @@ int neno6_step(neno6_handle* h, double* U, double cfl, double t_end, double* t_d
   if (h->cfg.precision != NENO6_FP64) return mixed_step(h, U, cfl, t_end, t_dev, dt_dev, nullptr, nullptr, s);
   double* S1 = h->d_stage;
   double* S2 = h->d_stage + h->state_elems;
-  cudaError_t e = launch_cfl_reduce(h->cfg.ndim, U, h->cfg.nx, h->cfg.ny, h->cfg.gamma, h->d_smax, h->d_status, s);
+  int nsmax = 0;
+  cudaError_t e = launch_cfl_reduce(h->cfg.ndim, U, h->cfg.nx, h->cfg.ny, h->cfg.gamma, h->d_smax, &nsmax, h->d_status, s);
   if (e != cudaSuccess) return cuda_fail(h, e, "step: cfl reduction");
   RhsArgs& a = h->rhs_args;
   fill_rhs_args(h, a);
   a.smax = h->d_smax;
+  a.nsmax = nsmax;
   a.dt_dev = h->d_dt;
   a.t_dev = t_dev ? t_dev : h->d_t;
   a.dt_user = dt_dev;

@@ -24,6 +24,7 @@
 // against 437 ms with every classifier row in binary64 and four lanes per
 // face; the FP64 operations alone would take 7.9 ms of a full FP64 pipe.
 #include <cmath>
+#include <utility>
 
 #include "fp64_ops.cuh"
 #include "internal.h"
@@ -33,6 +34,8 @@ namespace neno6 {
 namespace {
 
 using namespace f64ops;
+
+constexpr int kCflThreads = 128;  // one warp per SM quarter
 
 // Tile of TX x TY cells (TY = 1 in 1D) worked on by NT threads, OCC CTAs per
 // SM.  Faces are dealt to warps in runs of 32 of one direction.  SPLIT: a
@@ -57,12 +60,13 @@ struct Tile {
   static constexpr int kPark = 12;  // per thread: the "+" stencil, the mirrored "-" stencil
   static constexpr int kScratch = 128;  // per warp (binary64 classifier)
   // doubles: planes, face fluxes, parked stencils, warp scratch, and for
-  // SPLIT the faces' field fluxes and Roe states; then the FP32 table
+  // SPLIT the faces' field fluxes and Roe states; dt; then the FP32 table
   static constexpr int O_F = NPLANES * NC;
   static constexpr int O_P = O_F + NV * (NXF + NYF);
   static constexpr int O_W = O_P + kPark * NT;
   static constexpr int O_G = O_W + kScratch * (NT / 32);
-  static constexpr int O_T = (O_G + (SPLIT ? (NV + 5) * (NXF + NYF) : 0) + 1) / 2 * 2;
+  static constexpr int O_D = O_G + (SPLIT ? (NV + 5) * (NXF + NYF) : 0);
+  static constexpr int O_T = (O_D + 2) / 2 * 2;
   static constexpr size_t SMEM = sizeof(double) * O_T + sizeof(float) * kFiltFloats;
   static_assert(NT % 32 == 0 && OCC * (SMEM + 1024) <= 228 * 1024, "resident CTAs");
 };
@@ -72,6 +76,23 @@ __device__ __forceinline__ bool moderate(double x) {
   const unsigned long long b = (unsigned long long)dbits(x) & 0x7fffffffffffffffULL;
   return b == 0ull || (unsigned)(b >> 32) - (963u << 20) < (120u << 20);
 }
+// Programmatic dependent launch: the next kernel of the stream may be set up
+// (and run up to its own wait) while this one runs; the wait returns when every
+// earlier kernel of the stream has completed and its writes are visible.
+__device__ __forceinline__ void dependents_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_earlier_kernels() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
+  return a > b ? a : b;
+}
+__device__ __forceinline__ void warp_umax(unsigned long long& x, unsigned long long& y) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    x = umax64(x, __shfl_xor_sync(0xffffffffu, x, o));
+    y = umax64(y, __shfl_xor_sync(0xffffffffu, y, o));
+  }
+}
+
 // x / 2 for x = 0 or 2^-1021 <= |x| < inf, on the integer pipe.
 __device__ __forceinline__ double half_exact(double x) {
   const int hi = __double2hiint(x);
@@ -155,24 +176,40 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
   const size_t plane = (size_t)nx * ny;
   const double gm1 = a.gm1, gamma = a.gamma;
   const double* __restrict__ Wt = a.net64;
+  // the table is the handle's own and not written by the kernels before this
+  // one, so it is fetched while they drain (dependent_launch below); their
+  // results are read after the wait
   if (a.mask_mode == kMaskMLP) filt::load_filter(T, a.filter, t, NT);
+  dependents_may_launch();
+  wait_for_earlier_kernels();
 
-  // dt of an RK3 step (stage 1 computes it from max(|u|+c), max(|v|+c)).
-  double dt = 0.0;
-  if (a.stage == 1) {
-    const double sx = __longlong_as_double((long long)a.smax[0]);
-    double s = __ddiv_rn(sx, a.dx);
-    if (NDIM == 2) s = __dadd_rn(s, __ddiv_rn(__longlong_as_double((long long)a.smax[1]), a.dy));
-    dt = __ddiv_rn(a.cfl, s);
+  // dt of an RK3 step (stage 1 computes it from max(|u|+c), max(|v|+c)), by the
+  // last warp, which has the fewest cells, into shared memory until step 3.
+  double* sdt = smem + G::O_D;
+  if (a.stage && warp == NT / 32 - 1) {
     const double tm = *a.t_dev;
-    if (a.t_end > 0.0 && __dadd_rn(tm, dt) > a.t_end) dt = __dsub_rn(a.t_end, tm);
-    if (blockIdx.x == 0 && t == 0) {
-      *a.dt_dev = dt;
-      if (a.dt_user) *a.dt_user = dt;
+    double dt;
+    if (a.stage == 1) {
+      // maxima over the reduction's CTAs
+      unsigned long long mx = 0, my = 0;
+      for (int i = lane; i < a.nsmax; i += 32) {
+        mx = umax64(mx, a.smax[i]);
+        if (NDIM == 2) my = umax64(my, a.smax[kCflBlocks + i]);
+      }
+      warp_umax(mx, my);
+      double s = __ddiv_rn(__longlong_as_double((long long)mx), a.dx);
+      if (NDIM == 2) s = __dadd_rn(s, __ddiv_rn(__longlong_as_double((long long)my), a.dy));
+      dt = __ddiv_rn(a.cfl, s);
+      if (a.t_end > 0.0 && __dadd_rn(tm, dt) > a.t_end) dt = __dsub_rn(a.t_end, tm);
+      if (blockIdx.x == 0 && lane == 0) {
+        *a.dt_dev = dt;
+        if (a.dt_user) *a.dt_user = dt;
+      }
+    } else {
+      dt = *a.dt_dev;
+      if (a.stage == 3 && blockIdx.x == 0 && lane == 0) *a.t_dev = __dadd_rn(tm, dt);
     }
-  } else if (a.stage >= 2) {
-    dt = *a.dt_dev;
-    if (a.stage == 3 && blockIdx.x == 0 && t == 0) *a.t_dev = __dadd_rn(*a.t_dev, dt);
+    if (lane == 0) *sdt = dt;
   }
 
   const long long ntx = (nx + TX - 1) / TX, ntiles = ntx * ((ny + TY - 1) / TY);
@@ -242,6 +279,7 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
       }
     }
     odd |= !moderate(gm1);
+    filt::table_ready();
     odd = __syncthreads_or(odd);
 
     // ---- 2. faces
@@ -461,12 +499,16 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
     // ---- 3. conservative difference and (optionally) the RK3 stage update.
     // A division by a power of two is the exact product with its reciprocal.
     const double* sFy = sF + NV * G::NXF;
+    const double dt = a.stage ? *sdt : 0.0;
     for (int e = t; e < TX * TY; e += NT) {
       const int c = e % TX, rw = e / TX;
       const int gi = i0 + c, gj = j0 + rw;
       if (gi >= nx || gj >= ny) continue;
       const size_t g = (size_t)gj * nx + gi;
       const int bc = (G::HY + rw) * SX + 3 + c;
+      double u0[NV];  // loaded before the stores, which may alias it
+#pragma unroll
+      for (int n = 0; n < NV; ++n) u0[n] = a.stage >= 2 ? a.U0[n * plane + g] : 0.0;
 #pragma unroll
       for (int n = 0; n < NV; ++n) {
         const double dF = __dsub_rn(sF[(n * TY + rw) * (TX + 1) + c + 1], sF[(n * TY + rw) * (TX + 1) + c]);
@@ -480,9 +522,9 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
         if (a.stage == 1) {
           val = __fma_rn(dt, rr, Ucur);
         } else if (a.stage == 2) {
-          val = __fma_rn(0.75, a.U0[n * plane + g], __dmul_rn(0.25, __fma_rn(dt, rr, Ucur)));
+          val = __fma_rn(0.75, u0[n], __dmul_rn(0.25, __fma_rn(dt, rr, Ucur)));
         } else if (a.stage == 3) {
-          val = __fma_rn(a.third, a.U0[n * plane + g], __dmul_rn(a.two_thirds, __fma_rn(dt, rr, Ucur)));
+          val = __fma_rn(a.third, u0[n], __dmul_rn(a.two_thirds, __fma_rn(dt, rr, Ucur)));
         }
         a.out[n * plane + g] = val;
       }
@@ -522,19 +564,19 @@ __global__ void __launch_bounds__(256) classify_fp64_narrow_kernel(const __grid_
   }
 }
 
-__device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) {
-  return a > b ? a : b;
-}
-
-// max over cells of |u|+c (and |v|+c): bit patterns of non-negative doubles
-// order like the values, so integer max / atomicMax give the exact maximum.
+// max over a CTA's cells of |u|+c (and |v|+c), one value per CTA: bit patterns
+// of non-negative doubles order like the values, so integer max gives the exact
+// maximum.  The stage-1 kernel takes the maximum over the CTAs: nothing has to
+// be cleared before and nothing is contended.
 template <int NDIM>
-__global__ void __launch_bounds__(256) cfl_reduce_kernel(const double* __restrict__ U, int nx, int ny,
+__global__ void __launch_bounds__(kCflThreads) cfl_reduce_kernel(const double* __restrict__ U, int nx, int ny,
                                                          double gamma, unsigned long long* smax,
                                                          int* status) {
   const size_t plane = (size_t)nx * ny;
   const double gm1 = __dsub_rn(gamma, 1.0);
   unsigned long long mx = 0, my = 0;
+  dependents_may_launch();
+  wait_for_earlier_kernels();
   for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < plane;
        k += (size_t)gridDim.x * blockDim.x) {
     const double rho = U[k];
@@ -553,12 +595,8 @@ __global__ void __launch_bounds__(256) cfl_reduce_kernel(const double* __restric
     mx = umax64(mx, (unsigned long long)dbits(__dadd_rn(dabs(u), c)));
     if (NDIM == 2) my = umax64(my, (unsigned long long)dbits(__dadd_rn(dabs(v), c)));
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    mx = umax64(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    my = umax64(my, __shfl_xor_sync(0xffffffffu, my, o));
-  }
-  __shared__ unsigned long long wx[8], wy[8];
+  warp_umax(mx, my);
+  __shared__ unsigned long long wx[kCflThreads / 32], wy[kCflThreads / 32];
   const int warp = threadIdx.x >> 5;
   if ((threadIdx.x & 31) == 0) {
     wx[warp] = mx;
@@ -566,13 +604,37 @@ __global__ void __launch_bounds__(256) cfl_reduce_kernel(const double* __restric
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
+    for (int i = 1; i < kCflThreads / 32; ++i) {
       mx = umax64(mx, wx[i]);
       my = umax64(my, wy[i]);
     }
-    atomicMax(&smax[0], mx);
-    if (NDIM == 2) atomicMax(&smax[1], my);
+    smax[blockIdx.x] = mx;
+    if (NDIM == 2) smax[kCflBlocks + blockIdx.x] = my;
   }
+}
+
+}  // namespace
+
+namespace {
+
+// Launch a kernel that waits for its predecessors itself.  Small grids start
+// early (programmatic stream serialisation): of ten 1D 400-cell steps' 835 us
+// this takes 50, launch latency and the table's copy.  Grids of more than half
+// the SMs do not: their CTAs would be placed beside the running kernel's and end
+// up unevenly spread (200 x 136: 241 us per RHS against 191).
+template <class... P, class... A>
+cudaError_t dependent_launch(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = grid <= 76 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
 }
 
 }  // namespace
@@ -684,8 +746,7 @@ cudaError_t launch_tiles(const RhsArgs& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)((a.nx + G::TX - 1) / G::TX) * ((a.ny + G::TY - 1) / G::TY);
   const long long most = 152ll * G::OCC;
-  rhs_fp64_kernel<G><<<(unsigned)(tiles < most ? tiles : most), G::NT, G::SMEM, s>>>(a);
-  return cudaGetLastError();
+  return dependent_launch(rhs_fp64_kernel<G>, (unsigned)(tiles < most ? tiles : most), G::NT, G::SMEM, s, a);
 }
 
 // 1/d when d is a power of two whose reciprocal is normal, else 0.
@@ -738,17 +799,14 @@ cudaError_t launch_classify_fp64(const ClassifyParamsF64& p, bool narrow, cudaSt
 }
 
 cudaError_t launch_cfl_reduce(int ndim, const double* U, int nx, int ny, double gamma,
-                              unsigned long long* smax, int* status, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(smax, 0, 2 * sizeof(unsigned long long), s);
-  if (e != cudaSuccess) return e;
+                              unsigned long long* smax, int* nsmax, int* status, cudaStream_t s) {
   const size_t cells = (size_t)nx * ny;
-  unsigned blocks = (unsigned)((cells + 255) / 256);
-  if (blocks > 152u * 8u) blocks = 152u * 8u;
+  const size_t most = (cells + kCflThreads - 1) / kCflThreads;
+  const unsigned blocks = most < kCflBlocks ? (unsigned)most : (unsigned)kCflBlocks;
+  *nsmax = (int)blocks;
   if (ndim == 2)
-    cfl_reduce_kernel<2><<<blocks, 256, 0, s>>>(U, nx, ny, gamma, smax, status);
-  else
-    cfl_reduce_kernel<1><<<blocks, 256, 0, s>>>(U, nx, ny, gamma, smax, status);
-  return cudaGetLastError();
+    return dependent_launch(cfl_reduce_kernel<2>, blocks, kCflThreads, 0, s, U, nx, ny, gamma, smax, status);
+  return dependent_launch(cfl_reduce_kernel<1>, blocks, kCflThreads, 0, s, U, nx, ny, gamma, smax, status);
 }
 
 }  // namespace neno6

@@ -59,7 +59,8 @@ struct RhsArgs {
   const uint8_t* mask_in;
   uint8_t* mask_out;
   int* status;
-  const unsigned long long* smax;  // stage 1: bit patterns of max(|u|+c), max(|v|+c)
+  const unsigned long long* smax;  // stage 1: launch_cfl_reduce's maxima
+  int nsmax;                       // and their number per direction
   double* dt_dev;                  // stage 1 writes, stages 2/3 read
   double* t_dev;                   // stage 1 reads, stage 3 advances
   double* dt_user;                 // nullable copy of dt for the caller
@@ -259,7 +260,10 @@ cudaError_t launch_mlp_train(const MlpTrainArgs& a, cudaStream_t s);
 // Training data of Table 9 from uniform draws u [n][9] (csrc/datagen.cu).
 cudaError_t launch_datagen(const double* u, long long n, double* X, uint8_t* labels, uint8_t* family,
                            int* status, cudaStream_t s);
+// Wave-speed maxima of U as bit patterns, one per CTA and direction: max(|u|+c)
+// of CTA b in smax[b], max(|v|+c) in smax[kCflBlocks + b]; *nsmax CTAs.
+constexpr int kCflBlocks = 152 * 8;
 cudaError_t launch_cfl_reduce(int ndim, const double* U, int nx, int ny, double gamma,
-                              unsigned long long* smax, int* status, cudaStream_t s);
+                              unsigned long long* smax, int* nsmax, int* status, cudaStream_t s);
 
 }  // namespace neno6

@@ -18,8 +18,8 @@ namespace {
 // Largest state (nv * nx * ny float64 values) one call may advance.
 constexpr size_t kMaxElems = NENO6_NOALLOC_MAX_STATE_ELEMS;
 // Layout of the static array, in float64 slots: stage 1, stage 2, then the
-// small words (CFL maxima x2, dt, t, status)
-constexpr size_t kSmall = 8;
+// small words (dt, t, status) and the CFL maxima
+constexpr size_t kSmall = 4 + 2 * kCflBlocks;
 // ... and the classifier blob of the call's network.
 constexpr size_t kBlob = (kNetBlobBytes + sizeof(double) - 1) / sizeof(double);
 static __device__ __align__(256) double g_noalloc_scratch[2 * kMaxElems + kSmall + kBlob];
@@ -129,10 +129,10 @@ extern "C" int neno6_step_noalloc(const neno6_config* cfg, const double* net_par
   double* S2 = base + kMaxElems;
   double* small = base + 2 * kMaxElems;
   double* blob = small + kSmall;
-  unsigned long long* smax = reinterpret_cast<unsigned long long*>(small);
-  double* dt_s = small + 2;
-  double* t_s = small + 3;
-  int* status_s = reinterpret_cast<int*>(small + 4);
+  unsigned long long* smax = reinterpret_cast<unsigned long long*>(small + 4);
+  double* dt_s = small;
+  double* t_s = small + 1;
+  int* status_s = reinterpret_cast<int*>(small + 2);
   cudaStream_t s = static_cast<cudaStream_t>(stream);
 
   // The array keeps the previous call's contents: clear what starts at zero.
@@ -190,7 +190,7 @@ extern "C" int neno6_step_noalloc(const neno6_config* cfg, const double* net_par
   a.t_end = t_end;
   a.U0 = U;
 
-  e = launch_cfl_reduce(c.ndim, U, c.nx, c.ny, c.gamma, smax, status, s);
+  e = launch_cfl_reduce(c.ndim, U, c.nx, c.ny, c.gamma, smax, &a.nsmax, status, s);
   if (e != cudaSuccess) return NENO6_ERR_CUDA;
   const double* in[3] = {U, S1, S2};
   double* outp[3] = {S1, S2, U};
