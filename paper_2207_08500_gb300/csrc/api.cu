@@ -379,6 +379,9 @@ DiffArgs diff_args(const neno6_handle* h, const double* U, const double* U0, dou
   d.j1 = j1;
   d.inv_dx = 1.0 / h->cfg.dx;
   d.inv_dy = 1.0 / h->cfg.dy;
+  int e = 0;
+  const bool pow2 = std::frexp(d.inv_dx, &e) == 0.5;  // inv_dx = 2^(e-1)
+  d.pow2_x = pow2 && e > -62 && e < 64 ? e - 1 : 0;
   d.third = 1.0 / 3.0;
   d.two_thirds = 2.0 / 3.0;
   return d;

@@ -174,8 +174,12 @@ struct FacesMixedArgs {
   float wtab[16][4];
   // filled by the launcher: the launched x blocks are blk_x0 .. blk_x0 +
   // nblk_x - 1, then the y blocks blk_y0 .. blk_y0 + nblk_y - 1
-  long long blk_x0, nblk_x, blk_y0, nblk_y;
+  int blk_x0, nblk_x, blk_y0, nblk_y;
   int bxf, byc;
+  // likewise, kept out of the kernel's registers: nx * ny, gm1 / 2, gamma
+  size_t plane;
+  double hg1;
+  float gamma_f;
 };
 
 struct DiffArgs {
@@ -190,6 +194,7 @@ struct DiffArgs {
   int bcx, bcy;
   int j0, j1;        // rows j0 .. j1 - 1
   double inv_dx, inv_dy, third, two_thirds;
+  int pow2_x;        // inv_dx = 2^pow2_x with 0 < |pow2_x| < 64; 0: not such a power
 };
 
 // Face fluxes of the x faces of rows row0 .. row1 - 1 and of the y faces

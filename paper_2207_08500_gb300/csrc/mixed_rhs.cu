@@ -22,7 +22,14 @@
 // stage the 4 x 21 stencil cells (ghost cells by wrap / clamp), compute the
 // 64 Roe states once (one thread per face, FP64) while the other half of the
 // CTA forms the LLF alpha of every (face, field), then four 128-row
-// tensor-core batches of 16 faces x 4 fields x 2 sides.
+// tensor-core batches of 16 faces x 4 fields x 2 sides.  The kernel is bound by
+// the latency of that chain at 59 % of the issue slots and half of the FP64
+// pipe, so what counts is instructions, FP64 instructions (64 clocks of an SM
+// quarter each, whatever the active lanes) and registers kept across the
+// classifier: 2048^2 RHS 2.31 ms with exact halvings on the integer pipe, the
+// final FP64 addition of two batches in one instruction, the guard band in a
+// function of its own and its inputs formed anew, one 32-bit division per block
+// and no branch around the combination, 2.46 ms without them.
 //
 // Reference shift.  A cell near the block's centre is a reference state
 // (U_ref, F_ref); every cell is staged as the FP64 difference (U - U_ref,
@@ -66,11 +73,11 @@ constexpr int kOffNet = 0;
 // Scratch: during the staging and Roe phase of a block it holds the hand-off
 // of 20 cells' FP64 state (1280 B) and, from byte 2048, the FP64 Roe inputs of
 // every staged cell (4 x kMaxCells doubles); during the batches the guard
-// band's per-warp rows (4 x 128 floats).  The layer-1 input tile is free
+// band's per-warp hidden units (4 x 64 float4).  The layer-1 input tile is free
 // between blocks and holds each cell's FP32 (normal velocity, sound speed).
 constexpr int kCellDInScratch = 2048;
 constexpr int kScratchBytes = kCellDInScratch + 4 * kMaxCells * 8;
-static_assert(kCellDInScratch >= 20 * 64 && kCellDInScratch >= 4 * 128 * 4, "scratch layout");
+static_assert(kCellDInScratch >= 20 * 64 && kScratchBytes >= 4 * 64 * 16, "scratch layout");
 static_assert(kMaxCells * 8 <= kBufYBytes, "bufY reuse");
 constexpr int kOffScratch = align_up(kOffNet + kNetImageBytes);
 constexpr int kOffBufY = align_up(kOffScratch + kScratchBytes);
@@ -96,12 +103,22 @@ enum { CD_S = 0, CD_U = 1, CD_V = 2, CD_H = 3 };
 
 __device__ __forceinline__ int wrap_idx(int i, int n, int bc) {
   if (bc == 0) {
-    int r = i % n;
+    // a stencil reaches past the grid by less than a block: one period at most
+    // unless the grid is narrower
+    if (i < 0) i += n;
+    else if (i >= n) i -= n;
+    if ((unsigned)i < (unsigned)n) return i;
+    const int r = i % n;
     return r < 0 ? r + n : r;
   }
   return i < 0 ? 0 : (i >= n ? n - 1 : i);
 }
 
+// x / 2 on the integer pipe, for x = 0 or 2^-1021 <= x < inf (exact; the FP64
+// pipe takes 64 clocks of an SM quarter per warp instruction).
+__device__ __forceinline__ double half64(double x) {
+  return __hiloint2double(max(__double2hiint(x) - 0x00100000, 0), __double2loint(x));
+}
 // FP64 helpers of the mixed path: hardware reciprocal / reciprocal
 // square-root approximations refined by one Newton step (relative error
 // ~1e-10 or better).  That is ample here: every Roe quantity is rounded to
@@ -119,7 +136,7 @@ __device__ __forceinline__ double rsqrt64(double x) {
   double y;
   asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
   const double e = fma(-x, y * y, 1.0);
-  return fma(0.5 * y, e, y);
+  return fma(half64(y), e, y);
 }
 // x > 0 (and not NaN) on the integer pipe: the binary64 pattern of a
 // positive number (including +inf) is in (0, 0x7ff0000000000000].
@@ -151,85 +168,124 @@ __device__ __forceinline__ double f2d(float f) {
 }
 
 // Warp-cooperative FP32 re-evaluation of the classifier for the rows of this
-// warp whose lane has `flagged` set (guard band).  gw: FP32 parameters with
-// every W transposed ([in][out]), biases after each W.  ws: 128 floats of
-// per-warp shared scratch.
-__device__ __forceinline__ void guard_mlp(const float* __restrict__ gw, float* ws, const float (&x)[6],
-                                          float (&z)[4], bool flagged) {
+// warp whose lane has `flagged` set (guard band), four rows per pass (lane =
+// output of a layer; a pass costs its weight loads and its chains' latency, so
+// four rows take the time of one: near shocks the flagged rows come together;
+// 256 x 192, 1 % of the rows flagged: 75 us per RHS, one row per pass 104).
+// Every output is its bias, then one FMA chain over its inputs in ascending
+// order, for any number of rows.  gw: FP32 parameters with every W transposed
+// ([in][out]), biases after each W.  ws: 64 float4 of per-warp shared scratch,
+// element i holding hidden unit i of the four rows.
+// A function of its own, so that the registers it needs are taken where some
+// row is flagged and not from the batch loop.  `bal`: the flagged lanes; returns
+// the logits of the calling lane's row (z itself where it is not flagged).
+__device__ __noinline__ float4 guard_mlp(const float* __restrict__ gw, float4* ws, float2 x01, float2 x23, float2 x45,
+                                         float4 z4, unsigned bal) {
   const int lane = threadIdx.x & 31;
-  unsigned bal = __ballot_sync(0xffffffffu, flagged);
+  float* wf = reinterpret_cast<float*>(ws);
+  const float x[6] = {x01.x, x01.y, x23.x, x23.y, x45.x, x45.y};
+  float z[4] = {z4.x, z4.y, z4.z, z4.w};
   while (bal) {
-    const int src = __ffs(bal) - 1;
-    bal &= bal - 1;
-    float xs[6];
+    int src[4];
 #pragma unroll
-    for (int j = 0; j < 6; ++j) xs[j] = __shfl_sync(0xffffffffu, x[j], src);
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int o = lane + 32 * h;
-      float acc = gw[384 + o];
-#pragma unroll
-      for (int i = 0; i < 6; ++i) acc = fmaf(gw[i * 64 + o], xs[i], acc);
-      ws[o] = fmaxf(acc, 0.0f);
+    for (int r = 0; r < 4; ++r) {
+      src[r] = bal ? __ffs(bal) - 1 : src[0];
+      bal &= bal - 1;
     }
-    __syncwarp();
+    auto relu4 = [](const float (&v)[4]) {
+      return make_float4(fmaxf(v[0], 0.0f), fmaxf(v[1], 0.0f), fmaxf(v[2], 0.0f), fmaxf(v[3], 0.0f));
+    };
+    float a[4];
     {
-      float acc = gw[2496 + lane];
-#pragma unroll 8
-      for (int i = 0; i < 64; ++i) acc = fmaf(gw[448 + i * 32 + lane], ws[i], acc);
-      ws[64 + lane] = fmaxf(acc, 0.0f);
-    }
-    __syncwarp();
-    if (lane < 16) {
-      float acc = gw[3040 + lane];
-#pragma unroll 8
-      for (int i = 0; i < 32; ++i) acc = fmaf(gw[2528 + i * 16 + lane], ws[64 + i], acc);
-      ws[96 + lane] = fmaxf(acc, 0.0f);
-    }
-    __syncwarp();
-    if (lane < 8) {
-      float acc = gw[3184 + lane];
+      float b[4];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) acc = fmaf(gw[3056 + i * 8 + lane], ws[96 + i], acc);
-      ws[112 + lane] = fmaxf(acc, 0.0f);
-    }
-    __syncwarp();
-    if (lane < 4) {
-      float acc = gw[3224 + lane];
+      for (int r = 0; r < 4; ++r) {
+        a[r] = gw[384 + lane];
+        b[r] = gw[416 + lane];
+      }
 #pragma unroll
-      for (int i = 0; i < 8; ++i) acc = fmaf(gw[3192 + i * 4 + lane], ws[112 + i], acc);
-      ws[120 + lane] = acc;
-    }
-    __syncwarp();
-    if (lane == src) {
+      for (int i = 0; i < 6; ++i) {
+        const float wa = gw[i * 64 + lane], wb = gw[i * 64 + 32 + lane];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) z[k] = ws[120 + k];
+        for (int r = 0; r < 4; ++r) {
+          const float xs = __shfl_sync(0xffffffffu, x[i], src[r]);
+          a[r] = fmaf(wa, xs, a[r]);
+          b[r] = fmaf(wb, xs, b[r]);
+        }
+      }
+      ws[lane] = relu4(a);
+      ws[32 + lane] = relu4(b);
     }
     __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) a[r] = gw[2496 + lane];
+#pragma unroll 16
+    for (int i = 0; i < 64; ++i) {
+      const float w = gw[448 + i * 32 + lane];
+      const float4 h = ws[i];
+      a[0] = fmaf(w, h.x, a[0]);
+      a[1] = fmaf(w, h.y, a[1]);
+      a[2] = fmaf(w, h.z, a[2]);
+      a[3] = fmaf(w, h.w, a[3]);
+    }
+    __syncwarp();
+    ws[lane] = relu4(a);
+    __syncwarp();
+    {  // layer 3: sixteen outputs, two rows each per half warp
+      const int o = lane & 15, rp = lane >> 4;
+      float c0 = gw[3040 + o], c1 = c0;
+#pragma unroll 16
+      for (int i = 0; i < 32; ++i) {
+        const float w = gw[2528 + i * 16 + o];
+        const float2 h = reinterpret_cast<const float2*>(wf)[2 * i + rp];
+        c0 = fmaf(w, h.x, c0);
+        c1 = fmaf(w, h.y, c1);
+      }
+      __syncwarp();
+      reinterpret_cast<float2*>(wf)[2 * o + rp] = make_float2(fmaxf(c0, 0.0f), fmaxf(c1, 0.0f));
+      __syncwarp();
+    }
+    {  // layer 4: eight outputs x four rows
+      const int o = lane & 7, r = lane >> 3;
+      float c = gw[3184 + o];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) c = fmaf(gw[3056 + i * 8 + o], wf[4 * i + r], c);
+      __syncwarp();
+      wf[4 * o + r] = fmaxf(c, 0.0f);
+      __syncwarp();
+    }
+    {  // layer 5: output k of row r in lane 4 r + k, then to the row's own lane
+      const int k = lane & 3, r = (lane >> 2) & 3;
+      float c = gw[3224 + k];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) c = fmaf(gw[3192 + i * 4 + k], wf[4 * i + r], c);
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float v = __shfl_sync(0xffffffffu, c, 4 * q + j);
+          if (lane == src[q]) z[j] = v;
+        }
+    }
   }
+  return make_float4(z[0], z[1], z[2], z[3]);
 }
 
-// Geometry of launched block `blk`: the x blocks come first (kLines rows x
-// kLineFaces faces), then the y blocks (kLines columns x kLineFaces faces),
-// each range starting at its launch offset.
+// Geometry of a launched block: kLines lines (rows for x faces, columns for y
+// faces) from `line0` on, faces face0 .. face0 + kLineFaces - 1 of each.  The x
+// blocks come first, then the y blocks, each range starting at its launch
+// offset; consecutive blocks run along x.
 struct BlockGeom {
-  int dir;      // 0: x faces, 1: y faces
-  int row, f0;  // x block: first row, first face of each line
-  int i0, g0;   // y block: first column, first face of each line
+  int dir;           // 0: x faces, 1: y faces
+  int line0, face0;
 };
-__device__ __forceinline__ BlockGeom block_geom(long long blk, const FacesMixedArgs& a) {
-  BlockGeom b{0, 0, 0, 0, 0};
-  if (blk < a.nblk_x) {
-    blk += a.blk_x0;
-    b.row = (int)(blk / a.bxf) * kLines;
-    b.f0 = (int)(blk % a.bxf) * kLineFaces;
-  } else {
-    const long long q = blk - a.nblk_x + a.blk_y0;
-    b.dir = 1;
-    b.i0 = (int)(q % a.byc) * kLines;
-    b.g0 = (int)(q / a.byc) * kLineFaces;
-  }
-  return b;
+__device__ __forceinline__ BlockGeom block_geom(int blk, const FacesMixedArgs& a) {
+  const bool y = blk >= a.nblk_x;
+  const unsigned at = (unsigned)(y ? blk - a.nblk_x + a.blk_y0 : blk + a.blk_x0);
+  const unsigned per = (unsigned)(y ? a.byc : a.bxf);
+  const int q = (int)(at / per), r = (int)(at - (unsigned)q * per);
+  return BlockGeom{y ? 1 : 0, (y ? r : q) * kLines, (y ? q : r) * kLineFaces};
 }
 // Grid cell (j * nx + i) of staged cell c: ghost cells along the lines by
 // periodic wrap or clamp; lines beyond the grid clamp to its last line (their
@@ -237,11 +293,11 @@ __device__ __forceinline__ BlockGeom block_geom(long long blk, const FacesMixedA
 __device__ __forceinline__ size_t staged_cell(const BlockGeom& b, int c, const FacesMixedArgs& a) {
   int gi, gj;
   if (b.dir == 0) {
-    gi = wrap_idx(b.f0 - 3 + c % kLineCells, a.nx, a.bcx);
-    gj = min(b.row + c / kLineCells, a.ny - 1);
+    gi = wrap_idx(b.face0 - 3 + c % kLineCells, a.nx, a.bcx);
+    gj = min(b.line0 + c / kLineCells, a.ny - 1);
   } else {
-    gi = min(b.i0 + c % kLines, a.nx - 1);
-    gj = wrap_idx(b.g0 - 3 + c / kLines, a.ny, a.bcy);
+    gi = min(b.line0 + c % kLines, a.nx - 1);
+    gj = wrap_idx(b.face0 - 3 + c / kLines, a.ny, a.bcy);
   }
   return (size_t)gj * a.nx + gi;
 }
@@ -253,8 +309,8 @@ __device__ __forceinline__ int face_cb0(int dir, int k) {
 // Face k of the block exists on the grid (x faces 0..nx of rows 0..ny-1,
 // y faces 0..ny of columns 0..nx-1).
 __device__ __forceinline__ bool face_valid(const BlockGeom& b, int k, int nx, int ny) {
-  return b.dir == 0 ? (b.f0 + k % kLineFaces <= nx && b.row + k / kLineFaces < ny)
-                    : (b.g0 + k / kLines <= ny && b.i0 + k % kLines < nx);
+  return b.dir == 0 ? (b.face0 + k % kLineFaces <= nx && b.line0 + k / kLineFaces < ny)
+                    : (b.face0 + k / kLines <= ny && b.line0 + k % kLines < nx);
 }
 
 template <int NDIM, bool BF16>
@@ -267,16 +323,12 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
   float2* cuc = reinterpret_cast<float2*>(smem + kOffBufY);
   float* sL = reinterpret_cast<float*>(smem + kOffL);
   float* sA = reinterpret_cast<float*>(smem + kOffA);
-  float* ws = reinterpret_cast<float*>(smem + kOffScratch) + (threadIdx.x >> 5) * 128;
+  float4* ws = reinterpret_cast<float4*>(smem + kOffScratch) + (threadIdx.x >> 5) * 64;
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kOffBar);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffBar + 8);
   int* fail_flag = reinterpret_cast<int*>(smem + kOffBar + 12);
   const int t = threadIdx.x;
   const int nx = a.nx, ny = a.ny;
-  const size_t plane = (size_t)nx * ny;
-  const double gm1 = a.gm1;
-  const double hg1 = 0.5 * gm1;
-  const float gamma_f = (float)a.gamma;
 
   for (int i = t; i < kNetImageBytes / 16; i += kMlpThreads)
     reinterpret_cast<uint4*>(s_net)[i] = reinterpret_cast<const uint4*>(a.net_image)[i];
@@ -297,14 +349,14 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   MlpCtx mc{s_net, smem + kOffBufY, bar, *tmem_slot, 0u, BF16, fail_flag};
-  unsigned long long guarded = 0;
+  unsigned guarded = 0;
   bool failed = false;
 
-  const long long nblk = a.nblk_x + a.nblk_y;
+  const int nblk = a.nblk_x + a.nblk_y;
   double* refd = reinterpret_cast<double*>(smem + kOffRef);      // U_ref[4], F_ref[4] (FP64)
-  float* reff = reinterpret_cast<float*>(smem + kOffRef + 64);   // same, FP32
+  float* reff = reinterpret_cast<float*>(smem + kOffRef + 64);   // same, FP32, interleaved
   float* sRf = reinterpret_cast<float*>(smem + kOffR);           // ut, vt, Ht, ct, qt per face
-  for (long long blk = blockIdx.x; blk < nblk && !failed; blk += gridDim.x) {
+  for (int blk = (int)blockIdx.x; blk < nblk && !failed; blk += gridDim.x) {
     // ---- block geometry
     const BlockGeom bg = block_geom(blk, a);
     const int dir = bg.dir;
@@ -313,20 +365,20 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
     // thread index rotated by one warp per block, so that the partly
     // occupied cell and Roe phases fall on different warps (and SM
     // sub-partitions) from block to block
-    const int tr = (t + (int)((blk & 3) * 32)) & (kMlpThreads - 1);
+    const int tr = (t + (blk & 3) * 32) & (kMlpThreads - 1);
     // ---- stencil cells (one per thread): FP64 Roe inputs and fluxes
     double U[NV], F[4];
     if (tr < kMaxCells) {
       const size_t g = staged_cell(bg, tr, a);
 #pragma unroll
-      for (int n = 0; n < NV; ++n) U[n] = a.U[n * plane + g];
+      for (int n = 0; n < NV; ++n) U[n] = a.U[n * a.plane + g];
       const double rho = U[0], E = U[NV - 1];
       const double rs = rsqrt64(rho);  // 1/sqrt(rho)
       const double rr = rs * rs;       // 1/rho
       const double u = U[1] * rr;
       const double v = NDIM == 2 ? U[2] * rr : 0.0;
       const double rq = NDIM == 2 ? fma(U[2], v, U[1] * u) : U[1] * u;  // rho |u|^2
-      const double p = gm1 * fma(-0.5, rq, E);
+      const double p = a.gm1 * fma(-0.5, rq, E);
       const double Ep = E + p;
       if (!positive64(rho) || !positive64(p)) atomicOr(a.status, 1);
       cd[CD_S * kMaxCells + tr] = rho * rs;  // sqrt(rho)
@@ -340,7 +392,7 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
       } else {
         F[0] = U[2]; F[1] = U[1] * v; F[2] = fma(U[2], v, p); F[3] = Ep * v;
       }
-      cuc[tr] = make_float2(d2f(dir == 0 ? u : v), sqrtf(gamma_f * d2f(p) * d2f(rr)));
+      cuc[tr] = make_float2(d2f(dir == 0 ? u : v), sqrtf(a.gamma_f * d2f(p) * d2f(rr)));
       if (tr >= kFaces) {
         // cells kFaces.. are staged by Roe-phase threads: their deviations
         // are formed by the alpha-phase threads, from the scratch
@@ -356,8 +408,8 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
         for (int n = 0; n < 4; ++n) {
           refd[n] = n < NV ? U[n] : 0.0;
           refd[4 + n] = F[n];
-          reff[n] = n < NV ? d2f(U[n]) : 0.0f;
-          reff[4 + n] = d2f(F[n]);
+          reff[2 * n] = n < NV ? d2f(U[n]) : 0.0f;  // (U_n, F_n) pairs
+          reff[2 * n + 1] = d2f(F[n]);
         }
       }
     }
@@ -399,8 +451,8 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
       const double vt = fma(wb, cd[CD_V * kMaxCells + cb] - va, va);
       const double Ht = fma(wb, cd[CD_H * kMaxCells + cb] - Ha, Ha);
       const double qt = fma(vt, vt, ut * ut);
-      const double hq = 0.5 * qt;
-      const double c2 = gm1 * (Ht - hq);
+      const double hq = half64(qt);
+      const double c2 = a.gm1 * (Ht - hq);
       if (valid && !positive64(c2)) atomicOr(a.status, 2);
       const double ic = rsqrt64(c2);  // 1/c
       const double ct = c2 * ic;
@@ -408,9 +460,9 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
       // hb1 |u|^2/2, hic = 1/(2c).  L/2 is stored (the split's factor 1/2,
       // exact in binary): its entries are these halves rounded to FP32 and
       // scaled by exact powers of 2.
-      const double hb1 = hg1 * (ic * ic);
+      const double hb1 = a.hg1 * (ic * ic);
       const double hb2 = hb1 * hq;
-      const double hic = 0.5 * ic;
+      const double hic = half64(ic);
       const double hnc = (dir == 0 ? ut : vt) * hic;
       const double hb1u = hb1 * ut, hb1v = hb1 * vt;
       const double hbn = dir == 0 ? hb1u : hb1v;
@@ -449,6 +501,8 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
     }
     __syncthreads();
     // ---- four tensor-core batches of 16 faces x 4 fields x 2 sides
+    float corr_even = 0.0f;
+    unsigned ebits_even = 0u;
     for (int mt = 0; mt < kFaces / 16; ++mt) {
       const int k = mt * 16 + (t >> 3);
       const int fld = (t >> 1) & 3;
@@ -468,13 +522,12 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
       const float alpha = sA[k * 4 + m];
       const float sgn_alpha = side ? -alpha : alpha;
       // reference part of this side's split flux: (L F_ref +- alpha L U_ref)/2
-      float vr = Lr[0] * reff[0], gr = Lr[0] * reff[4];
-#pragma unroll
-      for (int n = 1; n < NV; ++n) {
-        vr = fmaf(Lr[n], reff[n], vr);
-        gr = fmaf(Lr[n], reff[4 + n], gr);
-      }
-      const float cref = fmaf(sgn_alpha, vr, gr);
+      const float4 rf0 = reinterpret_cast<const float4*>(reff)[0], rf1 = reinterpret_cast<const float4*>(reff)[1];
+      float2 vgr = __fmul2_rn(make_float2(Lr[0], Lr[0]), make_float2(rf0.x, rf0.y));
+      vgr = __ffma2_rn(make_float2(Lr[1], Lr[1]), make_float2(rf0.z, rf0.w), vgr);
+      vgr = __ffma2_rn(make_float2(Lr[2], Lr[2]), make_float2(rf1.x, rf1.y), vgr);
+      if (NV == 4) vgr = __ffma2_rn(make_float2(Lr[3], Lr[3]), make_float2(rf1.z, rf1.w), vgr);
+      const float cref = fmaf(sgn_alpha, vgr.x, vgr.y);
       // deviations of the split flux from the reference part, in this side's
       // stencil order ("+" side cells i-2..i+3, "-" side the mirror image
       // i+3..i-2).  Both sides of a (face, field), adjacent lanes, project the
@@ -519,6 +572,7 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
         store_input_row<BF16>(mc.bufY, t, x);
         fence_async_smem();
         __syncthreads();
+        asm volatile("" : "+f"(inv));  // x is formed anew below, not kept
         float z[4];
         if (!mlp_tc<BF16>(mc, z)) {
           failed = true;
@@ -529,7 +583,18 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
 #pragma unroll
           for (int q = 0; q < 4; ++q) flag |= fabsf(z[q]) < a.guard_tau;
           guarded += (flag && valid) ? 1 : 0;
-          guard_mlp(a.guard_w, ws, x, z, flag);
+          const unsigned bal = __ballot_sync(0xffffffffu, flag);
+          if (bal) {
+            // the inputs again, as above: two values live across the classifier
+            // instead of six
+            auto xin = [&](int j) { return (cref + ds[j]) * inv; };
+            const float4 zg = guard_mlp(a.guard_w, ws, make_float2(xin(0), xin(1)), make_float2(xin(2), xin(3)),
+                                        make_float2(xin(4), xin(5)), make_float4(z[0], z[1], z[2], z[3]), bal);
+            z[0] = zg.x;
+            z[1] = zg.y;
+            z[2] = zg.z;
+            z[3] = zg.w;
+          }
         }
         eta = 0;
 #pragma unroll
@@ -540,9 +605,7 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
       // candidates and renormalised combination of the deviations (FP32);
       // first-order fallback
       float gsum;
-      if (eta == 15u) {
-        gsum = ds[2];
-      } else {
+      {
         float f[4];
         f[0] = fmaf(a.cand[0][2], ds[3], fmaf(a.cand[0][1], ds[2], a.cand[0][0] * ds[1]));
         f[1] = fmaf(a.cand[1][2], ds[4], fmaf(a.cand[1][1], ds[3], a.cand[1][0] * ds[2]));
@@ -551,14 +614,16 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
         // discarded stencils have weight 0 in the table (fma(0, f, g) = g)
         const float4 w = s_wtab[eta];
         gsum = fmaf(w.w, f[3], fmaf(w.z, f[2], fmaf(w.y, f[1], w.x * f[0])));
+        gsum = eta == 15u ? ds[2] : gsum;
       }
       const float gh = gsum + __shfl_xor_sync(0xffffffffu, gsum, 1);
-      const unsigned eta_other = __shfl_xor_sync(0xffffffffu, eta, 1);
+      const unsigned eta_other = a.mask_out ? __shfl_xor_sync(0xffffffffu, eta, 1) : 0u;
       float ghq[4];
       const int fb = (t & 31) & ~7;
 #pragma unroll
       for (int q = 0; q < 4; ++q) ghq[q] = __shfl_sync(0xffffffffu, gh, fb + 2 * q);
-      if (side == 0 && valid) {
+      float corr = 0.0f;
+      if (side == 0) {
         // back-projection of the correction (FP32), plus F_ref (FP64)
         const float* Rd = sRf + k * 5;
         const float ut = Rd[0], vt = Rd[1], Ht = Rd[2], ct = Rd[3], qt = Rd[4];
@@ -574,7 +639,7 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
         const float A = is_rho ? 1.0f : (is_e ? Ht : (is_nrm ? nt : tt));
         const float B = is_e ? ntc : (is_nrm ? ct : 0.0f);
         const float C = is_rho ? 1.0f : (is_e ? 0.5f * qt : (is_nrm ? nt : tt));
-        float corr = (A - B) * ghq[0];
+        corr = (A - B) * ghq[0];
         corr = fmaf(C, ghq[1], corr);
         if (NDIM == 2) {
           const float D = is_e ? tt : ((is_rho || is_nrm) ? 0.0f : 1.0f);
@@ -583,26 +648,42 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
         } else {
           corr = fmaf(A + B, ghq[2], corr);
         }
-        const double Fh = refd[4 + n] + f2d(corr);
-        size_t idx;
-        if (dir == 0) {
-          const int f = bg.f0 + k % kLineFaces, r = bg.row + k / kLineFaces;
-          idx = ((size_t)n * ny + r) * (nx + 1) + f;
-          a.Fx[idx] = Fh;
-        } else {
-          const int g = bg.g0 + k / kLines, i = bg.i0 + k % kLines;
-          idx = ((size_t)n * (ny + 1) + g) * nx + i;
-          a.Fy[idx] = Fh;
-          idx += (size_t)NV * ny * (nx + 1);
+      }
+      // two batches at a time: the even one's corrections go to the odd lanes,
+      // so that the FP64 addition, the conversion and the stores of both are one
+      // instruction each
+      const unsigned ebits = eta | (eta_other << 4);
+      if ((mt & 1) == 0) {
+        corr_even = corr;
+        ebits_even = ebits;
+      } else {
+        const float ce = __shfl_xor_sync(0xffffffffu, corr_even, 1);
+        const int kw = side ? k - 16 : k;
+        if (fld < NV && face_valid(bg, kw, nx, ny)) {
+          const int n = m;
+          const double Fh = refd[4 + n] + f2d(side ? ce : corr);
+          size_t idx;
+          if (dir == 0) {
+            const int f = bg.face0 + kw % kLineFaces, r = bg.line0 + kw / kLineFaces;
+            idx = ((size_t)n * ny + r) * (nx + 1) + f;
+            a.Fx[idx] = Fh;
+          } else {
+            const int g = bg.face0 + kw / kLines, i = bg.line0 + kw % kLines;
+            idx = ((size_t)n * (ny + 1) + g) * nx + i;
+            a.Fy[idx] = Fh;
+            idx += (size_t)NV * ny * (nx + 1);
+          }
+          // the even batch's bits as the "-" side's lane holds them: swapped
+          if (a.mask_out)
+            a.mask_out[idx] = (uint8_t)(side ? (ebits_even >> 4) | ((ebits_even & 15u) << 4) : ebits);
         }
-        if (a.mask_out) a.mask_out[idx] = (uint8_t)(eta | (eta_other << 4));
       }
       __syncthreads();
     }
     __syncthreads();
   }
   if (failed && t == 0) atomicOr(a.status, 4);
-  if (a.guard_count && guarded) atomicAdd(a.guard_count, guarded);
+  if (a.guard_count && guarded) atomicAdd(a.guard_count, (unsigned long long)guarded);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -611,8 +692,21 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
 
 // Conservative difference (FP64) and optional SSP-RK3 stage update of the
 // rows j0 .. j1 - 1: thread per cell, a 2D grid of rows (blockIdx.y,
-// grid-stride beyond 65535 rows) by runs of 256 cells.  The difference of each direction is one DADD and the
-// two directions combine in one DMUL + DFMA: 4 FP64 operations per field.
+// grid-stride beyond 65535 rows) by runs of 256 cells.  Bound by the FP64 pipe:
+// the difference of each direction is one DADD and the two directions combine
+// in one DMUL + DFMA, 4 operations per field, and the stage adds up to 3; the
+// product with 1/dx, where that is a power of two, and the one with 1/4 are done
+// on the exponent instead (the same values).
+// x * 2^k on the integer pipe where x and the product are normal numbers, or x
+// is 0; by the product with `f` = 2^k otherwise.
+__device__ __forceinline__ double scale2(double x, int k, double f) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e - 64u < 1900u) return __hiloint2double(hi + k * 0x100000, lo);
+  if (((unsigned)hi << 1 | (unsigned)lo) == 0u) return x;
+  return x * f;
+}
+
 template <int NDIM>
 __global__ void __launch_bounds__(256) diff_mixed_kernel(DiffArgs a) {
   constexpr int NV = NDIM == 2 ? 4 : 3;
@@ -630,7 +724,8 @@ __global__ void __launch_bounds__(256) diff_mixed_kernel(DiffArgs a) {
 #pragma unroll
     for (int n = 0; n < NV; ++n) {
       const double* fx = a.Fx + ((size_t)n * a.ny + j) * (a.nx + 1);
-      const double rx = -a.inv_dx * (fx[ir] - fx[i]);
+      const double dF = fx[ir] - fx[i];
+      const double rx = a.pow2_x ? -scale2(dF, a.pow2_x, a.inv_dx) : -a.inv_dx * dF;
       double r = rx;
       if (NDIM == 2) {
         const double* fy = a.Fy + (size_t)n * (a.ny + 1) * a.nx + i;
@@ -639,7 +734,7 @@ __global__ void __launch_bounds__(256) diff_mixed_kernel(DiffArgs a) {
       const size_t e = n * plane + cell;
       double val = r;
       if (a.stage == 1) val = fma(dt, r, a.U[e]);
-      else if (a.stage == 2) val = fma(0.75, a.U0[e], 0.25 * fma(dt, r, a.U[e]));
+      else if (a.stage == 2) val = fma(0.75, a.U0[e], scale2(fma(dt, r, a.U[e]), -2, 0.25));
       else if (a.stage == 3) val = fma(a.third, a.U0[e], a.two_thirds * fma(dt, r, a.U[e]));
       a.out[e] = val;
     }
@@ -727,15 +822,19 @@ cudaError_t launch_faces_mixed(int ndim, FacesMixedArgs& a, cudaStream_t s, int 
   const int rg1 = row1 == a.ny ? (a.ny + kLines - 1) / kLines : row1 / kLines;
   const int fr0 = row0 / kLineFaces;
   const int fr1 = row1 == a.ny ? (a.ny + 1 + kLineFaces - 1) / kLineFaces : row1 / kLineFaces;
-  a.blk_x0 = (long long)a.bxf * rg0;
-  a.nblk_x = (long long)a.bxf * (rg1 - rg0);
-  a.blk_y0 = (long long)a.byc * fr0;
-  a.nblk_y = ndim == 2 ? (long long)a.byc * (fr1 - fr0) : 0;
-  const long long nblk = a.nblk_x + a.nblk_y;
+  // at most 2^34 cells: block numbers stay below 2^31
+  a.plane = (size_t)a.nx * a.ny;
+  a.hg1 = 0.5 * a.gm1;
+  a.gamma_f = (float)a.gamma;
+  a.blk_x0 = a.bxf * rg0;
+  a.nblk_x = a.bxf * (rg1 - rg0);
+  a.blk_y0 = a.byc * fr0;
+  a.nblk_y = ndim == 2 ? a.byc * (fr1 - fr0) : 0;
+  const int nblk = a.nblk_x + a.nblk_y;
   if (nblk <= 0) return cudaSuccess;
   // persistent grid: eight resident CTAs per SM (registers, shared memory,
   // 64 TMEM columns each)
-  const int blocks = (int)(nblk < 152 * 8 ? nblk : 152 * 8);
+  const int blocks = nblk < 152 * 8 ? nblk : 152 * 8;
   auto kern = ndim == 2 ? (a.bf16 ? faces_mixed_kernel<2, true> : faces_mixed_kernel<2, false>)
                         : (a.bf16 ? faces_mixed_kernel<1, true> : faces_mixed_kernel<1, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFacesSmem);
