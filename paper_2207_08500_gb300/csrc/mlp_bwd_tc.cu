@@ -38,60 +38,68 @@ using namespace tc;
 using namespace tcmlp;
 
 constexpr int kT = 128;
-constexpr uint32_t kSboS = (128 / 8) * 128;  // 8-row group stride of a K = 128 operand
-constexpr int kGroup = 2048;                  // bytes of one 8-row group at K = 128
+// Activations and deltas of a tile lie in shared memory by groups of eight
+// units: group g of a buffer is 128 samples x 16 bytes (eight 16-bit values), so
+// a thread stores its sample's eight units with one 16-byte store, without bank
+// conflicts.  One buffer serves two operands: M (or N) = units, K = samples
+// ("MN-major": the core matrix's 16-byte rows run along M) for the weight
+// gradients, M = samples, K = units (K-major) for the deltas, with the strides
+// between core matrices along units and samples
+constexpr int kGroup = 2048;
+constexpr uint32_t kUnits = kGroup, kSamples = 128;
 // shared memory (bytes): images, then the weight-gradient A operands (each
 // read as 16 groups = 32 KB from its start), then the rest
 constexpr int kOffNet = 0;
 constexpr int kOffBwd = kOffNet + kNetImageBytes;
-constexpr int kOffAH1T = kOffBwd + kBwdImageBytes;  // H1^T (64) + ones (row 64): 9 groups
-constexpr int kOffAH2T = kOffAH1T + 9 * kGroup;     // H2^T (32) + ones (row 32): 5 groups
-constexpr int kOffAH3T = kOffAH2T + 5 * kGroup;     // H3^T (16) + ones (row 16): 3 groups
-constexpr int kOffAH4T = kOffAH3T + 3 * kGroup;     // H4^T (8) + ones (row 8): 2 groups
-constexpr int kOffAD1T = kOffAH4T + 2 * kGroup;     // D1^T (64): 8 groups
-constexpr int kOffAX0 = kOffAD1T + 8 * kGroup;      // layer-1 input, 128 x 16
-constexpr int kOffAD3 = kOffAX0 + 128 * 16 * 2;     // D3, 128 x 16
-constexpr int kOffAD2 = kOffAD3 + 128 * 16 * 2;     // D2, 128 x 32
-constexpr int kOffBX0T = kOffAD2 + 128 * 32 * 2;    // X0^T (6) + ones (row 6), 16 x 128
-constexpr int kOffBD2T = kOffBX0T + 2 * kGroup;     // D2^T, 32 x 128
-constexpr int kOffBD3T = kOffBD2T + 4 * kGroup;     // D3^T, 16 x 128
-constexpr int kOffBD4T = kOffBD3T + 2 * kGroup;     // D4^T (8), 16 x 128
-constexpr int kOffBD5T = kOffBD4T + 2 * kGroup;     // D5^T (4), 16 x 128
-constexpr int kOffBar = kOffBD5T + 2 * kGroup;      // mbarrier, TMEM address, timeout flag
-constexpr int kOffLoss = kOffBar + 16;              // kT doubles
+constexpr int kOffH1 = kOffBwd + kBwdImageBytes;  // H1 (64 units), then 1 in unit 64: 9 groups
+constexpr int kOffH2 = kOffH1 + 9 * kGroup;       // H2 (32), 1 in unit 32: 5 groups
+constexpr int kOffH3 = kOffH2 + 5 * kGroup;       // H3 (16), 1 in unit 16: 3 groups
+constexpr int kOffH4 = kOffH3 + 3 * kGroup;       // H4 (8), 1 in unit 8: 2 groups
+constexpr int kOffD1 = kOffH4 + 2 * kGroup;       // D1 (64): 8 groups
+constexpr int kOffD2 = kOffD1 + 8 * kGroup;       // D2 (32): 4 groups
+constexpr int kOffD3 = kOffD2 + 4 * kGroup;       // D3 (16): 2 groups
+constexpr int kOffD4 = kOffD3 + 2 * kGroup;       // D4 (8 of 16): 2 groups
+constexpr int kOffD5 = kOffD4 + 2 * kGroup;       // D5 (4 of 16): 2 groups
+constexpr int kOffX0 = kOffD5 + 2 * kGroup;       // layer-1 input, 128 x 16, K-major (store_input_row)
+constexpr int kOffBar = kOffX0 + 128 * 16 * 2;    // mbarrier, TMEM address, timeout flag
+constexpr int kOffLoss = kOffBar + 16;            // kT doubles
 constexpr int kSmem = ((kOffLoss + kT * 8) + 127) / 128 * 128;
-static_assert(kOffAH1T % 128 == 0 && kOffAX0 % 128 == 0, "alignment");
-static_assert(kOffAD1T + 16 * kGroup <= kSmem, "the last weight-gradient A operand's 128 rows are addressable");
+static_assert(kOffH1 % 128 == 0 && kOffX0 % 128 == 0, "alignment");
+static_assert(kOffD1 + 16 * kGroup <= kSmem, "the last weight-gradient A operand's 128 rows are addressable");
 // two CTAs per SM (2 x 256 TMEM columns)
 static_assert(2 * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 // TMEM columns: forward / backward working area [0, 64), the weight-gradient
 // accumulators from column 128
 constexpr uint32_t kAcc1 = 128, kAcc2 = 144, kAcc3 = 176, kAcc4 = 192, kAcc5 = 208;
 
-__device__ __forceinline__ void st_u16(uint8_t* base, uint32_t off, uint16_t v) {
-  asm volatile("st.shared.u16 [%0], %1;" ::"r"(smem_u32(base + off)), "h"(v) : "memory");
+// Eight 16-bit units (group g of the buffer) of sample t.
+__device__ __forceinline__ void st_group(uint8_t* base, int g, int t, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(smem_u32(base + g * kGroup + t * 16)), "r"(a), "r"(b),
+               "r"(c), "r"(d)
+               : "memory");
 }
-template <bool BF16>
-__device__ __forceinline__ uint16_t bits16(float x) {
-  if (BF16) {
-    const __nv_bfloat16 b = __float2bfloat16_rn(x);
-    return *reinterpret_cast<const uint16_t*>(&b);
-  }
-  const __half h = __float2half_rn(x);
-  return *reinterpret_cast<const uint16_t*>(&h);
-}
-// Element (row, sample t) of a K = 128 operand (rows x 128 samples).
-__device__ __forceinline__ uint32_t kt_off(int row, int t) { return kmajor_offset(row, t, 128); }
 
-// D[col] (+)= A (128 x K rows in smem, group stride sbo) * B (N x K) ^ T,
-// K / 16 MMAs issued by this thread; acc0 = accumulate on the first step.
-__device__ __forceinline__ void mma_ss(uint32_t d_tmem, const uint8_t* A, uint32_t a_sbo, const uint8_t* B,
-                                       uint32_t b_sbo, int K, int N, bool bf16, bool acc0) {
+// D[col] (+)= A (units x samples) * B (units x samples)^T over the tile's 128
+// samples, both MN-major: unit groups a_mn / b_mn bytes apart, groups of eight
+// samples a_k / b_k; issued by this thread.
+__device__ __forceinline__ void mma_grad(uint32_t d_tmem, const uint8_t* A, const uint8_t* B, uint32_t b_mn,
+                                         uint32_t b_k, int N, bool bf16, bool acc0) {
+  const uint32_t idesc = idesc_f16(128, N, bf16) | (1u << 15) | (1u << 16);
+  const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks)
+    mma_f16(d_tmem, smem_desc(a0 + 2u * kSamples * ks, kSamples, kUnits), smem_desc(b0 + 2u * b_k * ks, b_k, b_mn),
+            idesc, (ks > 0 || acc0) ? 1u : 0u);
+}
+// D[col] = A (128 samples x K units, K-major) * W^T (N x K image at B).
+__device__ __forceinline__ void mma_delta(uint32_t d_tmem, const uint8_t* A, const uint8_t* B, uint32_t b_sbo, int K,
+                                          int N, bool bf16) {
   const uint32_t idesc = idesc_f16(128, N, bf16);
   const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
+#pragma unroll
   for (int ks = 0; ks < K / 16; ++ks)
-    mma_f16(d_tmem, smem_desc(a0 + 256u * ks, 128u, a_sbo), smem_desc(b0 + 256u * ks, 128u, b_sbo), idesc,
-            (ks > 0 || acc0) ? 1u : 0u);
+    mma_f16(d_tmem, smem_desc(a0 + 2u * kUnits * ks, kUnits, kSamples), smem_desc(b0 + 256u * ks, 128u, b_sbo), idesc,
+            ks > 0 ? 1u : 0u);
 }
 
 template <bool BF16>
@@ -111,20 +119,18 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
   const int t = threadIdx.x;
   const uint32_t lane = (uint32_t)(t & ~31) << 16;
 
-  // images; every operand buffer zeroed, then the constant rows of ones
+  // images; every operand buffer zeroed, then the constant units of one
   for (int i = t; i < kNetImageBytes / 16; i += kT)
     reinterpret_cast<uint4*>(s_net)[i] = reinterpret_cast<const uint4*>(net_image)[i];
   for (int i = t; i < kBwdImageBytes / 16; i += kT)
     reinterpret_cast<uint4*>(smem + kOffBwd)[i] = reinterpret_cast<const uint4*>(bwd_image)[i];
-  for (int i = t; i < (kOffBar - kOffAH1T) / 16; i += kT)
-    reinterpret_cast<uint4*>(smem + kOffAH1T)[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int i = t; i < (kOffBar - kOffH1) / 16; i += kT)
+    reinterpret_cast<uint4*>(smem + kOffH1)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  const uint16_t one = bits16<BF16>(1.0f);
-  st_u16(smem + kOffAH1T, kt_off(64, t), one);
-  st_u16(smem + kOffAH2T, kt_off(32, t), one);
-  st_u16(smem + kOffAH3T, kt_off(16, t), one);
-  st_u16(smem + kOffAH4T, kt_off(8, t), one);
-  st_u16(smem + kOffBX0T, kt_off(6, t), one);
+  st_group(smem + kOffH1, 8, t, one0<BF16>(), 0u, 0u, 0u);
+  st_group(smem + kOffH2, 4, t, one0<BF16>(), 0u, 0u, 0u);
+  st_group(smem + kOffH3, 2, t, one0<BF16>(), 0u, 0u, 0u);
+  st_group(smem + kOffH4, 1, t, one0<BF16>(), 0u, 0u, 0u);
   if (t == 0) {
     mbar_init(bar, 1);
     fence_mbar_init();
@@ -138,7 +144,7 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  MlpCtx mc{s_net, smem + kOffAX0, bar, tmem, 0u, BF16, fail};
+  MlpCtx mc{s_net, smem + kOffX0, bar, tmem, 0u, BF16, fail};
   const float* fbias = reinterpret_cast<const float*>(s_net + kNetImageBias);  // b3 at 0, b4 at 16, b5 at 24
   const float* W4 = reinterpret_cast<const float*>(s_bwd + kBwdW4);          // [8][16]
   const float* W5 = reinterpret_cast<const float*>(s_bwd + kBwdW5);          // [4][8]
@@ -160,14 +166,12 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     const unsigned lab = live ? y[s] : 0u;
     // the previous tile's weight-gradient MMAs read the operand buffers
     if (!first) wait_layer(mc);
-    store_input_row<BF16>(smem + kOffAX0, t, x0);
-#pragma unroll
-    for (int j = 0; j < 6; ++j) st_u16(smem + kOffBX0T, kt_off(j, t), bits16<BF16>(x0[j]));
+    store_input_row<BF16>(smem + kOffX0, t, x0);
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     // ---- layer 1 (bias on the ones columns) -> H1
-    if (t == 0) issue_layer<BF16>(mc, smem + kOffAX0, 16, kNetImageB1, 64, (int)kColD1);
+    if (t == 0) issue_layer<BF16>(mc, smem + kOffX0, 16, kNetImageB1, 64, (int)kColD1);
     wait_layer(mc);
     uint32_t mask1[2] = {0u, 0u};
 #pragma unroll
@@ -184,9 +188,10 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
         mask1[c32] |= (z0 > 0.0f ? 1u : 0u) << (2 * i);
         mask1[c32] |= (z1 > 0.0f ? 1u : 0u) << (2 * i + 1);
         pk[i] = relu_pack2<BF16>(z0, z1);
-        st_u16(smem + kOffAH1T, kt_off(32 * c32 + 2 * i, t), (uint16_t)(pk[i] & 0xffffu));
-        st_u16(smem + kOffAH1T, kt_off(32 * c32 + 2 * i + 1, t), (uint16_t)(pk[i] >> 16));
       }
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        st_group(smem + kOffH1, 4 * c32 + g, t, pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
       tmem_st16(tmem + lane + kColA2 + 16u * c32, pk);
     }
     tmem_st_wait();
@@ -209,9 +214,9 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
         mask2 |= (z0 > 0.0f ? 1u : 0u) << (2 * i);
         mask2 |= (z1 > 0.0f ? 1u : 0u) << (2 * i + 1);
         pk[i] = relu_pack2<BF16>(z0, z1);
-        st_u16(smem + kOffAH2T, kt_off(2 * i, t), (uint16_t)(pk[i] & 0xffffu));
-        st_u16(smem + kOffAH2T, kt_off(2 * i + 1, t), (uint16_t)(pk[i] >> 16));
       }
+#pragma unroll
+      for (int g = 0; g < 4; ++g) st_group(smem + kOffH2, g, t, pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
       tmem_st16(tmem + lane + kColA3, pk);
     }
     tmem_st_wait();
@@ -233,9 +238,9 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
         mask3 |= (z0 > 0.0f ? 1u : 0u) << (2 * i);
         mask3 |= (z1 > 0.0f ? 1u : 0u) << (2 * i + 1);
         pk[i] = relu_pack2<BF16>(z0, z1);
-        st_u16(smem + kOffAH3T, kt_off(2 * i, t), (uint16_t)(pk[i] & 0xffffu));
-        st_u16(smem + kOffAH3T, kt_off(2 * i + 1, t), (uint16_t)(pk[i] >> 16));
       }
+#pragma unroll
+      for (int g = 0; g < 2; ++g) st_group(smem + kOffH3, g, t, pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
       tmem_st8(tmem + lane + kColA4, pk);
     }
     tmem_st_wait();
@@ -255,8 +260,9 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
         const float z = __uint_as_float(r[i]) + fbias[16 + i];
         mask4 |= (z > 0.0f ? 1u : 0u) << i;
         h4[i] = fmaxf(z, 0.0f);
-        st_u16(smem + kOffAH4T, kt_off(i, t), bits16<BF16>(h4[i]));
       }
+      st_group(smem + kOffH4, 0, t, pack2<BF16>(h4[0], h4[1]), pack2<BF16>(h4[2], h4[3]), pack2<BF16>(h4[4], h4[5]),
+               pack2<BF16>(h4[6], h4[7]));
     }
     float d5[4];
 #pragma unroll
@@ -268,8 +274,8 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
       // -[y log s + (1-y) log(1-s)] = softplus(z) - y z
       if (live) loss += (double)(fmaxf(z, 0.0f) + log1pf(__expf(-fabsf(z))) - yk * z);
       d5[k] = live ? 1.0f / (1.0f + __expf(-z)) - yk : 0.0f;
-      st_u16(smem + kOffBD5T, kt_off(k, t), bits16<BF16>(d5[k]));
     }
+    st_group(smem + kOffD5, 0, t, pack2<BF16>(d5[0], d5[1]), pack2<BF16>(d5[2], d5[3]), 0u, 0u);
     float d4[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -277,8 +283,9 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
 #pragma unroll
       for (int k = 0; k < 4; ++k) a = fmaf(W5[k * 8 + i], d5[k], a);
       d4[i] = (mask4 >> i) & 1u ? a : 0.0f;
-      st_u16(smem + kOffBD4T, kt_off(i, t), bits16<BF16>(d4[i]));
     }
+    st_group(smem + kOffD4, 0, t, pack2<BF16>(d4[0], d4[1]), pack2<BF16>(d4[2], d4[3]), pack2<BF16>(d4[4], d4[5]),
+             pack2<BF16>(d4[6], d4[7]));
     float d3[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -286,22 +293,21 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
 #pragma unroll
       for (int k = 0; k < 8; ++k) a = fmaf(W4[k * 16 + i], d4[k], a);
       d3[i] = (mask3 >> i) & 1u ? a : 0.0f;
-      st_u16(smem + kOffBD3T, kt_off(i, t), bits16<BF16>(d3[i]));
     }
-    st_row8(smem + kOffAD3, t, 0, 16, pack2<BF16>(d3[0], d3[1]), pack2<BF16>(d3[2], d3[3]),
-            pack2<BF16>(d3[4], d3[5]), pack2<BF16>(d3[6], d3[7]));
-    st_row8(smem + kOffAD3, t, 8, 16, pack2<BF16>(d3[8], d3[9]), pack2<BF16>(d3[10], d3[11]),
-            pack2<BF16>(d3[12], d3[13]), pack2<BF16>(d3[14], d3[15]));
+#pragma unroll
+    for (int g = 0; g < 2; ++g)
+      st_group(smem + kOffD3, g, t, pack2<BF16>(d3[8 * g], d3[8 * g + 1]), pack2<BF16>(d3[8 * g + 2], d3[8 * g + 3]),
+               pack2<BF16>(d3[8 * g + 4], d3[8 * g + 5]), pack2<BF16>(d3[8 * g + 6], d3[8 * g + 7]));
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
     // ---- D2 = (D3 W3) * relu'(Z2); gradients of layers 5, 4, 3
     if (t == 0) {
       tc_fence_after();
-      mma_ss(tmem + 0u, smem + kOffAD3, 256u, s_bwd + kBwdBW3, 256u, 16, 32, BF16, false);
-      mma_ss(tmem + kAcc5, smem + kOffAH4T, kSboS, smem + kOffBD5T, kSboS, 128, 16, BF16, !first);
-      mma_ss(tmem + kAcc4, smem + kOffAH3T, kSboS, smem + kOffBD4T, kSboS, 128, 16, BF16, !first);
-      mma_ss(tmem + kAcc3, smem + kOffAH2T, kSboS, smem + kOffBD3T, kSboS, 128, 16, BF16, !first);
+      mma_delta(tmem + 0u, smem + kOffD3, s_bwd + kBwdBW3, 256u, 16, 32, BF16);
+      mma_grad(tmem + kAcc5, smem + kOffH4, smem + kOffD5, kUnits, kSamples, 16, BF16, !first);
+      mma_grad(tmem + kAcc4, smem + kOffH3, smem + kOffD4, kUnits, kSamples, 16, BF16, !first);
+      mma_grad(tmem + kAcc3, smem + kOffH2, smem + kOffD3, kUnits, kSamples, 16, BF16, !first);
       mma_commit(bar);
     }
     wait_layer(mc);
@@ -315,13 +321,11 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
       for (int i = 0; i < 32; ++i) {
         const float v = __uint_as_float(i < 16 ? r[i] : q[i - 16]);
         d2[i] = (mask2 >> i) & 1u ? v : 0.0f;
-        st_u16(smem + kOffBD2T, kt_off(i, t), bits16<BF16>(d2[i]));
       }
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
-        st_row8(smem + kOffAD2, t, 8 * c, 32, pack2<BF16>(d2[8 * c], d2[8 * c + 1]),
-                pack2<BF16>(d2[8 * c + 2], d2[8 * c + 3]), pack2<BF16>(d2[8 * c + 4], d2[8 * c + 5]),
-                pack2<BF16>(d2[8 * c + 6], d2[8 * c + 7]));
+      for (int g = 0; g < 4; ++g)
+        st_group(smem + kOffD2, g, t, pack2<BF16>(d2[8 * g], d2[8 * g + 1]), pack2<BF16>(d2[8 * g + 2], d2[8 * g + 3]),
+                 pack2<BF16>(d2[8 * g + 4], d2[8 * g + 5]), pack2<BF16>(d2[8 * g + 6], d2[8 * g + 7]));
     }
     fence_async_smem();
     tc_fence_before();
@@ -329,8 +333,8 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     // ---- D1 = (D2 W2) * relu'(Z1); gradient of layer 2
     if (t == 0) {
       tc_fence_after();
-      mma_ss(tmem + 0u, smem + kOffAD2, 512u, s_bwd + kBwdBW2, 512u, 32, 64, BF16, false);
-      mma_ss(tmem + kAcc2, smem + kOffAH1T, kSboS, smem + kOffBD2T, kSboS, 128, 32, BF16, !first);
+      mma_delta(tmem + 0u, smem + kOffD2, s_bwd + kBwdBW2, 512u, 32, 64, BF16);
+      mma_grad(tmem + kAcc2, smem + kOffH1, smem + kOffD2, kUnits, kSamples, 32, BF16, !first);
       mma_commit(bar);
     }
     wait_layer(mc);
@@ -341,9 +345,15 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
       tmem_ld16(tmem + lane + 32u * c32 + 16u, q);
       tmem_ld_wait();
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const float v = __uint_as_float(i < 16 ? r[i] : q[i - 16]);
-        st_u16(smem + kOffAD1T, kt_off(32 * c32 + i, t), bits16<BF16>((mask1[c32] >> i) & 1u ? v : 0.0f));
+      for (int g = 0; g < 4; ++g) {
+        uint32_t w[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const int i = 8 * g + 2 * h;
+          const float a = __uint_as_float(i < 16 ? r[i] : q[i - 16]), b = __uint_as_float(i < 16 ? r[i + 1] : q[i - 15]);
+          w[h] = pack2<BF16>((mask1[c32] >> i) & 1u ? a : 0.0f, (mask1[c32] >> (i + 1)) & 1u ? b : 0.0f);
+        }
+        st_group(smem + kOffD1, 4 * c32 + g, t, w[0], w[1], w[2], w[3]);
       }
     }
     fence_async_smem();
@@ -352,7 +362,10 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     // ---- gradient of layer 1 (waited for before the next tile's operands)
     if (t == 0) {
       tc_fence_after();
-      mma_ss(tmem + kAcc1, smem + kOffAD1T, kSboS, smem + kOffBX0T, kSboS, 128, 16, BF16, !first);
+      // the layer-1 input tile as the N operand: stencil values in columns 0-5,
+      // ones from ones_col on; its core matrices lie 128 bytes apart along the
+      // columns, 256 along the samples
+      mma_grad(tmem + kAcc1, smem + kOffD1, smem + kOffX0, 128u, 256u, 16, BF16, !first);
       mma_commit(bar);
     }
     first = false;
@@ -364,12 +377,12 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
   float* part = partial + (size_t)blockIdx.x * kNetParams;
   {
     uint32_t r[16];
-    tmem_ld16(tmem + lane + kAcc1, r);  // row o of dW1 (o < 64): cols 0..5, db1 in col 6
+    tmem_ld16(tmem + lane + kAcc1, r);  // row o of dW1 (o < 64): cols 0..5, db1 in col ones_col
     tmem_ld_wait();
     if (t < 64) {
 #pragma unroll
       for (int i = 0; i < 6; ++i) part[t * 6 + i] = __uint_as_float(r[i]);
-      part[384 + t] = __uint_as_float(r[6]);
+      part[384 + t] = __uint_as_float(r[ones_col(BF16)]);
     }
   }
 #pragma unroll
