@@ -39,10 +39,10 @@ using namespace tcmlp;
 // CTA's shared memory to ~28 KB, so that eight are resident per SM (their
 // 8 x 64 TMEM columns are exactly the SM's 512) and a ninth never is, whose
 // allocation would wait.
-constexpr int kResidencyPad = 14 * 1024;
-// static shared memory of the kernel below: image, input tile, barrier, TMEM
-// address, timeout flag
-constexpr int kClassifySmem = kNetImageBytes + kBufYBytes + 16;
+constexpr int kResidencyPad = 8 * 1024;
+// static shared memory of the kernel below: image, input tile, the next tile's
+// stencils, barriers, TMEM address, timeout flag
+constexpr int kClassifySmem = kNetImageBytes + kBufYBytes + 128 * 48 + 24;
 
 template <bool BF16, bool NARROW>
 __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const double* __restrict__ X,
@@ -52,15 +52,19 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
                                                                       int* status) {
   __shared__ __align__(128) uint8_t s_net[kNetImageBytes];
   __shared__ __align__(128) uint8_t s_bufY[kBufYBytes];
-  __shared__ __align__(8) uint64_t s_bar;
+  __shared__ __align__(128) double s_x[128 * 6];
+  __shared__ __align__(8) uint64_t s_bar, s_xbar;
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
   const int t = threadIdx.x;
   load_net_image(s_net, net_image);
+  TileRows rows{X, n, s_x, &s_xbar, 0u, (reinterpret_cast<uintptr_t>(X) & 15u) == 0};
   if (t == 0) {
     mbar_init(&s_bar, 1);
+    mbar_init(&s_xbar, 1);
     fence_mbar_init();
     s_fail = 0;
+    rows.fetch(blockIdx.x);
   }
   if (t < 32) {
     tmem_alloc(&s_tmem, 64);
@@ -75,19 +79,20 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
     const long long r = tile * 128 + t;
     float x[6];
     float m = 1.0f;
+    if (!rows.get(tile, x)) s_fail = 1;
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      x[j] = r < n ? (float)X[r * 6 + j] : 0.0f;
-      m = fmaxf(m, fabsf(x[j]));
-    }
+    for (int j = 0; j < 6; ++j) m = fmaxf(m, fabsf(x[j]));
 #pragma unroll
     for (int j = 0; j < 6; ++j) x[j] = x[j] / m;
     store_input_row<BF16>(s_bufY, t, x);
     fence_async_smem();
     __syncthreads();
+    if (t == 0) rows.fetch(tile + gridDim.x);
     float z[4];
     if (!(NARROW ? mlp_tc_narrow<BF16>(c, z) : mlp_tc<BF16>(c, z))) {
       if (t == 0) atomicOr(status, 4);
+      // a copy may still be in flight: wait for it (bounded) before leaving
+      rows.get(tile, x);
       break;
     }
     if (r < n) {

@@ -52,17 +52,24 @@ constexpr uint32_t kUnits = kGroup, kSamples = 128;
 constexpr int kOffNet = 0;
 constexpr int kOffBwd = kOffNet + kNetImageBytes;
 constexpr int kOffH1 = kOffBwd + kBwdImageBytes;  // H1 (64 units), then 1 in unit 64: 9 groups
+// H2, H3 and H4 follow one another, and D3, D4 and D5: one product of the two
+// runs holds the gradients of layers 3, 4 and 5 in its diagonal blocks (the rest
+// is not read), in a third of the MMAs and of the tensor memory
 constexpr int kOffH2 = kOffH1 + 9 * kGroup;       // H2 (32), 1 in unit 32: 5 groups
 constexpr int kOffH3 = kOffH2 + 5 * kGroup;       // H3 (16), 1 in unit 16: 3 groups
 constexpr int kOffH4 = kOffH3 + 3 * kGroup;       // H4 (8), 1 in unit 8: 2 groups
 constexpr int kOffD1 = kOffH4 + 2 * kGroup;       // D1 (64): 8 groups
 constexpr int kOffD2 = kOffD1 + 8 * kGroup;       // D2 (32): 4 groups
 constexpr int kOffD3 = kOffD2 + 4 * kGroup;       // D3 (16): 2 groups
-constexpr int kOffD4 = kOffD3 + 2 * kGroup;       // D4 (8 of 16): 2 groups
-constexpr int kOffD5 = kOffD4 + 2 * kGroup;       // D5 (4 of 16): 2 groups
-constexpr int kOffX0 = kOffD5 + 2 * kGroup;       // layer-1 input, 128 x 16, K-major (store_input_row)
-constexpr int kOffBar = kOffX0 + 128 * 16 * 2;    // mbarrier, TMEM address, timeout flag
-constexpr int kOffLoss = kOffBar + 16;            // kT doubles
+constexpr int kOffD4 = kOffD3 + 2 * kGroup;       // D4 (8)
+constexpr int kOffD5 = kOffD4 + kGroup;           // D5 (4 of 8)
+constexpr int kOffX0 = kOffD5 + kGroup;           // layer-1 input, 128 x 16, K-major (store_input_row)
+constexpr int kOffXs = kOffX0 + 128 * 16 * 2;     // the next tile's stencils, 128 x 6 doubles
+constexpr int kOffBar = kOffXs + 128 * 48;        // mbarrier, TMEM address, timeout flag, stencils' mbarrier
+constexpr int kOffLoss = kOffBar + 32;            // kT doubles
+// rows of the combined product's units
+constexpr int kRowH3 = 40, kRowH4 = 64;
+static_assert(kOffH3 - kOffH2 == kRowH3 / 8 * kGroup && kOffH4 - kOffH2 == kRowH4 / 8 * kGroup, "combined product");
 constexpr int kSmem = ((kOffLoss + kT * 8) + 127) / 128 * 128;
 static_assert(kOffH1 % 128 == 0 && kOffX0 % 128 == 0, "alignment");
 static_assert(kOffD1 + 16 * kGroup <= kSmem, "the last weight-gradient A operand's 128 rows are addressable");
@@ -70,7 +77,7 @@ static_assert(kOffD1 + 16 * kGroup <= kSmem, "the last weight-gradient A operand
 static_assert(2 * (kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 // TMEM columns: forward / backward working area [0, 64), the weight-gradient
 // accumulators from column 128
-constexpr uint32_t kAcc1 = 128, kAcc2 = 144, kAcc3 = 176, kAcc4 = 192, kAcc5 = 208;
+constexpr uint32_t kAcc1 = 128, kAcc2 = 144, kAcc3 = 176;  // kAcc3: layers 3, 4, 5
 
 // Eight 16-bit units (group g of the buffer) of sample t.
 __device__ __forceinline__ void st_group(uint8_t* base, int g, int t, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
@@ -91,8 +98,9 @@ __device__ __forceinline__ void mma_grad(uint32_t d_tmem, const uint8_t* A, cons
     mma_f16(d_tmem, smem_desc(a0 + 2u * kSamples * ks, kSamples, kUnits), smem_desc(b0 + 2u * b_k * ks, b_k, b_mn),
             idesc, (ks > 0 || acc0) ? 1u : 0u);
 }
-// D[col] = A (128 samples x K units, K-major) * W^T (N x K image at B).
-__device__ __forceinline__ void mma_delta(uint32_t d_tmem, const uint8_t* A, const uint8_t* B, uint32_t b_sbo, int K,
+// D[col] = A (128 samples x K units, K-major) * W^T (N x K image at B): a layer's
+// forward pass or its delta.
+__device__ __forceinline__ void mma_layer(uint32_t d_tmem, const uint8_t* A, const uint8_t* B, uint32_t b_sbo, int K,
                                           int N, bool bf16) {
   const uint32_t idesc = idesc_f16(128, N, bf16);
   const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
@@ -124,17 +132,21 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     reinterpret_cast<uint4*>(s_net)[i] = reinterpret_cast<const uint4*>(net_image)[i];
   for (int i = t; i < kBwdImageBytes / 16; i += kT)
     reinterpret_cast<uint4*>(smem + kOffBwd)[i] = reinterpret_cast<const uint4*>(bwd_image)[i];
-  for (int i = t; i < (kOffBar - kOffH1) / 16; i += kT)
+  for (int i = t; i < (kOffXs - kOffH1) / 16; i += kT)
     reinterpret_cast<uint4*>(smem + kOffH1)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   st_group(smem + kOffH1, 8, t, one0<BF16>(), 0u, 0u, 0u);
   st_group(smem + kOffH2, 4, t, one0<BF16>(), 0u, 0u, 0u);
   st_group(smem + kOffH3, 2, t, one0<BF16>(), 0u, 0u, 0u);
   st_group(smem + kOffH4, 1, t, one0<BF16>(), 0u, 0u, 0u);
+  TileRows rows{X, n, reinterpret_cast<double*>(smem + kOffXs), reinterpret_cast<uint64_t*>(smem + kOffBar + 16), 0u,
+                (reinterpret_cast<uintptr_t>(X) & 15u) == 0};
   if (t == 0) {
     mbar_init(bar, 1);
+    mbar_init(rows.bar, 1);
     fence_mbar_init();
     *fail = 0;
+    rows.fetch(blockIdx.x);
   }
   if (t < 32) {
     tmem_alloc(tmem_slot, 256);
@@ -155,15 +167,13 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     const long long s = tile * kT + t;
     const bool live = s < n;
     // ---- Eq. (normalizainput) in FP32
+    const unsigned lab = live ? y[s] : 0u;
     float x0[6], m = 1.0f;
+    if (!rows.get(tile, x0)) *fail = 1;
 #pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      x0[j] = live ? (float)X[s * 6 + j] : 0.0f;
-      m = fmaxf(m, fabsf(x0[j]));
-    }
+    for (int j = 0; j < 6; ++j) m = fmaxf(m, fabsf(x0[j]));
 #pragma unroll
     for (int j = 0; j < 6; ++j) x0[j] = x0[j] / m;
-    const unsigned lab = live ? y[s] : 0u;
     // the previous tile's weight-gradient MMAs read the operand buffers
     if (!first) wait_layer(mc);
     store_input_row<BF16>(smem + kOffX0, t, x0);
@@ -171,7 +181,10 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     tc_fence_before();
     __syncthreads();
     // ---- layer 1 (bias on the ones columns) -> H1
-    if (t == 0) issue_layer<BF16>(mc, smem + kOffX0, 16, kNetImageB1, 64, (int)kColD1);
+    if (t == 0) {
+      issue_layer<BF16>(mc, smem + kOffX0, 16, kNetImageB1, 64, (int)kColD1);
+      rows.fetch(tile + gridDim.x);
+    }
     wait_layer(mc);
     uint32_t mask1[2] = {0u, 0u};
 #pragma unroll
@@ -192,13 +205,18 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
 #pragma unroll
       for (int g = 0; g < 4; ++g)
         st_group(smem + kOffH1, 4 * c32 + g, t, pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
-      tmem_st16(tmem + lane + kColA2 + 16u * c32, pk);
     }
-    tmem_st_wait();
+    fence_async_smem();
     tc_fence_before();
     __syncthreads();
     // ---- layer 2 (bias K-step on the layer-1 input tile) -> H2
-    if (t == 0) issue_layer_t<BF16>(mc, kColA2, 64, kNetImageB2, 32, kColD2, kNetImageB2b);
+    if (t == 0) {
+      tc_fence_after();
+      mma_layer(tmem + kColD2, smem + kOffH1, s_net + kNetImageB2, 1024u, 64, 32, BF16);
+      mma_f16(tmem + kColD2, smem_desc(smem_u32(smem + kOffX0), 128u, 256u),
+              smem_desc(smem_u32(s_net + kNetImageB2b), 128u, 256u), idesc_f16(128, 32, BF16), 1u);
+      mma_commit(bar);
+    }
     wait_layer(mc);
     uint32_t mask2 = 0u;
     {
@@ -217,13 +235,16 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
       }
 #pragma unroll
       for (int g = 0; g < 4; ++g) st_group(smem + kOffH2, g, t, pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
-      tmem_st16(tmem + lane + kColA3, pk);
     }
-    tmem_st_wait();
+    fence_async_smem();
     tc_fence_before();
     __syncthreads();
     // ---- layer 3 (+ b3 in FP32) -> H3
-    if (t == 0) issue_layer_t<BF16>(mc, kColA3, 32, kNetImageB3, 16, kColD3);
+    if (t == 0) {
+      tc_fence_after();
+      mma_layer(tmem + kColD3, smem + kOffH2, s_net + kNetImageB3, 512u, 32, 16, BF16);
+      mma_commit(bar);
+    }
     wait_layer(mc);
     uint32_t mask3 = 0u;
     {
@@ -241,13 +262,16 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
       }
 #pragma unroll
       for (int g = 0; g < 2; ++g) st_group(smem + kOffH3, g, t, pk[4 * g], pk[4 * g + 1], pk[4 * g + 2], pk[4 * g + 3]);
-      tmem_st8(tmem + lane + kColA4, pk);
     }
-    tmem_st_wait();
+    fence_async_smem();
     tc_fence_before();
     __syncthreads();
     // ---- layer 4 (+ b4 in FP32) -> H4; layer 5 in FP32; deltas D5, D4, D3
-    if (t == 0) issue_layer_t<BF16>(mc, kColA4, 16, kNetImageB4, 16, kColD4);
+    if (t == 0) {
+      tc_fence_after();
+      mma_layer(tmem + kColD4, smem + kOffH3, s_net + kNetImageB4, 256u, 16, 16, BF16);
+      mma_commit(bar);
+    }
     wait_layer(mc);
     float h4[8];
     uint32_t mask4 = 0u;
@@ -304,10 +328,8 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     // ---- D2 = (D3 W3) * relu'(Z2); gradients of layers 5, 4, 3
     if (t == 0) {
       tc_fence_after();
-      mma_delta(tmem + 0u, smem + kOffD3, s_bwd + kBwdBW3, 256u, 16, 32, BF16);
-      mma_grad(tmem + kAcc5, smem + kOffH4, smem + kOffD5, kUnits, kSamples, 16, BF16, !first);
-      mma_grad(tmem + kAcc4, smem + kOffH3, smem + kOffD4, kUnits, kSamples, 16, BF16, !first);
-      mma_grad(tmem + kAcc3, smem + kOffH2, smem + kOffD3, kUnits, kSamples, 16, BF16, !first);
+      mma_layer(tmem + 0u, smem + kOffD3, s_bwd + kBwdBW3, 256u, 16, 32, BF16);
+      mma_grad(tmem + kAcc3, smem + kOffH2, smem + kOffD3, kUnits, kSamples, 32, BF16, !first);
       mma_commit(bar);
     }
     wait_layer(mc);
@@ -333,7 +355,7 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     // ---- D1 = (D2 W2) * relu'(Z1); gradient of layer 2
     if (t == 0) {
       tc_fence_after();
-      mma_delta(tmem + 0u, smem + kOffD2, s_bwd + kBwdBW2, 512u, 32, 64, BF16);
+      mma_layer(tmem + 0u, smem + kOffD2, s_bwd + kBwdBW2, 512u, 32, 64, BF16);
       mma_grad(tmem + kAcc2, smem + kOffH1, smem + kOffD2, kUnits, kSamples, 32, BF16, !first);
       mma_commit(bar);
     }
@@ -372,6 +394,11 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     if (__syncthreads_or(*fail)) break;
   }
   if (!first) wait_layer(mc);
+  if (*fail) {
+    // a copy may still be in flight: wait for it (bounded) before leaving
+    float x[6];
+    rows.get(blockIdx.x, x);
+  }
   const bool failed = __syncthreads_or(*fail) != 0;
   // ---- this CTA's partial gradients, from the accumulator rows
   float* part = partial + (size_t)blockIdx.x * kNetParams;
@@ -405,19 +432,17 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
       if (t < 32) part[2528 + o * 32 + t] = __uint_as_float(r[o]);
       if (t == 32) part[3040 + o] = __uint_as_float(r[o]);
     }
-    tmem_ld16(tmem + lane + kAcc4, r);  // row i of dW4^T (i < 16), db4 in row 16
+    tmem_ld16(tmem + lane + kAcc3 + 16u, r);  // columns of D4 (8), then D5
     tmem_ld_wait();
 #pragma unroll
-    for (int o = 0; o < 8; ++o) {
-      if (t < 16) part[3056 + o * 16 + t] = __uint_as_float(r[o]);
-      if (t == 16) part[3184 + o] = __uint_as_float(r[o]);
+    for (int o = 0; o < 8; ++o) {  // row i of dW4^T, db4 in the row after
+      if (t >= kRowH3 && t < kRowH3 + 16) part[3056 + o * 16 + t - kRowH3] = __uint_as_float(r[o]);
+      if (t == kRowH3 + 16) part[3184 + o] = __uint_as_float(r[o]);
     }
-    tmem_ld16(tmem + lane + kAcc5, r);  // row i of dW5^T (i < 8), db5 in row 8
-    tmem_ld_wait();
 #pragma unroll
-    for (int o = 0; o < 4; ++o) {
-      if (t < 8) part[3192 + o * 8 + t] = __uint_as_float(r[o]);
-      if (t == 8) part[3224 + o] = __uint_as_float(r[o]);
+    for (int o = 0; o < 4; ++o) {  // row i of dW5^T, db5 in the row after
+      if (t >= kRowH4 && t < kRowH4 + 8) part[3192 + o * 8 + t - kRowH4] = __uint_as_float(r[8 + o]);
+      if (t == kRowH4 + 8) part[3224 + o] = __uint_as_float(r[8 + o]);
     }
   }
   // block loss (fixed-order tree)

@@ -271,6 +271,60 @@ __device__ __forceinline__ bool mlp_tc_narrow(MlpCtx& c, float z[4]) {
   return __syncthreads_or(*c.fail) == 0;
 }
 
+// (float)x, round to nearest: on the integer pipe for values in the normal FP32
+// range and 0 (a conversion takes the FP64 pipe, 64 clocks of an SM quarter).
+__device__ __forceinline__ float to_f32(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e - 897u < 253u) {
+    const unsigned long long r = ((unsigned long long)(unsigned)hi << 32 | (unsigned)lo) + 0x0fffffffull + ((lo >> 29) & 1);
+    const unsigned f = __funnelshift_l((unsigned)r, (unsigned)(r >> 32), 3);
+    return __uint_as_float(((f ^ 0x40000000u) & 0x7fffffffu) | ((unsigned)hi & 0x80000000u));
+  }
+  if ((((unsigned)hi << 1) | (unsigned)lo) == 0u) return __uint_as_float((unsigned)hi);
+  return (float)x;
+}
+
+// The stencils of a kernel's 128-row tiles, fetched a tile ahead: a tile's rows
+// (48 bytes each) are consecutive, so one bulk copy brings them while the tile
+// before runs its chain of layers, which a load from DRAM would lengthen by a
+// quarter.  Where X is not 16-byte aligned the rows are loaded when needed.
+struct TileRows {
+  const double* X;
+  long long n;
+  double* buf;  // 128 x 6, 16-byte aligned shared memory
+  uint64_t* bar;
+  uint32_t phase;
+  bool bulk;
+  // thread 0, once every thread has read the rows before
+  __device__ __forceinline__ void fetch(long long tile) {
+    const long long rows = n - tile * 128 < 128 ? n - tile * 128 : 128;
+    if (!bulk || rows <= 0) return;
+    mbar_arrive_expect_tx(bar, (uint32_t)rows * 48u);
+    bulk_load(buf, X + tile * 768, (uint32_t)rows * 48u, bar);
+  }
+  // this thread's row of `tile` in FP32 (0 past the end); false on a timeout
+  __device__ __forceinline__ bool get(long long tile, float (&x)[6]) {
+    const long long r = tile * 128 + threadIdx.x;
+    bool ok = true;
+    if (bulk) {
+      ok = mbar_wait(bar, phase);
+      phase ^= 1u;
+      const double2* b = reinterpret_cast<const double2*>(buf) + 3 * threadIdx.x;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const double2 v = b[j];
+        x[2 * j] = r < n ? to_f32(v.x) : 0.0f;
+        x[2 * j + 1] = r < n ? to_f32(v.y) : 0.0f;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 6; ++j) x[j] = r < n ? to_f32(X[r * 6 + j]) : 0.0f;
+    }
+    return ok;
+  }
+};
+
 // Copy the classifier image (16-byte chunks) into shared memory.
 __device__ __forceinline__ void load_net_image(uint8_t* dst, const uint8_t* __restrict__ src) {
   const uint4* s = reinterpret_cast<const uint4*>(src);
