@@ -11,20 +11,24 @@
 //
 // Design (GB300): the binary64 pipe issues two lanes per clock and SM, 1/61 of
 // the FP32 pipe's rate, so the classifier (3104 multiply-adds per stencil, 16
-// stencils per cell and RHS) is evaluated in FP32 with a certified bound and in
-// binary64 only where the bound does not settle a logit's sign
-// (mlp_filter.cuh).  What stays on the FP64 pipe is the reconstruction itself,
+// stencils per cell and RHS) is evaluated in FP32 and split 16-bit matrix
+// products with a certified bound and in binary64 only where the bound does not
+// settle a logit's sign (mlp_filter.cuh).  What stays on the FP64 pipe is the reconstruction itself,
 // ~1150 operations per cell, and each is done once: a thread takes a face
 // with all its characteristic fields, so the Roe state is formed once per face.
 // Persistent CTAs take tiles of cells: the tile plus a 3-cell halo (periodic
 // wrap or zero-gradient copy done in the load) and the per-cell quantities are
 // staged in shared memory, the faces' fluxes written back there and
 // differenced, with no scratch in global memory.  Comparisons (ReLU, max, |x|)
-// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 13.6 ms,
+// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 11.7 ms,
 // against 437 ms with every classifier row in binary64 and four lanes per
 // face; the FP64 operations alone would take 7.9 ms of a full FP64 pipe.
+#include <cuda_fp16.h>
+
 #include <cmath>
+#include <cstring>
 #include <utility>
+#include <vector>
 
 #include "fp64_ops.cuh"
 #include "internal.h"
@@ -58,9 +62,9 @@ struct Tile {
   static constexpr int P_F = P_c + 3;
   static constexpr int NPLANES = P_F + NDIM * (NV - 1);
   static constexpr int kPark = 12;  // per thread: the "+" stencil, the mirrored "-" stencil
-  static constexpr int kScratch = 128;  // per warp (binary64 classifier)
+  static constexpr int kScratch = 72;   // per warp (binary64 classifier)
   // doubles: planes, face fluxes, parked stencils, warp scratch, and for
-  // SPLIT the faces' field fluxes and Roe states; dt; then the FP32 table
+  // SPLIT the faces' field fluxes and Roe states; dt; then the filter's table
   static constexpr int O_F = NPLANES * NC;
   static constexpr int O_P = O_F + NV * (NXF + NYF);
   static constexpr int O_W = O_P + kPark * NT;
@@ -416,7 +420,7 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
           // rather than kept in registers across it
           asm volatile("" ::: "memory");
           unsigned res[2];
-          filt::filter_rows<2>(T, x, res);
+          filt::filter_rows(T, x, res);
           eta_side[0] = res[0] & 15u;
           eta_side[1] = res[1] & 15u;
           filt::settle_rows(Wt, park0 + warp * 32, NT, ws, valid && !(ok0 && (res[0] & 16u)), eta_side[0]);
@@ -639,11 +643,50 @@ cudaError_t dependent_launch(void (*kern)(P...), unsigned grid, unsigned block, 
 
 }  // namespace
 
+namespace {
+
+// Round x to binary16 (nearest even); returns its value.  The table takes
+// 60 us of a solver's creation so, 115 with the library's host conversions.
+float round16(float x, uint16_t& bits) {
+  uint32_t b;
+  std::memcpy(&b, &x, 4);
+  const uint32_t sign = b >> 16 & 0x8000u, mag = b & 0x7fffffffu;
+  if (mag < 0x38800000u) {  // below 2^-14: a multiple of 2^-24
+    const float n = std::nearbyint(std::fabs(x) * 16777216.0f);
+    bits = (uint16_t)(sign | (uint32_t)n);
+    return std::copysign(n * (1.0f / 16777216.0f), x);
+  }
+  if (mag < 0x477fe000u) {  // up to 65504
+    const uint32_t r = (mag + 0xfffu + (mag >> 13 & 1u)) & ~0x1fffu;
+    bits = (uint16_t)(sign | ((r >> 13) - (112u << 10)));
+    b = (b & 0x80000000u) | r;
+    std::memcpy(&x, &b, 4);
+    return x;
+  }
+  const __half h = __float2half(x);
+  std::memcpy(&bits, &h, 2);
+  return __half2float(h);
+}
+// v = hi + lo + error in binary16 terms of v's FP32 rounding
+struct Split {
+  uint16_t hi, lo;
+  double error;
+};
+Split split_terms(double v) {
+  Split s;
+  const float f = (float)v, h = round16(f, s.hi), l = round16(f - h, s.lo);
+  s.error = std::fabs(v - (double)h - (double)l);
+  return s;
+}
+
+}  // namespace
+
 // Coefficients of the filter's bound (mlp_filter.cuh).
-static void build_filter_kappa(const NetF64& net, FilterKappa& out) {
+// `split`: the terms of the weights of layers 2 to 5 (layer 5 scaled), filled in.
+static void build_filter_kappa(const NetF64& net, FilterKappa& out, Split* split) {
   constexpr int W[6] = {6, 64, 32, 16, 8, 4};
   constexpr int off[5] = {0, 448, 2528, 3056, 3192};
-  const double u = 1.0 / 16777216.0, tiny = std::ldexp(1.0, -125);
+  const double u = 1.0 / 16777216.0, tiny = std::ldexp(1.0, -125), gap = std::ldexp(1.0, -25);
   auto aw = [&](int l, int o, int i) { return std::fmax(std::fabs(net.p[off[l] + o * W[l] + i]), tiny); };
   auto ab = [&](int l, int o) { return std::fmax(std::fabs(net.p[off[l] + W[l] * W[l + 1] + o]), tiny); };
   // static bound per logit over |x| <= 1: the logits' relative scales
@@ -678,38 +721,56 @@ static void build_filter_kappa(const NetF64& net, FilterKappa& out) {
   float* dst[5] = {out.in, out.h1, out.h2, out.h3, out.h4};
   for (int l = 4; l >= 0; --l) {
     const int n = W[l], m = W[l + 1];
-    for (int i = 0; i < n; ++i) {
-      double worst = 0.0;
-      for (int k = 0; k < 4; ++k) {
-        double g = 0.0;
-        for (int o = 0; o < m; ++o) g += G[k][o] * aw(l, o, i);
-        Gn[k][i] = g;
-        // the i-th FMA of the chain and those after it, and the weight's rounding
-        double c = (n - i + 1) * u * g;
-        if (l == 0) {
-          c += 8.0 * u * g;
-          k0[k] += g * tiny;
-        }
-        worst = std::fmax(worst, c);
-        if (!(c == c)) worst = c;  // a NaN weight: nothing is certified
+    const int T = 3 * ((n + 15) / 16);  // matrix instructions per output (layers 2-5)
+    double A[2048], D[2048] = {};  // |w|, its split error
+    for (int o = 0; o < m; ++o)
+      for (int i = 0; i < n; ++i) {
+        A[o * n + i] = aw(l, o, i);
+        if (l == 0) continue;
+        const Split s = split[off[l] + o * n + i] = split_terms(net.p[off[l] + o * n + i] * (l == 4 ? out.scale[o] : 1.0));
+        D[o * n + i] = s.error;
       }
-      dst[l][i] = up(worst);
+    double worst[64] = {};
+    for (int k = 0; k < 4; ++k) {
+      double dw[64] = {};
+      for (int i = 0; i < n; ++i) Gn[k][i] = 0.0;
+      for (int o = 0; o < m; ++o) {
+        const double g = G[k][o], gs = l == 4 ? g / out.scale[k] : g;  // G holds the scale already
+        for (int i = 0; i < n; ++i) {
+          Gn[k][i] += g * A[o * n + i];
+          dw[i] += gs * D[o * n + i];
+        }
+      }
+      for (int i = 0; i < n; ++i) {
+        const double g = Gn[k][i];
+        double c;
+        if (l == 0) {  // the i-th FMA of the chain and those after it, the weight's and the input's rounding
+          c = (n - i + 1 + 8) * u * g;
+          k0[k] += g * tiny;
+        } else {  // the instructions from its block on, its split and the dropped product, the weight's split
+          c = (4 * (T - 3 * (i / 16)) + 2) * u * g + dw[i];
+          k0[k] += g * gap;
+        }
+        worst[i] = std::fmax(worst[i], c == c ? c : INFINITY);  // a NaN weight: nothing is certified
+      }
     }
+    for (int i = 0; i < n; ++i) dst[l][i] = up(worst[i]);
     for (int k = 0; k < 4; ++k)
-      for (int o = 0; o < m; ++o) k0[k] += (n + 1) * u * G[k][o] * ab(l, o);
+      for (int o = 0; o < m; ++o) k0[k] += (l == 0 ? n + 1 : 4 * T + 1) * u * G[k][o] * ab(l, o);
     for (int k = 0; k < 4; ++k)
       for (int i = 0; i < n; ++i) G[k][i] = Gn[k][i];
   }
   double worst = 0.0;
-  for (int k = 0; k < 4; ++k) worst = k0[k] == k0[k] ? std::fmax(worst, k0[k]) : k0[k];
+  for (int k = 0; k < 4; ++k) worst = std::fmax(worst, k0[k] == k0[k] ? k0[k] : INFINITY);
   out.k0 = up(worst);
 }
 
 void build_net_blob(const NetF64& net, void* blob) {
   constexpr int W[6] = {6, 64, 32, 16, 8, 4};
-  constexpr int kW[5] = {kFiltW1, kFiltW2, kFiltW3, kFiltW4, kFiltW5}, kB[5] = {0, kFiltB2, kFiltB3, kFiltB4, kFiltB5};
+  constexpr int kW[5] = {0, kFiltW2, kFiltW3, kFiltW4, kFiltW5}, kB[5] = {0, kFiltB2, kFiltB3, kFiltB4, kFiltB5};
   FilterKappa k;
-  build_filter_kappa(net, k);
+  std::vector<Split> split(kNetParams);
+  build_filter_kappa(net, k, split.data());
   double* Wt = static_cast<double*>(blob);
   float* T = reinterpret_cast<float*>(Wt + kNetParams);
   for (int i = 0; i < kFiltFloats; ++i) T[i] = 0.0f;
@@ -721,7 +782,17 @@ void build_net_blob(const NetF64& net, void* blob) {
       for (int i = 0; i < nin; ++i) {
         const double w = net.p[p + o * nin + i];
         Wt[p + i * nout + o] = w;
-        T[l == 0 ? kFiltW1 + 8 * o + i : kW[l] + i * nout + o] = (float)(w * scale);
+        if (l == 0) {
+          T[kFiltW1 + 8 * o + i] = (float)w;
+          continue;
+        }
+        // input i of its block: pair (i % 8) / 2 of lane 4 (o % 8) + pair, word
+        // i / 8 of hi and of lo
+        const int tiles = (nout + 7) / 8, in = i % 16;
+        uint16_t* at = reinterpret_cast<uint16_t*>(T + kW[l] + 128 * ((i / 16) * tiles + o / 8) +
+                                                   4 * (4 * (o % 8) + in % 8 / 2) + in / 8) + in % 2;
+        at[0] = split[p + o * nin + i].hi;
+        at[4] = split[p + o * nin + i].lo;
       }
       const double b = net.p[p + nin * nout + o];
       Wt[p + nin * nout + o] = b;
@@ -763,29 +834,29 @@ cudaError_t launch_rhs_fp64(int ndim, RhsArgs& a, cudaStream_t s) {
   // Tiles whose (TX + 1) TY x faces and (TY + 1) TX y faces fill whole runs of
   // 32 (the FP64 pipe takes 64 clocks per warp instruction and SM quarter
   // however few lanes are active): 2.13 face slots per cell for 15 x 16, 2.29
-  // for 7 x 16 and 7 x 8.  The smaller the grid, the smaller the tile, so that
-  // every SM has warps; the smallest grids give a warp a single field.
-  // Measured in us per RHS, periodic quadrants:
-  //             24x16   64x64  130x97 200x136 300x300   512^2   1024^2   2048^2
-  //   15 x 16    242     179     187     187     420     974     3533    13621
-  //   7 x 16     144      98     104     139     362     907     3535    13920
-  //   7 x 8       95      56      77     145     364     919     3609    14298
-  //   7 x 3 SPLIT 70      48     110     203     561    1454     5669    22704
-  // (16 x 16 with 192 threads: 2048^2 in 14109.)
-  // 1D, n =                    400    4096   16384  131072
-  //   31 SPLIT                22.7    20.8    37.5   195
-  //   127                     43.2    41.4    43.4   181
+  // for 7 x 16.  The smaller the grid, the smaller the tile, so that every SM
+  // has warps; the smallest grids give a warp a single field.  Measured in us
+  // per RHS, periodic quadrants (threads x CTAs per SM; * taken):
+  //                        24x16 64x64 100x100 200x136 300x300 400x400 512^2 700^2 1024^2 2048^2
+  //   15 x 16       256x2   209   135    140     142     350     551    822* 1467*  3034*  11696*
+  //   15 x 16       192x2   236   154            161                    848         3107   12058
+  //   7 x 16        256x2   110    70     74*    114*    330*    547*   842  1606   3229   12769
+  //   7 x 8         128x4    99    52     77     118     324     541    831  1569   3201   12611
+  //   7 x 3 SPLIT   256x2    68*   44*    84     200     573    1012   1555  3030   6166   24579
+  // 1D, n =                       400   4096  16384  65536  131072  1048576
+  //   31 SPLIT      96x4           18*    17*    33*   111     197     1411
+  //   127           128x4          38     36     39     85*    163*    1030*
+  //   127           128x3          36     35     37     97     163     1077
   const auto tiles = [&](int tx, int ty) {
     return (long long)((a.nx + tx - 1) / tx) * ((a.ny + ty - 1) / ty);
   };
   if (ndim == 1) {
     if (tiles(31, 1) <= 152 * 4) return launch_tiles<Tile<1, 31, 1, 96, 4, true>>(a, s);
-    return launch_tiles<Tile<1, 127, 1, 128, 3, false>>(a, s);
+    return launch_tiles<Tile<1, 127, 1, 128, 4, false>>(a, s);
   }
   if (tiles(7, 3) <= 152 * 2) return launch_tiles<Tile<2, 7, 3, 256, 2, true>>(a, s);
-  if (tiles(7, 8) <= 152 * 3) return launch_tiles<Tile<2, 7, 8, 128, 3, false>>(a, s);
-  if (tiles(15, 16) < 152 * 2 * 12) return launch_tiles<Tile<2, 7, 16, 128, 3, false>>(a, s);
-  return launch_tiles<Tile<2, 15, 16, 192, 2, false>>(a, s);
+  if (tiles(15, 16) < 152 * 2 * 3) return launch_tiles<Tile<2, 7, 16, 256, 2, false>>(a, s);
+  return launch_tiles<Tile<2, 15, 16, 256, 2, false>>(a, s);
 }
 
 cudaError_t launch_classify_fp64(const ClassifyParamsF64& p, bool narrow, cudaStream_t s) {

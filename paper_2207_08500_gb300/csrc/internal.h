@@ -29,15 +29,17 @@ enum MaskMode { kMaskMLP = 0, kMaskSmooth = 1, kMaskRough = 2, kMaskTeno = 3, kM
 constexpr int kTenoTable = 79;
 void teno_tables(double out[kTenoTable]);
 
-// FP32 table of the certified classifier filter (mlp_filter.cuh), in floats:
-// k0 and the six input coefficients, then per unit of layer 1 its six weights,
-// bias and kappa, and for the layers after it W transposed ([in][out]), bias
-// and kappa of the outputs (none for layer 5).
+// Table of the certified classifier filter (mlp_filter.cuh), in floats: k0 and
+// the six input coefficients; per unit of layer 1 its six weights, bias and
+// kappa; for the layers after it the weights as binary16 pairs in the matrix
+// instruction's order (per block of 16 inputs, tile of 8 outputs and lane: two
+// words of hi, two of lo), FP32 biases, and kappa of the outputs (none for layer
+// 5, whose four outputs are padded to eight).
 constexpr int kFiltIn = 0, kFiltW1 = 8;
-constexpr int kFiltW2 = kFiltW1 + 64 * 8, kFiltB2 = kFiltW2 + 64 * 32, kFiltK2 = kFiltB2 + 32;
-constexpr int kFiltW3 = kFiltK2 + 32, kFiltB3 = kFiltW3 + 32 * 16, kFiltK3 = kFiltB3 + 16;
-constexpr int kFiltW4 = kFiltK3 + 16, kFiltB4 = kFiltW4 + 16 * 8, kFiltK4 = kFiltB4 + 8;
-constexpr int kFiltW5 = kFiltK4 + 8, kFiltB5 = kFiltW5 + 8 * 4, kFiltFloats = kFiltB5 + 4;
+constexpr int kFiltW2 = kFiltW1 + 64 * 8, kFiltW3 = kFiltW2 + 4 * 4 * 128, kFiltW4 = kFiltW3 + 2 * 2 * 128;
+constexpr int kFiltW5 = kFiltW4 + 128, kFiltB2 = kFiltW5 + 128, kFiltB3 = kFiltB2 + 32, kFiltB4 = kFiltB3 + 16;
+constexpr int kFiltB5 = kFiltB4 + 8, kFiltK2 = kFiltB5 + 8, kFiltK3 = kFiltK2 + 32, kFiltK4 = kFiltK3 + 16;
+constexpr int kFiltFloats = kFiltK4 + 8;
 static_assert(kFiltFloats % 4 == 0, "copied in 16-byte chunks");
 struct FilterKappa {
   double scale[4];  // logit k's row of W5 and b5 is multiplied by this

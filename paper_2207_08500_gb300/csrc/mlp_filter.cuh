@@ -1,23 +1,41 @@
-// Certified FP32 evaluation of the 6-64-32-16-8-4 classifier (Sec. 3.1) for
-// the FP64 paths.  Those paths need the classifier for four bits only -- the
-// signs of the logits that the binary64 network yields in the canonical order
-// -- and GB300's FP32 pipe runs at 61 times its FP64 pipe's rate.  So the
-// network is evaluated in FP32 together with a bound on the distance of its
-// logits from the binary64 ones; a logit beyond the bound has the binary64
-// logit's sign, and every other row is evaluated again in binary64 in the
-// canonical order (mlp64_warp / mlp64_rows below).  The bits are the binary64
-// network's, always.
+// Certified evaluation of the 6-64-32-16-8-4 classifier (Sec. 3.1) for the FP64
+// paths.  Those paths need the classifier for four bits only -- the signs of the
+// logits that the binary64 network yields in the canonical order -- and GB300's
+// FP32 and tensor pipes run at 61 and several hundred times its FP64 pipe's
+// rate.  So the network is evaluated in FP32 (layer 1) and in split 16-bit
+// products with FP32 accumulation (layers 2 to 5), together with a bound on the
+// distance of its logits from the binary64 ones; a logit beyond the bound has
+// the binary64 logit's sign, and every other row is evaluated again in binary64
+// in the canonical order (mlp64_warp / mlp64_rows below).  The bits are the
+// binary64 network's, always.
 //
-// The bound (forward error analysis of a fixed-order FMA chain, Higham,
-// "Accuracy and Stability of Numerical Algorithms", ch. 3).  A unit of n
-// inputs is its bias followed by n FMAs, on weights rounded to FP32, so with
-// u = 2^-24 its computed pre-activation differs from the exact one of the
-// same computed inputs h by at most
-//   sum_j (n - j + 2) u |w_j| |h_j| + (n + 1) u |b|,    j = 1..n,
-// up to O(u^2).  ReLU does not enlarge a difference, and layers l+1..5 carry
-// one of layer l to logit k multiplied by at most G_l = |W5| ... |W_{l+1}|.
-// Summed over the layers the bound is linear in the computed hidden values
-// (all >= 0) and inputs:
+// Each FP32 value v of layers 2 to 5 (weights and inputs) is split into two
+// binary16 terms, v = hi + lo + d with |d| <= u |v| + 2^-25, u = 2^-24, and a
+// product is hi hi' + lo hi' + hi lo': warp-level matrix instructions (16 rows x
+// 8 outputs x 16 inputs, three per block of 16 inputs), whose operands and
+// results stay in registers.  They fit this kernel: a warp's 64 rows (32 faces,
+// two sides) need no barrier, no tensor memory and no wait on other warps, and
+// at 2 clocks per instruction and SM they take a quarter of the FP64 time beside
+// which they run.  2048^2 RHS: 11.7 ms, against 13.8 ms with every layer in FP32
+// on the CUDA cores (weights by broadcast loads, which bound it).
+//
+// The bound (forward error analysis, Higham, "Accuracy and Stability of
+// Numerical Algorithms", ch. 3).  Layer 1: a bias and six FMAs on weights
+// rounded to FP32 differ from the exact value of the same inputs x by at most
+//   sum_j (6 - j + 2) u |w_j| |x_j| + 7 u |b|,   j = 1..6.
+// A layer above: T matrix instructions in turn on one accumulator that starts
+// at the bias; each is taken to add at most 4 u times the magnitudes it sums
+// (the products and the accumulator; products of binary16 values are exact, the
+// sums are kept to at least 24 bits and truncated: Fasi, Higham, Mikaitis and
+// Pranesh, "Numerical behavior of NVIDIA tensor cores", PeerJ CS 7:e330; 1.7 u
+// is the largest seen on this GPU).  An input j of block k is in T - 3 k of
+// them, so with dw the weight's split error and 2 u for the input's and the
+// dropped lo lo' the unit is off by at most
+//   sum_j ((4 (T - 3 k_j) + 2) u |w_j| + dw_j) |h_j| + 2^-25 sum_j |w_j| + (4 T + 1) u |b|
+// up to O(u^2).  ReLU does not enlarge a difference, and layers l+1..5 carry one
+// of layer l to logit k multiplied by at most G_l = |W5| ... |W_{l+1}|.  Summed
+// over the layers the bound is linear in the computed hidden values (all >= 0)
+// and inputs:
 //   |error of logit k| <= k0 + sum_j kin_j |x_j| + sum_l sum_i kappa_l,i h_l,i,
 // one more FMA per hidden unit.  The coefficients (build_filter_kappa, on the
 // host in binary64) take the maximum over the four logits after dividing
@@ -26,10 +44,13 @@
 // input's conversion (8 u relative: two truncations to 24 bits, a reciprocal
 // to 1 ulp and a product), underflow (every |w|, |b| counted as at least
 // 2^-125) and a factor 1.01 for the O(u^2) terms, the binary64 network's own
-// rounding (2^-29 of the FP32 bound) and the rounding of the bound itself.
+// rounding (2^-29 of the bound) and the rounding of the bound itself.
 // A row whose inputs leave [0, 2^100], or any of whose logits or whose bound
-// is not finite, is never certified.
+// is not finite (a value outside the binary16 range makes it so), is never
+// certified.
 #pragma once
+
+#include <cuda_fp16.h>
 
 #include "fp64_ops.cuh"
 #include "internal.h"
@@ -70,158 +91,183 @@ __device__ __forceinline__ bool filter_input(const double (&s)[6], float (&x)[6]
   return top < kTopLimit;
 }
 
-// The network of R rows per thread against the table T in shared memory (the
-// kFilt* layout; every lane reads the same address).  Outputs packed in pairs
-// (fma.rn.f32x2 rounds each half like a scalar FMA).  Returns per row the eta
-// bits in bits 0-3 and, in bit 4, whether they are certified.
-template <int R>
-__device__ __forceinline__ void filter_rows(const float* __restrict__ T, const float (&x)[R][6],
-                                            unsigned (&res)[R]) {
-  float err[R];
-  {
-    const float4 e0 = *reinterpret_cast<const float4*>(T + kFiltIn);
-    const float4 e1 = *reinterpret_cast<const float4*>(T + kFiltIn + 4);
+// d += a b: 16 rows x 16 inputs times 16 inputs x 8 outputs, binary16 operands,
+// FP32 accumulators.  Lane 4 g + q holds of d: rows g (first two) and g + 8,
+// outputs 2 q, 2 q + 1; of a: the pairs of inputs 2 q, 2 q + 1 of rows g and g +
+// 8, then the pairs 2 q + 8, 2 q + 9; of b: the same pairs of output g.
+__device__ __forceinline__ void mma16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// ReLU that keeps NaN: a value outside the binary16 range splits into infinities
+// of both signs, whose products are NaN, and reaches the logits as NaN.
+__device__ __forceinline__ float relu_nan(float x) {
+  float y;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(y) : "f"(x));
+  return y;
+}
+// Split a pair of FP32 values into packed binary16 terms.
+__device__ __forceinline__ void split16(float x, float y, uint32_t& hi, uint32_t& lo) {
+  const __half2 h = __floats2half2_rn(x, y);
+  const float2 f = __half22float2(h);
+  const __half2 l = __floats2half2_rn(x - f.x, y - f.y);
+  hi = *reinterpret_cast<const uint32_t*>(&h);
+  lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+// One block of 16 inputs (pairs p: rows g, g + 8 of inputs 2q.., then of 2q + 8..)
+// into NT tiles of 8 outputs of both row tiles: T points at the block's weights,
+// per tile and lane hi b0, b1, lo b0, b1.
+template <int NT>
+__device__ __forceinline__ void block16(float (&acc)[2][NT][4], const uint32_t (&hi)[2][4], const uint32_t (&lo)[2][4],
+                                        const float* T, int lane) {
+  uint4 b[NT];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      float e = e0.x;  // k0, then the six inputs
-      e = fmaf(e0.y, fabsf(x[r][0]), e);
-      e = fmaf(e0.z, fabsf(x[r][1]), e);
-      e = fmaf(e0.w, fabsf(x[r][2]), e);
-      e = fmaf(e1.x, fabsf(x[r][3]), e);
-      e = fmaf(e1.y, fabsf(x[r][4]), e);
-      err[r] = fmaf(e1.z, fabsf(x[r][5]), e);
+  for (int nt = 0; nt < NT; ++nt) b[nt] = reinterpret_cast<const uint4*>(T)[32 * nt + lane];
+  // term by term: the instructions on one accumulator are 2 NT apart
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) mma16(acc[mt][nt], hi[mt], b[nt].x, b[nt].y);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) mma16(acc[mt][nt], lo[mt], b[nt].x, b[nt].y);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) mma16(acc[mt][nt], hi[mt], b[nt].z, b[nt].w);
+}
+// Accumulators start at the biases of their outputs.
+template <int NT>
+__device__ __forceinline__ void start16(float (&acc)[2][NT][4], const float* B, int q) {
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt) {
+    const float2 b = reinterpret_cast<const float2*>(B)[4 * nt + q];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) {
+      acc[mt][nt][0] = acc[mt][nt][2] = b.x;
+      acc[mt][nt][1] = acc[mt][nt][3] = b.y;
     }
   }
-  float2 a[R][16];
+}
+// ReLU of one tile of outputs (8 nt ..) of a layer, its share of the bound, and
+// its terms as half (`h` = 0, 1) of the next layer's block of 16 inputs.
+template <int NT>
+__device__ __forceinline__ void next16(const float (&acc)[2][NT][4], int nt, int h, const float* K, int q,
+                                       float (&err)[4], uint32_t (&hi)[2][4], uint32_t (&lo)[2][4]) {
+  const float2 k = reinterpret_cast<const float2*>(K)[4 * nt + q];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const float2 b = reinterpret_cast<const float2*>(T + kFiltB2)[q];
+  for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int r = 0; r < R; ++r) a[r][q] = b;
-  }
-  // layers 1 and 2 fused: hidden unit i of layer 1 goes into the 32 sums of
-  // layer 2 (each sum's order: bias, then inputs in ascending order).  The
-  // weights of the first 16 sums and of layer 1 are loaded one unit ahead, the
-  // others while the unit's layer 1 runs: a pass of a warp alone on its SM
-  // quarter takes 7.4-8.5 k clocks instead of 10.7 k.
-  float4 w0 = *reinterpret_cast<const float4*>(T + kFiltW1);
-  float4 w1 = *reinterpret_cast<const float4*>(T + kFiltW1 + 4);  // w4, w5, bias, kappa
-  float4 wa[4], wb[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) wa[q] = *reinterpret_cast<const float4*>(T + kFiltW2 + 4 * q);
+    for (int r = 0; r < 2; ++r) {
+      const float x = relu_nan(acc[mt][nt][2 * r]), y = relu_nan(acc[mt][nt][2 * r + 1]);
+      err[2 * mt + r] = fmaf(k.x, x, err[2 * mt + r]);
+      err[2 * mt + r] = fmaf(k.y, y, err[2 * mt + r]);
+      split16(x, y, hi[mt][2 * h + r], lo[mt][2 * h + r]);
+    }
+}
+
+// The network for a warp's 64 rows: lane l's rows x[0], x[1] (the two sides of
+// its face), against the table T in shared memory (the kFilt* layout).  Returns
+// per row the eta bits in bits 0-3 and, in bit 4, whether they are certified.
+// All 32 lanes call it.
+__device__ __forceinline__ void filter_rows(const float* __restrict__ T, const float (&x)[2][6], unsigned (&res)[2]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
 #pragma unroll 1
-  for (int i = 0; i < 64; ++i) {
+  for (int side = 0; side < 2; ++side) {
+    // inputs of rows g, g + 8, g + 16, g + 24 (row = lane of origin)
+    float xr[4][6], err[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) wb[q] = *reinterpret_cast<const float4*>(T + kFiltW2 + 32 * i + 16 + 4 * q);
-    float2 h[R];
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      float v = fmaf(w0.x, x[r][0], w1.z);
-      v = fmaf(w0.y, x[r][1], v);
-      v = fmaf(w0.z, x[r][2], v);
-      v = fmaf(w0.w, x[r][3], v);
-      v = fmaf(w1.x, x[r][4], v);
-      v = fmaf(w1.y, x[r][5], v);
-      v = fmaxf(v, 0.0f);
-      err[r] = fmaf(w1.w, v, err[r]);
-      h[r] = make_float2(v, v);
-    }
-    const int nx = min(i + 1, 63);
-    w0 = *reinterpret_cast<const float4*>(T + kFiltW1 + 8 * nx);
-    w1 = *reinterpret_cast<const float4*>(T + kFiltW1 + 8 * nx + 4);
+      for (int j = 0; j < 6; ++j) xr[r][j] = __shfl_sync(0xffffffffu, side ? x[1][j] : x[0][j], g + 8 * r);
+    {
+      const float4 e0 = *reinterpret_cast<const float4*>(T + kFiltIn);  // k0, then the six inputs
+      const float4 e1 = *reinterpret_cast<const float4*>(T + kFiltIn + 4);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        a[r][2 * q] = __ffma2_rn(make_float2(wa[q].x, wa[q].y), h[r], a[r][2 * q]);
-        a[r][2 * q + 1] = __ffma2_rn(make_float2(wa[q].z, wa[q].w), h[r], a[r][2 * q + 1]);
-      }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) wa[q] = *reinterpret_cast<const float4*>(T + kFiltW2 + 32 * nx + 4 * q);
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        a[r][8 + 2 * q] = __ffma2_rn(make_float2(wb[q].x, wb[q].y), h[r], a[r][8 + 2 * q]);
-        a[r][9 + 2 * q] = __ffma2_rn(make_float2(wb[q].z, wb[q].w), h[r], a[r][9 + 2 * q]);
-      }
-  }
-  float2 c[R][8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const float2 b = reinterpret_cast<const float2*>(T + kFiltB3)[q];
-#pragma unroll
-    for (int r = 0; r < R; ++r) c[r][q] = b;
-  }
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    float2 h[R];
-    const float kap = T[kFiltK2 + i];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const float v = fmaxf(i & 1 ? a[r][i / 2].y : a[r][i / 2].x, 0.0f);
-      err[r] = fmaf(kap, v, err[r]);
-      h[r] = make_float2(v, v);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 w = *reinterpret_cast<const float4*>(T + kFiltW3 + 16 * i + 4 * q);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        c[r][2 * q] = __ffma2_rn(make_float2(w.x, w.y), h[r], c[r][2 * q]);
-        c[r][2 * q + 1] = __ffma2_rn(make_float2(w.z, w.w), h[r], c[r][2 * q + 1]);
+      for (int r = 0; r < 4; ++r) {
+        float e = fmaf(e0.y, fabsf(xr[r][0]), e0.x);
+        e = fmaf(e0.z, fabsf(xr[r][1]), e);
+        e = fmaf(e0.w, fabsf(xr[r][2]), e);
+        e = fmaf(e1.x, fabsf(xr[r][3]), e);
+        e = fmaf(e1.y, fabsf(xr[r][4]), e);
+        err[r] = q == 0 ? fmaf(e1.z, fabsf(xr[r][5]), e) : 0.0f;  // the four lanes' shares are added below
       }
     }
-  }
-  float2 d[R][4];
+    uint32_t hi[2][4], lo[2][4];
+    float a2[2][4][4];
+    start16<4>(a2, T + kFiltB2, q);
+    // layer 1 a block of 16 units at a time, straight into layer 2
+#pragma unroll 1
+    for (int kb = 0; kb < 4; ++kb) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const float2 b = reinterpret_cast<const float2*>(T + kFiltB4)[q];
+      for (int h = 0; h < 2; ++h) {
+        float v[2][4];  // units 16 kb + 8 h + 2 q + {0, 1} of the four rows
 #pragma unroll
-    for (int r = 0; r < R; ++r) d[r][q] = b;
-  }
+        for (int w = 0; w < 2; ++w) {
+          const float* W = T + kFiltW1 + 8 * (16 * kb + 8 * h + 2 * q + w);
+          const float4 w0 = *reinterpret_cast<const float4*>(W), w1 = *reinterpret_cast<const float4*>(W + 4);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    float2 h[R];
-    const float kap = T[kFiltK3 + i];
+          for (int r = 0; r < 4; ++r) {
+            float s = fmaf(w0.x, xr[r][0], w1.z);
+            s = fmaf(w0.y, xr[r][1], s);
+            s = fmaf(w0.z, xr[r][2], s);
+            s = fmaf(w0.w, xr[r][3], s);
+            s = fmaf(w1.x, xr[r][4], s);
+            s = fmaf(w1.y, xr[r][5], s);
+            s = relu_nan(s);
+            err[r] = fmaf(w1.w, s, err[r]);
+            v[w][r] = s;
+          }
+        }
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const float v = fmaxf(i & 1 ? c[r][i / 2].y : c[r][i / 2].x, 0.0f);
-      err[r] = fmaf(kap, v, err[r]);
-      h[r] = make_float2(v, v);
-    }
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const float4 w = *reinterpret_cast<const float4*>(T + kFiltW4 + 8 * i + 4 * q);
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        d[r][2 * q] = __ffma2_rn(make_float2(w.x, w.y), h[r], d[r][2 * q]);
-        d[r][2 * q + 1] = __ffma2_rn(make_float2(w.z, w.w), h[r], d[r][2 * q + 1]);
+        for (int r = 0; r < 4; ++r) split16(v[0][r], v[1][r], hi[r >> 1][2 * h + (r & 1)], lo[r >> 1][2 * h + (r & 1)]);
       }
+      block16<4>(a2, hi, lo, T + kFiltW2 + 512 * kb, lane);
     }
-  }
+    float a3[2][2][4];
+    start16<2>(a3, T + kFiltB3, q);
 #pragma unroll
-  for (int r = 0; r < R; ++r) {
-    const float4 b = *reinterpret_cast<const float4*>(T + kFiltB5);
-    float z[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float v = fmaxf(i & 1 ? d[r][i / 2].y : d[r][i / 2].x, 0.0f);
-      err[r] = fmaf(T[kFiltK4 + i], v, err[r]);
-      const float4 w = *reinterpret_cast<const float4*>(T + kFiltW5 + 4 * i);
-      z[0] = fmaf(w.x, v, z[0]);
-      z[1] = fmaf(w.y, v, z[1]);
-      z[2] = fmaf(w.z, v, z[2]);
-      z[3] = fmaf(w.w, v, z[3]);
+    for (int kb = 0; kb < 2; ++kb) {
+      next16<4>(a2, 2 * kb, 0, T + kFiltK2, q, err, hi, lo);
+      next16<4>(a2, 2 * kb + 1, 1, T + kFiltK2, q, err, hi, lo);
+      block16<2>(a3, hi, lo, T + kFiltW3 + 256 * kb, lane);
     }
-    unsigned eta = 0u;
-    bool sure = true;
+    float a4[2][1][4];
+    start16<1>(a4, T + kFiltB4, q);
+    next16<2>(a3, 0, 0, T + kFiltK3, q, err, hi, lo);
+    next16<2>(a3, 1, 1, T + kFiltK3, q, err, hi, lo);
+    block16<1>(a4, hi, lo, T + kFiltW4, lane);
+    float z[2][1][4];
+    start16<1>(z, T + kFiltB5, q);
+    next16<1>(a4, 0, 0, T + kFiltK4, q, err, hi, lo);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      eta |= (z[k] > 0.0f ? 1u : 0u) << k;
-      sure = sure && fabsf(z[k]) > err[r] && fabsf(z[k]) <= 3.0e38f;
+    for (int mt = 0; mt < 2; ++mt) hi[mt][2] = hi[mt][3] = lo[mt][2] = lo[mt][3] = 0u;  // eight inputs only
+    block16<1>(z, hi, lo, T + kFiltW5, lane);
+    // rows' bits: lane q = 0 holds logits 0, 1 of its rows, q = 1 logits 2, 3
+    unsigned w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      float e = err[r];
+      e += __shfl_xor_sync(0xffffffffu, e, 1);
+      e += __shfl_xor_sync(0xffffffffu, e, 2);
+      const float z0 = z[r >> 1][0][2 * (r & 1)], z1 = z[r >> 1][0][2 * (r & 1) + 1];
+      const bool sure = fabsf(z0) > e && fabsf(z0) <= 3.0e38f && fabsf(z1) > e && fabsf(z1) <= 3.0e38f;
+      unsigned b = ((z0 > 0.0f ? 1u : 0u) | (z1 > 0.0f ? 2u : 0u)) << (2 * q) | (sure ? 0u : 16u);
+      b = q < 2 ? b : 0u;
+      b |= __shfl_xor_sync(0xffffffffu, b, 1);
+      w[r] = b;  // complete in lanes 4 g and 4 g + 1
     }
-    res[r] = eta | (sure ? 16u : 0u);
+    unsigned mine = 0u;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const unsigned b = __shfl_sync(0xffffffffu, w[r], 4 * (lane & 7));
+      if ((lane >> 3) == r) mine = b;
+    }
+    mine ^= 16u;
+    if (side == 0) res[0] = mine;
+    else res[1] = mine;
   }
 }
 
@@ -282,7 +328,7 @@ __device__ __forceinline__ unsigned mlp64_rows(const double* __restrict__ Wt, co
 // The same for one row by a whole warp (lane = output, each output's chain in
 // the canonical order): 138 dependent FMA issues instead of 3104.  s: the
 // row's six raw stencil values, readable by every lane, `sstride` doubles
-// apart; ws: 128 doubles of the warp's scratch.  Returns the eta bits in all
+// apart; ws: 72 doubles of the warp's scratch (64 hidden values, 6 inputs).  Returns the eta bits in all
 // lanes.  All 32 lanes call it.
 __device__ __forceinline__ unsigned mlp64_warp(const double* __restrict__ Wt, const double* s, int sstride,
                                                double* ws) {
@@ -293,7 +339,7 @@ __device__ __forceinline__ unsigned mlp64_warp(const double* __restrict__ Wt, co
     for (int j = 0; j < 6; ++j) st[j] = s[j * sstride];
     normalise6(st, x);
 #pragma unroll
-    for (int j = 0; j < 6; ++j) ws[120 + j] = x[j];
+    for (int j = 0; j < 6; ++j) ws[64 + j] = x[j];
   }
   __syncwarp();
 #pragma unroll
@@ -301,36 +347,36 @@ __device__ __forceinline__ unsigned mlp64_warp(const double* __restrict__ Wt, co
     const int o = lane + 32 * q;
     double h = Wt[384 + o];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) h = __fma_rn(Wt[k * 64 + o], ws[120 + k], h);
+    for (int k = 0; k < 6; ++k) h = __fma_rn(Wt[k * 64 + o], ws[64 + k], h);
     ws[o] = relu(h);
   }
   __syncwarp();
-  {
-    double h = Wt[2496 + lane];
+  // each layer's values replace those two layers below
+  double h2 = Wt[2496 + lane];
 #pragma unroll 16
-    for (int i = 0; i < 64; ++i) h = __fma_rn(Wt[448 + i * 32 + lane], ws[i], h);
-    ws[64 + lane] = relu(h);
-  }
+  for (int i = 0; i < 64; ++i) h2 = __fma_rn(Wt[448 + i * 32 + lane], ws[i], h2);
+  __syncwarp();
+  ws[lane] = relu(h2);
   __syncwarp();
   if (lane < 16) {
     double h = Wt[3040 + lane];
 #pragma unroll 16
-    for (int i = 0; i < 32; ++i) h = __fma_rn(Wt[2528 + i * 16 + lane], ws[64 + i], h);
-    ws[96 + lane] = relu(h);
+    for (int i = 0; i < 32; ++i) h = __fma_rn(Wt[2528 + i * 16 + lane], ws[i], h);
+    ws[32 + lane] = relu(h);
   }
   __syncwarp();
   if (lane < 8) {
     double h = Wt[3184 + lane];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) h = __fma_rn(Wt[3056 + i * 8 + lane], ws[96 + i], h);
-    ws[112 + lane] = relu(h);
+    for (int i = 0; i < 16; ++i) h = __fma_rn(Wt[3056 + i * 8 + lane], ws[32 + i], h);
+    ws[lane] = relu(h);
   }
   __syncwarp();
   bool bit = false;
   if (lane < 4) {
     double z = Wt[3224 + lane];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) z = __fma_rn(Wt[3192 + i * 4 + lane], ws[112 + i], z);
+    for (int i = 0; i < 8; ++i) z = __fma_rn(Wt[3192 + i * 4 + lane], ws[i], z);
     bit = gt0(z);
   }
   const unsigned eta = __ballot_sync(0xffffffffu, bit) & 15u;
