@@ -14,7 +14,7 @@
 //         rows whose logits fall within +-guard_tau of 0 re-evaluated in FP32
 //         on the CUDA cores.
 //
-// Face kernel: persistent CTAs of one warpgroup (eight per SM, each with 64
+// Face kernel: CTAs of one warpgroup that take block after block (eight per SM, each with 64
 // TMEM columns -- all 512 of the SM's -- 64 registers per thread and 26 KB
 // of shared memory; the classifier's hidden activations stay in TMEM).  A
 // block is 64 faces on 4 grid lines: 4 rows x 16 consecutive x faces, or 4
@@ -65,6 +65,17 @@ static_assert(kMaxCells <= 128, "one stencil cell per thread");
 // deviations small: at most 10 cells along and 2 across the lines.
 constexpr int kRefX = 1 * kLineCells + kLineCells / 2;
 constexpr int kRefY = (kLineCells / 2) * kLines + 1;
+// Blocks are handed out as CTAs finish: a grid of one CTA per block, of which
+// those that run take over the ones not launched yet (clusterlaunchcontrol).  The
+// eight CTAs of an SM do not advance evenly: with the blocks dealt out beforehand
+// 29.1 of an SM's 32 warps were active on average, and a grid of one and a third
+// waves waited for whole CTAs of two blocks.  A step, dealt out -> handed out:
+// 256 x 192 270 -> 218 us, 400^2 515 -> 414 us, 4096^2 28.4 -> 26.5 ms.  The next
+// block is asked for in a block's last batch: asked for at once the CTAs that
+// start first take blocks from SMs not filled yet (256 x 192: 285 us).  Up to
+// kResident blocks all run at once and nobody asks.
+constexpr unsigned kResident = 152 * 8;
+constexpr int kAskBatch = 3;
 constexpr int kAlign = 128;
 
 constexpr int align_up(int x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -91,11 +102,12 @@ constexpr int kOffA = align_up(kOffL + kFaces * 12 * 4);
 constexpr int kOffR = align_up(kOffA + kFaces * 4 * 4);           // kFaces x 5 floats
 constexpr int kOffRef = align_up(kOffR + kFaces * 5 * 4);         // 8 doubles + 8 floats
 constexpr int kOffBar = kOffRef + 8 * 8 + 8 * 4;  // mbarrier, TMEM address, timeout flag
-constexpr int kOffWtab = align_up(kOffBar + 16);    // 16 masks x 4 renormalised weights
+constexpr int kOffNext = kOffBar + 16;              // the next block: answer, mbarrier; rows re-evaluated
+constexpr int kOffWtab = align_up(kOffNext + 28);   // 16 masks x 4 renormalised weights
 constexpr int kFacesSmem = align_up(kOffWtab + 16 * 4 * 4);
 // Eight CTAs per SM: 228 KB of shared memory, allocated in 128-byte units
 // plus 1 KB reserved per CTA (and 8 x 64 TMEM columns = 512).
-static_assert(kOffBar % 8 == 0 && kFacesSmem % 128 == 0, "alignment");
+static_assert(kOffBar % 8 == 0 && kOffNext % 16 == 0 && kFacesSmem % 128 == 0, "alignment");
 static_assert(8 * (kFacesSmem + 1024) <= 228 * 1024, "face kernel: CTAs per SM");
 
 // per-cell arrays
@@ -313,6 +325,17 @@ __device__ __forceinline__ bool face_valid(const BlockGeom& b, int k, int nx, in
                     : (b.face0 + k / kLines <= ny && b.line0 + k % kLines < nx);
 }
 
+// After a timeout nothing more is started: take the blocks not launched yet off
+// the grid (one thread; `phase` is the next answer's).
+__device__ __noinline__ void drain_blocks(void* answer, uint64_t* bar, uint32_t phase) {
+  while (mbar_wait(bar, phase ^ 1u)) {
+    try_cancel(answer, bar);
+    if (!mbar_wait(bar, phase) || cancelled_block(answer) < 0) break;
+    phase ^= 1u;
+    fence_async_smem();
+  }
+}
+
 template <int NDIM, bool BF16>
 __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __grid_constant__ FacesMixedArgs a) {
   constexpr int NV = NDIM == 2 ? 4 : 3;
@@ -327,6 +350,8 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
   uint64_t* bar = reinterpret_cast<uint64_t*>(smem + kOffBar);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kOffBar + 8);
   int* fail_flag = reinterpret_cast<int*>(smem + kOffBar + 12);
+  int* s_guarded = reinterpret_cast<int*>(smem + kOffNext + 24);  // rows re-evaluated
+  uint64_t* next_bar = reinterpret_cast<uint64_t*>(smem + kOffNext + 16);
   const int t = threadIdx.x;
   const int nx = a.nx, ny = a.ny;
 
@@ -338,8 +363,10 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
   if (t < 16) s_wtab[t] = make_float4(a.wtab[t][0], a.wtab[t][1], a.wtab[t][2], a.wtab[t][3]);
   if (t == 0) {
     mbar_init(bar, 1);
+    mbar_init(next_bar, 1);
     fence_mbar_init();
     *fail_flag = 0;
+    *s_guarded = 0;
   }
   if (t < 32) {
     tmem_alloc(tmem_slot, 64);
@@ -349,14 +376,13 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   MlpCtx mc{s_net, smem + kOffBufY, bar, *tmem_slot, 0u, BF16, fail_flag};
-  unsigned guarded = 0;
-  bool failed = false;
 
-  const int nblk = a.nblk_x + a.nblk_y;
   double* refd = reinterpret_cast<double*>(smem + kOffRef);      // U_ref[4], F_ref[4] (FP64)
   float* reff = reinterpret_cast<float*>(smem + kOffRef + 64);   // same, FP32, interleaved
   float* sRf = reinterpret_cast<float*>(smem + kOffR);           // ut, vt, Ht, ct, qt per face
-  for (int blk = (int)blockIdx.x; blk < nblk && !failed; blk += gridDim.x) {
+  uint32_t nphase = 0u;
+  int blk = (int)blockIdx.x;
+  while (blk >= 0) {
     // ---- block geometry
     const BlockGeom bg = block_geom(blk, a);
     const int dir = bg.dir;
@@ -504,6 +530,7 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
     float corr_even = 0.0f;
     unsigned ebits_even = 0u;
     for (int mt = 0; mt < kFaces / 16; ++mt) {
+      if (mt == kAskBatch && t == 0 && gridDim.x > kResident) try_cancel(smem + kOffNext, next_bar);
       const int k = mt * 16 + (t >> 3);
       const int fld = (t >> 1) & 3;
       const int m = min(fld, NV - 1);
@@ -575,16 +602,18 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
         asm volatile("" : "+f"(inv));  // x is formed anew below, not kept
         float z[4];
         if (!mlp_tc<BF16>(mc, z)) {
-          failed = true;
+          // the end of the block expects an answer
+          if (mt < kAskBatch && t == 0 && gridDim.x > kResident) try_cancel(smem + kOffNext, next_bar);
           break;
         }
         if (a.guard_tau > 0.0f) {
           bool flag = false;
 #pragma unroll
           for (int q = 0; q < 4; ++q) flag |= fabsf(z[q]) < a.guard_tau;
-          guarded += (flag && valid) ? 1 : 0;
           const unsigned bal = __ballot_sync(0xffffffffu, flag);
           if (bal) {
+            const unsigned counted = __ballot_sync(0xffffffffu, flag && valid);
+            if ((t & 31) == 0) atomicAdd(s_guarded, __popc(counted));
             // the inputs again, as above: two values live across the classifier
             // instead of six
             auto xin = [&](int j) { return (cref + ds[j]) * inv; };
@@ -680,13 +709,21 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
       }
       __syncthreads();
     }
-    __syncthreads();
+    if (gridDim.x <= kResident) break;
+    if (!mbar_wait(next_bar, nphase)) *fail_flag = 1;
+    nphase ^= 1u;
+    blk = cancelled_block(smem + kOffNext);
+    fence_async_smem();
+    if (__syncthreads_or(*fail_flag)) break;
   }
-  if (failed && t == 0) atomicOr(a.status, 4);
-  if (a.guard_count && guarded) atomicAdd(a.guard_count, (unsigned long long)guarded);
+  if (*fail_flag && t == 0) {
+    atomicOr(a.status, 4);
+    if (gridDim.x > kResident && blk >= 0) drain_blocks(smem + kOffNext, next_bar, nphase);
+  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (t == 0 && a.guard_count && *s_guarded) atomicAdd(a.guard_count, (unsigned long long)*s_guarded);
   if (t < 32) tmem_dealloc(*tmem_slot, 64);
 }
 
@@ -832,14 +869,13 @@ cudaError_t launch_faces_mixed(int ndim, FacesMixedArgs& a, cudaStream_t s, int 
   a.nblk_y = ndim == 2 ? a.byc * (fr1 - fr0) : 0;
   const int nblk = a.nblk_x + a.nblk_y;
   if (nblk <= 0) return cudaSuccess;
-  // persistent grid: eight resident CTAs per SM (registers, shared memory,
-  // 64 TMEM columns each)
-  const int blocks = nblk < 152 * 8 ? nblk : 152 * 8;
+  // a CTA per block, eight resident per SM (registers, shared memory, 64 TMEM
+  // columns each); see kResident
   auto kern = ndim == 2 ? (a.bf16 ? faces_mixed_kernel<2, true> : faces_mixed_kernel<2, false>)
                         : (a.bf16 ? faces_mixed_kernel<1, true> : faces_mixed_kernel<1, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kFacesSmem);
   if (e != cudaSuccess) return e;
-  kern<<<blocks, kMlpThreads, kFacesSmem, s>>>(a);
+  kern<<<nblk, kMlpThreads, kFacesSmem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -29,6 +29,9 @@ __host__ __device__ constexpr uint32_t kmajor_offset(int r, int k, int K) {
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
+__device__ __forceinline__ void mbar_inval(uint64_t* bar) {
+  asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
 __device__ __forceinline__ void fence_mbar_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
@@ -68,6 +71,27 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
                : "memory");
+}
+// Ask for a block of this grid that has not been launched yet, to be run by this
+// one instead; the answer (16 bytes, 16-byte aligned) arrives on `bar`.
+__device__ __forceinline__ void try_cancel(void* answer, uint64_t* bar) {
+  mbar_arrive_expect_tx(bar, 16u);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                   smem_u32(answer)),
+               "r"(smem_u32(bar))
+               : "memory");
+}
+// Its blockIdx.x, or -1 when every block has been launched.
+__device__ __forceinline__ int cancelled_block(const void* answer) {
+  int x;
+  asm volatile(
+      "{\n .reg .pred p;\n .reg .b128 h;\n ld.shared::cta.b128 h, [%1];\n"
+      " clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n mov.b32 %0, -1;\n"
+      " @p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n}"
+      : "=r"(x)
+      : "r"(smem_u32(answer))
+      : "memory");
+  return x;
 }
 // Bulk copy of `bytes` (a multiple of 16; both addresses 16-byte aligned) from
 // global to this CTA's shared memory, completing on `bar`.

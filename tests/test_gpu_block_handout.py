@@ -1,0 +1,41 @@
+"""The mixed face kernel's blocks, handed out to the running CTAs as they finish.
+
+A state tiled periodically from whole face blocks (64 x 48 cells) gives every
+block the stencils, the reference state and hence the bits of its counterpart
+in the small grid, so dU/dt and the masks of the large grid are those of the
+small one, repeated: a block left out, taken twice or misplaced shows.  Sizes on
+both sides of the 1216 blocks that run at once, and far above.
+"""
+import numpy as np
+import pytest
+import torch
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision,mode", [("fp16", "mlp"), ("bf16", "mlp"), ("fp16", "smooth")])
+@pytest.mark.parametrize("kx,ky", [(3, 3), (4, 3), (7, 5), (16, 16)])
+def test_a_tiled_state_gives_a_tiled_result(precision, mode, kx, ky):
+    import paper_2207_08500_gb300 as p
+    nx, ny = 64, 48
+    U = synth.noisy(synth.quadrants_2d(nx, ny, seed=41), 42)
+    out = []
+    for a, b in ((1, 1), (kx, ky)):
+        g = p.Neno6(ndim=2, nx=nx * a, ny=ny * b, dx=1.0 / nx, dy=1.0 / ny, precision=precision, mask_mode=mode)
+        V = torch.from_numpy(np.ascontiguousarray(np.tile(U, (1, b, a)))).cuda()
+        d = torch.full_like(V, float("nan"))
+        for _ in range(3):
+            d.copy_(g.rhs(V))
+        m = g.rhs(V, want_mask=True)[1].cpu().numpy() if mode == "mlp" else None
+        assert g.status() == 0
+        out.append((d.cpu().numpy(), m, nx * a, ny * b))
+    (d1, m1, _, _), (d2, m2, NX, NY) = out
+    assert np.array_equal(np.tile(d1, (1, ky, kx)), d2)
+    if m1 is not None:
+        def split(m, w, h):  # x faces (4, h, w + 1), then y faces (4, h + 1, w)
+            n = 4 * h * (w + 1)
+            return m.reshape(-1)[:n].reshape(4, h, w + 1)[:, :, :-1], m.reshape(-1)[n:].reshape(4, h + 1, w)[:, :-1]
+        for s, l in zip(split(m1, nx, ny), split(m2, NX, NY)):
+            assert np.array_equal(np.tile(s, (1, ky, kx)), l)
