@@ -16,11 +16,11 @@
 // settle a logit's sign (mlp_filter.cuh).  What stays on the FP64 pipe is the reconstruction itself,
 // ~1150 operations per cell, and each is done once: a thread takes a face
 // with all its characteristic fields, so the Roe state is formed once per face.
-// Persistent CTAs take tiles of cells: the tile plus a 3-cell halo (periodic
+// CTAs take tile after tile of cells: the tile plus a 3-cell halo (periodic
 // wrap or zero-gradient copy done in the load) and the per-cell quantities are
 // staged in shared memory, the faces' fluxes written back there and
 // differenced, with no scratch in global memory.  Comparisons (ReLU, max, |x|)
-// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 11.7 ms,
+// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 11.4 ms,
 // against 437 ms with every classifier row in binary64 and four lanes per
 // face; the FP64 operations alone would take 7.9 ms of a full FP64 pipe.
 #include <cuda_fp16.h>
@@ -33,6 +33,7 @@
 #include "fp64_ops.cuh"
 #include "internal.h"
 #include "mlp_filter.cuh"
+#include "tc.cuh"
 
 namespace neno6 {
 namespace {
@@ -49,6 +50,7 @@ template <int NDIM_, int TX_, int TY_, int NT_, int OCC_, bool SPLIT_>
 struct Tile {
   static constexpr int NDIM = NDIM_, TX = TX_, TY = TY_, NT = NT_, OCC = OCC_;
   static constexpr bool SPLIT = SPLIT_;
+  static constexpr unsigned kResident = 152 * OCC;  // CTAs that run at a time
   static constexpr int NV = NDIM == 2 ? 4 : 3;
   static constexpr int HY = NDIM == 2 ? 3 : 0;
   static constexpr int SX = TX + 6, SY = TY + 2 * HY, NC = SX * SY;
@@ -72,7 +74,7 @@ struct Tile {
   static constexpr int O_D = O_G + (SPLIT ? (NV + 5) * (NXF + NYF) : 0);
   static constexpr int O_T = (O_D + 2) / 2 * 2;
   static constexpr size_t SMEM = sizeof(double) * O_T + sizeof(float) * kFiltFloats;
-  static_assert(NT % 32 == 0 && OCC * (SMEM + 1024) <= 228 * 1024, "resident CTAs");
+  static_assert(NT % 32 == 0 && OCC * (SMEM + 1024 + 128) <= 228 * 1024, "resident CTAs");
 };
 
 // x is 0 or its magnitude lies in [2^-60, 2^60).
@@ -173,7 +175,13 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
   double* sF = smem + G::O_F;            // x faces [NV][TY][TX+1], then y faces [NV][TY+1][TX]
   double* park0 = smem + G::O_P;         // [kPark][NT]
   float* T = reinterpret_cast<float*>(smem + G::O_T);
+  __shared__ __align__(16) uint4 s_next;  // the next tile's answer
+  __shared__ __align__(8) uint64_t s_nbar;
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t == 0) {
+    tc::mbar_init(&s_nbar, 1);
+    tc::fence_mbar_init();
+  }
   double* park = park0 + t;
   double* ws = smem + G::O_W + warp * G::kScratch;
   const int nx = a.nx, ny = a.ny;
@@ -216,9 +224,11 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
     if (lane == 0) *sdt = dt;
   }
 
-  const long long ntx = (nx + TX - 1) / TX, ntiles = ntx * ((ny + TY - 1) / TY);
-  for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int i0 = (int)(tile % ntx) * TX, j0 = (int)(tile / ntx) * TY;
+  const int ntx = (nx + TX - 1) / TX;
+  uint32_t nphase = 0u;
+  int tile = (int)blockIdx.x;
+  do {
+    const int i0 = tile % ntx * TX, j0 = tile / ntx * TY;
     // ---- 1. tile + halo (without its corners) and per-cell quantities.
     // `odd`: some value is not 0 or in [2^-60, 2^60), or a cell is not
     // physical; the tile's faces then take every operation of the
@@ -480,8 +490,11 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
       }
     }
     __syncthreads();
-    if (!a.out) continue;
-    if (G::SPLIT) {
+    // Tiles are handed out: a CTA takes over one that has not been launched yet.
+    // Rows evaluated again in binary64 make tiles uneven, and an SM's two CTAs do
+    // not advance evenly (2048^2 11.69 ms dealt out beforehand, 11.42 handed out).
+    if (t == 0 && gridDim.x > G::kResident) tc::try_cancel(&s_next, &s_nbar);
+    if (G::SPLIT && a.out) {
       const double* sG = smem + G::O_G;
       for (int e = t; e < NV * (G::NXF + G::NYF); e += NT) {
         const int n = e / (G::NXF + G::NYF), fi = e % (G::NXF + G::NYF);
@@ -504,7 +517,7 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
     // A division by a power of two is the exact product with its reciprocal.
     const double* sFy = sF + NV * G::NXF;
     const double dt = a.stage ? *sdt : 0.0;
-    for (int e = t; e < TX * TY; e += NT) {
+    for (int e = a.out ? t : TX * TY; e < TX * TY; e += NT) {
       const int c = e % TX, rw = e / TX;
       const int gi = i0 + c, gj = j0 + rw;
       if (gi >= nx || gj >= ny) continue;
@@ -533,8 +546,17 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
         a.out[n * plane + g] = val;
       }
     }
-    __syncthreads();  // the next tile's cells overwrite what the difference reads
-  }
+    if (gridDim.x <= G::kResident) break;
+    const bool lost = !tc::mbar_wait(&s_nbar, nphase);
+    nphase ^= 1u;
+    tile = tc::cancelled_block(&s_next);
+    tc::fence_async_smem();
+    // the next tile's cells overwrite what the difference reads
+    if (__syncthreads_or(lost)) {
+      if (t == 0) atomicOr(a.status, 4);
+      break;
+    }
+  } while (tile >= 0);
 }
 
 __global__ void __launch_bounds__(256) classify_fp64_kernel(const __grid_constant__ ClassifyParamsF64 P) {
@@ -816,8 +838,7 @@ cudaError_t launch_tiles(const RhsArgs& a, cudaStream_t s) {
       cudaFuncSetAttribute(rhs_fp64_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
   if (e != cudaSuccess) return e;
   const long long tiles = (long long)((a.nx + G::TX - 1) / G::TX) * ((a.ny + G::TY - 1) / G::TY);
-  const long long most = 152ll * G::OCC;
-  return dependent_launch(rhs_fp64_kernel<G>, (unsigned)(tiles < most ? tiles : most), G::NT, G::SMEM, s, a);
+  return dependent_launch(rhs_fp64_kernel<G>, (unsigned)tiles, G::NT, G::SMEM, s, a);
 }
 
 // 1/d when d is a power of two whose reciprocal is normal, else 0.
@@ -836,7 +857,9 @@ cudaError_t launch_rhs_fp64(int ndim, RhsArgs& a, cudaStream_t s) {
   // however few lanes are active): 2.13 face slots per cell for 15 x 16, 2.29
   // for 7 x 16.  The smaller the grid, the smaller the tile, so that every SM
   // has warps; the smallest grids give a warp a single field.  Measured in us
-  // per RHS, periodic quadrants (threads x CTAs per SM; * taken):
+  // per RHS, periodic quadrants (threads x CTAs per SM; * taken; tiles dealt out
+  // beforehand, handed out the starred ones take 327 at 300^2, 807 at 512^2, 2951
+  // at 1024^2 and 11420 at 2048^2):
   //                        24x16 64x64 100x100 200x136 300x300 400x400 512^2 700^2 1024^2 2048^2
   //   15 x 16       256x2   209   135    140     142     350     551    822* 1467*  3034*  11696*
   //   15 x 16       192x2   236   154            161                    848         3107   12058

@@ -16,7 +16,7 @@
 // results stay in registers.  They fit this kernel: a warp's 64 rows (32 faces,
 // two sides) need no barrier, no tensor memory and no wait on other warps, and
 // at 2 clocks per instruction and SM they take a quarter of the FP64 time beside
-// which they run.  2048^2 RHS: 11.7 ms, against 13.8 ms with every layer in FP32
+// which they run.  2048^2 RHS: 11.69 ms, against 13.8 ms with every layer in FP32
 // on the CUDA cores (weights by broadcast loads, which bound it).
 //
 // The bound (forward error analysis, Higham, "Accuracy and Stability of

@@ -1,10 +1,12 @@
-"""The mixed face kernel's blocks, handed out to the running CTAs as they finish.
+"""The face blocks of the mixed kernel and the tiles of the FP64 one, handed out to
+the running CTAs as they finish.
 
 A state tiled periodically from whole face blocks (64 x 48 cells) gives every
 block the stencils, the reference state and hence the bits of its counterpart
 in the small grid, so dU/dt and the masks of the large grid are those of the
 small one, repeated: a block left out, taken twice or misplaced shows.  Sizes on
-both sides of the 1216 blocks that run at once, and far above.
+both sides of the 1216 blocks that run at once, and far above; the FP64 result
+does not depend on the tile at all.
 """
 import numpy as np
 import pytest
@@ -15,7 +17,7 @@ import synth
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("precision,mode", [("fp16", "mlp"), ("bf16", "mlp"), ("fp16", "smooth")])
+@pytest.mark.parametrize("precision,mode", [("fp16", "mlp"), ("bf16", "mlp"), ("fp16", "smooth"), ("fp64", "mlp")])
 @pytest.mark.parametrize("kx,ky", [(3, 3), (4, 3), (7, 5), (16, 16)])
 def test_a_tiled_state_gives_a_tiled_result(precision, mode, kx, ky):
     import paper_2207_08500_gb300 as p
