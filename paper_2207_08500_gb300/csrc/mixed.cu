@@ -42,9 +42,18 @@ using namespace tcmlp;
 constexpr int kResidencyPad = 8 * 1024;
 // static shared memory of the kernel below: image, input tile, the next tile's
 // stencils, barriers, TMEM address, timeout flag
-constexpr int kClassifySmem = kNetImageBytes + kBufYBytes + 128 * 48 + 24;
+constexpr int kClassifySmem = kNetImageBytes + kBufYBytes + 128 * 48 + 56;
 
-template <bool BF16, bool NARROW>
+// HANDOUT: a CTA per tile, of which those that run take over the ones not
+// launched yet, as the CTAs of an SM do not advance evenly: dealt out beforehand
+// an SM had 25 of its 32 warps active on average.  From kHandout tiles on; below,
+// what the first CTAs take before the other SMs are filled costs more than that.
+// us for 2^20, 2^21, 2^22, 2^23 stencils: dealt out 29.1, 51.6, 94.6, 178.6, handed
+// out 30.1, 49.7, 90.5, 170.2.
+constexpr unsigned kResident = 152 * 8;
+constexpr unsigned kHandout = 12 * kResident;
+
+template <bool BF16, bool NARROW, bool HANDOUT>
 __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const double* __restrict__ X,
                                                                       long long n, uint8_t* __restrict__ eta,
                                                                       double* __restrict__ logits,
@@ -53,7 +62,9 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
   __shared__ __align__(128) uint8_t s_net[kNetImageBytes];
   __shared__ __align__(128) uint8_t s_bufY[kBufYBytes];
   __shared__ __align__(128) double s_x[128 * 6];
-  __shared__ __align__(8) uint64_t s_bar, s_xbar;
+  __shared__ __align__(16) uint4 s_answer;
+  __shared__ __align__(8) uint64_t s_bar, s_xbar, s_nbar;
+  __shared__ int s_next;
   __shared__ uint32_t s_tmem;
   __shared__ int s_fail;
   const int t = threadIdx.x;
@@ -62,6 +73,7 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
   if (t == 0) {
     mbar_init(&s_bar, 1);
     mbar_init(&s_xbar, 1);
+    if (HANDOUT) mbar_init(&s_nbar, 1);
     fence_mbar_init();
     s_fail = 0;
     rows.fetch(blockIdx.x);
@@ -75,7 +87,10 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
   tc_fence_after();
   MlpCtx c{s_net, s_bufY, &s_bar, s_tmem, 0u, BF16, &s_fail};
   const long long tiles = (n + 127) / 128;
-  for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+  bool asked = false;  // thread 0's: an answer is due, and its phase
+  uint32_t nphase = 0u;
+  for (long long tile = blockIdx.x; HANDOUT ? tile >= 0 : tile < tiles;
+       tile = HANDOUT ? (long long)s_next : tile + gridDim.x) {
     const long long r = tile * 128 + t;
     float x[6];
     float m = 1.0f;
@@ -86,13 +101,30 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
     for (int j = 0; j < 6; ++j) x[j] = x[j] / m;
     store_input_row<BF16>(s_bufY, t, x);
     fence_async_smem();
+    if (HANDOUT && t == 0) {
+      if (!asked) try_cancel(&s_answer, &s_nbar);
+      asked = true;
+      if (!mbar_wait(&s_nbar, nphase)) s_fail = 1;
+      nphase ^= 1u;
+      s_next = cancelled_block(&s_answer);
+    }
     __syncthreads();
-    if (t == 0) rows.fetch(tile + gridDim.x);
+    if (!HANDOUT) {
+      if (t == 0) rows.fetch(tile + gridDim.x);
+    } else if (t == 0 && s_next >= 0) {
+      rows.fetch(s_next);
+      fence_async_smem();
+      try_cancel(&s_answer, &s_nbar);
+    }
     float z[4];
     if (!(NARROW ? mlp_tc_narrow<BF16>(c, z) : mlp_tc<BF16>(c, z))) {
       if (t == 0) atomicOr(status, 4);
-      // a copy may still be in flight: wait for it (bounded) before leaving
-      rows.get(tile, x);
+      // copies may still be in flight: wait for them (bounded) before leaving
+      if (!HANDOUT || s_next >= 0) rows.get(tile, x);
+      if (HANDOUT && t == 0 && s_next >= 0 && mbar_wait(&s_nbar, nphase) && cancelled_block(&s_answer) >= 0) {
+        fence_async_smem();
+        drain_blocks(&s_answer, &s_nbar, nphase ^ 1u);
+      }
       break;
     }
     if (r < n) {
@@ -270,21 +302,14 @@ cudaError_t launch_classify_mixed(const double* X, long long n, uint8_t* eta, do
   static_assert(8 * kPerCta <= 228 * 1024, "eight resident CTAs");
   static_assert(9 * kPerCta > 228 * 1024, "nine resident CTAs would oversubscribe TMEM");
   static_assert(kClassifySmem + kResidencyPad <= 48 * 1024, "no opt-in needed");
-  const int blocks = (int)(tiles < 152 * 8 ? tiles : 152 * 8);
-  if (narrow) {
-    if (bf16)
-      classify_mixed_kernel<true, true><<<blocks, kMlpThreads, kResidencyPad, s>>>(X, n, eta, logits, net_image,
-                                                                                  status);
-    else
-      classify_mixed_kernel<false, true><<<blocks, kMlpThreads, kResidencyPad, s>>>(X, n, eta, logits, net_image,
-                                                                                   status);
-  } else if (bf16) {
-    classify_mixed_kernel<true, false><<<blocks, kMlpThreads, kResidencyPad, s>>>(X, n, eta, logits, net_image,
-                                                                                 status);
-  } else {
-    classify_mixed_kernel<false, false><<<blocks, kMlpThreads, kResidencyPad, s>>>(X, n, eta, logits, net_image,
-                                                                                  status);
-  }
+  const bool handout = tiles >= kHandout;
+  const unsigned blocks = (unsigned)(tiles < kResident || handout ? tiles : kResident);
+  auto pick = [&](auto dealt, auto handed) { return handout ? handed : dealt; };
+  auto kern = narrow ? (bf16 ? pick(classify_mixed_kernel<true, true, false>, classify_mixed_kernel<true, true, true>)
+                             : pick(classify_mixed_kernel<false, true, false>, classify_mixed_kernel<false, true, true>))
+                     : (bf16 ? pick(classify_mixed_kernel<true, false, false>, classify_mixed_kernel<true, false, true>)
+                             : pick(classify_mixed_kernel<false, false, false>, classify_mixed_kernel<false, false, true>));
+  kern<<<blocks, kMlpThreads, kResidencyPad, s>>>(X, n, eta, logits, net_image, status);
   return cudaGetLastError();
 }
 

@@ -325,17 +325,6 @@ __device__ __forceinline__ bool face_valid(const BlockGeom& b, int k, int nx, in
                     : (b.face0 + k / kLines <= ny && b.line0 + k % kLines < nx);
 }
 
-// After a timeout nothing more is started: take the blocks not launched yet off
-// the grid (one thread; `phase` is the next answer's).
-__device__ __noinline__ void drain_blocks(void* answer, uint64_t* bar, uint32_t phase) {
-  while (mbar_wait(bar, phase ^ 1u)) {
-    try_cancel(answer, bar);
-    if (!mbar_wait(bar, phase) || cancelled_block(answer) < 0) break;
-    phase ^= 1u;
-    fence_async_smem();
-  }
-}
-
 template <int NDIM, bool BF16>
 __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __grid_constant__ FacesMixedArgs a) {
   constexpr int NV = NDIM == 2 ? 4 : 3;

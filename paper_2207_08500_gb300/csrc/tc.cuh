@@ -207,5 +207,16 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
                : "memory");
 }
 
+// After a timeout nothing more is started: take the blocks not launched yet off
+// the grid (one thread; `phase` is the next answer's, the one before has come).
+static __device__ __noinline__ void drain_blocks(void* answer, uint64_t* bar, uint32_t phase) {
+  while (mbar_wait(bar, phase ^ 1u)) {
+    try_cancel(answer, bar);
+    if (!mbar_wait(bar, phase) || cancelled_block(answer) < 0) break;
+    phase ^= 1u;
+    fence_async_smem();
+  }
+}
+
 }  // namespace tc
 }  // namespace neno6

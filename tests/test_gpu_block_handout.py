@@ -8,6 +8,8 @@ small one, repeated: a block left out, taken twice or misplaced shows.  Sizes on
 both sides of the 1216 blocks that run at once, and far above; the FP64 result
 does not depend on the tile at all.
 """
+import os
+
 import numpy as np
 import pytest
 import torch
@@ -41,3 +43,23 @@ def test_a_tiled_state_gives_a_tiled_result(precision, mode, kx, ky):
             return m.reshape(-1)[:n].reshape(4, h, w + 1)[:, :, :-1], m.reshape(-1)[n:].reshape(4, h + 1, w)[:, :-1]
         for s, l in zip(split(m1, nx, ny), split(m2, NX, NY)):
             assert np.array_equal(np.tile(s, (1, ky, kx)), l)
+
+
+@pytest.mark.parametrize("width", ["paper", "narrow"])
+@pytest.mark.parametrize("n", [12 * 1216 * 128 - 128, 12 * 1216 * 128 - 127, 12 * 1216 * 128 + 1, 2500017])
+def test_classify_repeats_a_repeated_input(width, n):
+    """Both sides of the 12 x 1216 tiles of 128 rows from which tiles are handed
+    out: rows repeated with a period that no tile divides give repeated results."""
+    import paper_2207_08500_gb300 as p
+    weights = p.DEFAULT_WEIGHTS
+    if width == "narrow":
+        weights = os.path.join(os.path.dirname(weights), "neno6_mlp_6x32x32x32x4.bin")
+    g = p.Neno6(ndim=1, nx=64, precision="fp16", weights=weights)
+    base = torch.from_numpy(synth.mlp_stencils(1009, seed=43)).cuda()
+    X = base.repeat((n + 1008) // 1009, 1)[:n].contiguous()
+    e1, z1 = g.classify(base, want_logits=True)
+    e2, z2 = g.classify(X, want_logits=True)
+    k = torch.arange(n, device="cuda") % 1009
+    assert torch.equal(e2, e1[k]) and torch.equal(z2, z1[k])
+    assert torch.equal(g.classify(X), e2)
+    assert g.status() == 0
