@@ -212,9 +212,9 @@ int neno6_classify(neno6_handle* h, const double* X, int64_t n, uint8_t* eta_out
  * LLF alpha argmax (first index on ties) held at their values for U.  Not in
  * the paper: the derivative of the scheme where the mask is locally
  * constant.  Evaluated in FP64 for every precision; each face is recomputed
- * from U (no stored intermediates) and differentiated exactly with
- * forward-mode dual numbers; each cell gathers the contributions of the faces
- * whose stencils contain it (no atomics, deterministic).
+ * from U (no stored intermediates) and differentiated exactly in reverse mode;
+ * each cell gathers the contributions of the faces whose stencils contain it
+ * (no atomics, deterministic).
  *   U       [nv][ny][nx] float64 state.
  *   lambda  [nv][ny][nx] float64 cotangent of dU/dt.
  *   mask    nullable; the frozen mask (layout of neno6_mask_bytes).  NULL:

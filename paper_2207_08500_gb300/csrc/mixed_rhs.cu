@@ -23,13 +23,14 @@
 // 64 Roe states once (one thread per face, FP64) while the other half of the
 // CTA forms the LLF alpha of every (face, field), then four 128-row
 // tensor-core batches of 16 faces x 4 fields x 2 sides.  The kernel is bound by
-// the latency of that chain at 59 % of the issue slots and half of the FP64
+// the latency of that chain at 66 % of the issue slots and half of the FP64
 // pipe, so what counts is instructions, FP64 instructions (64 clocks of an SM
 // quarter each, whatever the active lanes) and registers kept across the
 // classifier: 2048^2 RHS 2.31 ms with exact halvings on the integer pipe, the
 // final FP64 addition of two batches in one instruction, the guard band in a
 // function of its own and its inputs formed anew, one 32-bit division per block
-// and no branch around the combination, 2.46 ms without them.
+// and no branch around the combination, 2.46 ms without them (both before the
+// blocks were handed out, kResident below).
 //
 // Reference shift.  A cell near the block's centre is a reference state
 // (U_ref, F_ref); every cell is staged as the FP64 difference (U - U_ref,
