@@ -89,8 +89,9 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
   const long long tiles = (n + 127) / 128;
   bool asked = false;  // thread 0's: an answer is due, and its phase
   uint32_t nphase = 0u;
+  int next = 0;  // this thread's copy of s_next
   for (long long tile = blockIdx.x; HANDOUT ? tile >= 0 : tile < tiles;
-       tile = HANDOUT ? (long long)s_next : tile + gridDim.x) {
+       tile = HANDOUT ? (long long)next : tile + gridDim.x) {
     const long long r = tile * 128 + t;
     float x[6];
     float m = 1.0f;
@@ -109,10 +110,14 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
       s_next = cancelled_block(&s_answer);
     }
     __syncthreads();
+    // read between this barrier and the classifier's: thread 0 writes the word
+    // again in the next round, before its first barrier, when another warp may
+    // not have got to the end of this one
+    if (HANDOUT) next = s_next;
     if (!HANDOUT) {
       if (t == 0) rows.fetch(tile + gridDim.x);
-    } else if (t == 0 && s_next >= 0) {
-      rows.fetch(s_next);
+    } else if (t == 0 && next >= 0) {
+      rows.fetch(next);
       fence_async_smem();
       try_cancel(&s_answer, &s_nbar);
     }
@@ -120,8 +125,8 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
     if (!(NARROW ? mlp_tc_narrow<BF16>(c, z) : mlp_tc<BF16>(c, z))) {
       if (t == 0) atomicOr(status, 4);
       // copies may still be in flight: wait for them (bounded) before leaving
-      if (!HANDOUT || s_next >= 0) rows.get(tile, x);
-      if (HANDOUT && t == 0 && s_next >= 0 && mbar_wait(&s_nbar, nphase) && cancelled_block(&s_answer) >= 0) {
+      if (!HANDOUT || next >= 0) rows.get(tile, x);
+      if (HANDOUT && t == 0 && next >= 0 && mbar_wait(&s_nbar, nphase) && cancelled_block(&s_answer) >= 0) {
         fence_async_smem();
         drain_blocks(&s_answer, &s_nbar, nphase ^ 1u);
       }
