@@ -188,12 +188,13 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
   const size_t plane = (size_t)nx * ny;
   const double gm1 = a.gm1, gamma = a.gamma;
   const double* __restrict__ Wt = a.net64;
-  // the table is the handle's own and not written by the kernels before this
-  // one, so it is fetched while they drain (dependent_launch below); their
-  // results are read after the wait
-  if (a.mask_mode == kMaskMLP) filt::load_filter(T, a.filter, t, NT);
+  // a handle's table is never written by the kernels before this one, so it is
+  // fetched while they drain (dependent_launch below); what they write, a table
+  // laid out on the stream among it, is read after the wait
+  if (a.mask_mode == kMaskMLP && !a.net_on_stream) filt::load_filter(T, a.filter, t, NT);
   dependents_may_launch();
   wait_for_earlier_kernels();
+  if (a.mask_mode == kMaskMLP && a.net_on_stream) filt::load_filter(T, a.filter, t, NT);
 
   // dt of an RK3 step (stage 1 computes it from max(|u|+c), max(|v|+c)), by the
   // last warp, which has the fewest cells, into shared memory until step 3.

@@ -55,6 +55,7 @@ void build_net_blob(const NetF64& net, void* blob);
 struct RhsArgs {
   const double* net64;  // blob: transposed binary64 parameters
   const float* filter;  // blob: filter table
+  int net_on_stream;    // the blob is written by kernels launched just before on the stream
   const double* U;   // state the right-hand side is evaluated on
   const double* U0;  // state at the start of the RK3 step (stages 2, 3)
   double* out;       // dU/dt (stage 0) or the next stage state; null: mask_out alone

@@ -167,6 +167,7 @@ extern "C" int neno6_step_noalloc(const neno6_config* cfg, const double* net_par
   std::memset(&a, 0, sizeof a);
   a.net64 = blob;
   a.filter = reinterpret_cast<const float*>(blob + kNetParams);
+  a.net_on_stream = 1;
   double d[4];
   scheme_tables(c.linear_weights, d, a.cand, a.wtab);
   a.nx = c.nx;
