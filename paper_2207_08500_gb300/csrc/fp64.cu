@@ -690,15 +690,17 @@ float round16(float x, uint16_t& bits) {
   std::memcpy(&bits, &h, 2);
   return __half2float(h);
 }
-// v = hi + lo + error in binary16 terms of v's FP32 rounding
+// v as two binary16 terms of its FP32 rounding: what they miss, |hi| + |lo|, |lo|
 struct Split {
   uint16_t hi, lo;
-  double error;
+  double error, size, low;
 };
 Split split_terms(double v) {
   Split s;
   const float f = (float)v, h = round16(f, s.hi), l = round16(f - h, s.lo);
   s.error = std::fabs(v - (double)h - (double)l);
+  s.low = std::fabs((double)l);
+  s.size = std::fabs((double)h) + s.low;
   return s;
 }
 
@@ -744,42 +746,43 @@ static void build_filter_kappa(const NetF64& net, FilterKappa& out, Split* split
   float* dst[5] = {out.in, out.h1, out.h2, out.h3, out.h4};
   for (int l = 4; l >= 0; --l) {
     const int n = W[l], m = W[l + 1];
-    const int T = 3 * ((n + 15) / 16);  // matrix instructions per output (layers 2-5)
-    double A[2048], D[2048] = {};  // |w|, its split error
+    const int blocks = (n + 15) / 16;  // of inputs (layers 2-5)
+    const double c = 2.0 * ((n < 16 ? n : 16) + 2);  // units u an instruction may lose
+    double A[2048];  // |w|
     for (int o = 0; o < m; ++o)
       for (int i = 0; i < n; ++i) {
         A[o * n + i] = aw(l, o, i);
-        if (l == 0) continue;
-        const Split s = split[off[l] + o * n + i] = split_terms(net.p[off[l] + o * n + i] * (l == 4 ? out.scale[o] : 1.0));
-        D[o * n + i] = s.error;
+        if (l > 0) split[off[l] + o * n + i] = split_terms(net.p[off[l] + o * n + i] * (l == 4 ? out.scale[o] : 1.0));
       }
     double worst[64] = {};
     for (int k = 0; k < 4; ++k) {
-      double dw[64] = {};
+      double own[64] = {};  // layers 2-5: the unit's coefficient
       for (int i = 0; i < n; ++i) Gn[k][i] = 0.0;
       for (int o = 0; o < m; ++o) {
-        const double g = G[k][o], gs = l == 4 ? g / out.scale[k] : g;  // G holds the scale already
+        const double g = G[k][o], gs = l == 4 ? g / out.scale[k] : g;  // G and layer 5's terms hold the scale already
         for (int i = 0; i < n; ++i) {
           Gn[k][i] += g * A[o * n + i];
-          dw[i] += gs * D[o * n + i];
+          if (l == 0) continue;
+          const Split& w = split[off[l] + o * n + i];
+          // the block's instruction, the additions from it on and the input's
+          // split, the weight's split, the dropped product
+          own[i] += gs * ((c + blocks - i / 16 + 2) * u * w.size + w.error + w.low / 2048.0);
+          k0[k] += gs * gap * (w.size + w.low);
         }
+        if (l > 0) k0[k] += gs * 4 * blocks * tiny;
       }
       for (int i = 0; i < n; ++i) {
-        const double g = Gn[k][i];
-        double c;
+        double e = own[i];
         if (l == 0) {  // the i-th FMA of the chain and those after it, the weight's and the input's rounding
-          c = (n - i + 1 + 8) * u * g;
-          k0[k] += g * tiny;
-        } else {  // the instructions from its block on, its split and the dropped product, the weight's split
-          c = (4 * (T - 3 * (i / 16)) + 2) * u * g + dw[i];
-          k0[k] += g * gap;
+          e = (n - i + 1 + 8) * u * Gn[k][i];
+          k0[k] += Gn[k][i] * tiny;
         }
-        worst[i] = std::fmax(worst[i], c == c ? c : INFINITY);  // a NaN weight: nothing is certified
+        worst[i] = std::fmax(worst[i], e == e ? e : INFINITY);  // a NaN weight: nothing is certified
       }
     }
     for (int i = 0; i < n; ++i) dst[l][i] = up(worst[i]);
     for (int k = 0; k < 4; ++k)
-      for (int o = 0; o < m; ++o) k0[k] += (l == 0 ? n + 1 : 4 * T + 1) * u * G[k][o] * ab(l, o);
+      for (int o = 0; o < m; ++o) k0[k] += (l == 0 ? n + 1 : blocks + 1) * u * G[k][o] * ab(l, o);
     for (int k = 0; k < 4; ++k)
       for (int i = 0; i < n; ++i) G[k][i] = Gn[k][i];
   }

@@ -10,32 +10,47 @@
 // binary64 network's, always.
 //
 // Each FP32 value v of layers 2 to 5 (weights and inputs) is split into two
-// binary16 terms, v = hi + lo + d with |d| <= u |v| + 2^-25, u = 2^-24, and a
-// product is hi hi' + lo hi' + hi lo': warp-level matrix instructions (16 rows x
-// 8 outputs x 16 inputs, three per block of 16 inputs), whose operands and
-// results stay in registers.  They fit this kernel: a warp's 64 rows (32 faces,
-// two sides) need no barrier, no tensor memory and no wait on other warps, and
-// at 2 clocks per instruction and SM they take a quarter of the FP64 time beside
-// which they run.  2048^2 RHS: 11.69 ms, against 13.8 ms with every layer in FP32
-// on the CUDA cores (weights by broadcast loads, which bound it).
+// binary16 terms, v = hi + lo + d, and a product is hi hi' + lo hi' + hi lo':
+// warp-level matrix instructions (16 rows x 8 outputs x 16 inputs, three per block
+// of 16 inputs), whose operands and results stay in registers.  They fit this
+// kernel: a warp's 64 rows (32 faces, two sides) need no barrier, no tensor memory
+// and no wait on other warps, and at 2 clocks per instruction and SM they take a
+// quarter of the FP64 time beside which they run.  2048^2 RHS: 11.70 ms, against
+// 13.8 ms with every layer in FP32 on the CUDA cores (weights by broadcast loads,
+// which bound it).
 //
 // The bound (forward error analysis, Higham, "Accuracy and Stability of
-// Numerical Algorithms", ch. 3).  Layer 1: a bias and six FMAs on weights
-// rounded to FP32 differ from the exact value of the same inputs x by at most
+// Numerical Algorithms", ch. 3), u = 2^-24.  Layer 1: a bias and six FMAs on
+// weights rounded to FP32 differ from the exact value of the same inputs x by at
+// most
 //   sum_j (6 - j + 2) u |w_j| |x_j| + 7 u |b|,   j = 1..6.
-// A layer above: T matrix instructions in turn on one accumulator that starts
-// at the bias; each is taken to add at most 4 u times the magnitudes it sums
-// (the products and the accumulator; products of binary16 values are exact, the
-// sums are kept to at least 24 bits and truncated: Fasi, Higham, Mikaitis and
-// Pranesh, "Numerical behavior of NVIDIA tensor cores", PeerJ CS 7:e330; 1.7 u
-// is the largest seen on this GPU).  An input j of block k is in T - 3 k of
-// them, so with dw the weight's split error and 2 u for the input's and the
-// dropped lo lo' the unit is off by at most
-//   sum_j ((4 (T - 3 k_j) + 2) u |w_j| + dw_j) |h_j| + 2^-25 sum_j |w_j| + (4 T + 1) u |b|
-// up to O(u^2).  ReLU does not enlarge a difference, and layers l+1..5 carry one
-// of layer l to logit k multiplied by at most G_l = |W5| ... |W_{l+1}|.  Summed
-// over the layers the bound is linear in the computed hidden values (all >= 0)
-// and inputs:
+// A layer above takes its inputs in blocks of 16; a block's sum starts at 0, takes
+// the products with a lo term in two instructions, those of the hi terms in a
+// third, and is added to the blocks before it, which start at the bias.
+//  * Splitting: binary16 keeps 11 bits, so lo is at most 2^-11 |v| and d at most
+//    2 u |v| + 2^-25 (hi + lo need not reach 24 bits: 1 + 2^-12 + 2^-23).  Of the
+//    weight both are known, |lo| and dw; with s = |hi| + |lo| of the weight a product
+//    is off by 2 u s |h| for the input's split, dw |h| for the weight's, and
+//    2^-11 |lo| |h| for the dropped lo lo'; besides 2^-25 (s + |lo|).
+//  * An instruction sums the accumulator and at most 16 products, themselves exact.
+//    All that is promised is at least single precision, in any order and with any
+//    rounding.  Additions one after the other, cut off at 24 bits, lose 2 u each, 16
+//    of them; addends aligned to the largest and cut off at its 24 bits (Fasi,
+//    Higham, Mikaitis and Pranesh, "Numerical behavior of NVIDIA tensor cores",
+//    PeerJ CS 7:e330) lose 2 u of it each, 17 of them, and 2 u for the result.  So it
+//    loses at most 36 u (n inputs in a block below 16: 2 (n + 2) u) of the magnitudes
+//    it sums.  The first two work on magnitudes 2^-10 of the third's: only that one
+//    counts.  Were all three to work on the layer's whole sum, as they may, a layer
+//    of 64 inputs would lose 432 u: 2.5 times as many rows would stay undecided
+//    (200 x 136: 189 us, 153 as it is).
+//  * Of B blocks an addition rounds block k and those before it, B - k times.
+// Together the unit is off by at most
+//   sum_j ((36 + B - k_j + 2) u s_j + dw_j + 2^-11 |lo_j|) |h_j|
+//     + 2^-25 sum_j (s_j + |lo_j|) + (B + 1) u |b|
+// up to O(u^2) and relative 2^-8.  ReLU does not enlarge a difference, and layers
+// l+1..5 carry one of layer l to logit k multiplied by at most
+// G_l = |W5| ... |W_{l+1}|.  Summed over the layers the bound is linear in the
+// computed hidden values (all >= 0) and inputs:
 //   |error of logit k| <= k0 + sum_j kin_j |x_j| + sum_l sum_i kappa_l,i h_l,i,
 // one more FMA per hidden unit.  The coefficients (build_filter_kappa, on the
 // host in binary64) take the maximum over the four logits after dividing
@@ -43,8 +58,9 @@
 // changes no sign and makes one bound serve all four.  They include the
 // input's conversion (8 u relative: two truncations to 24 bits, a reciprocal
 // to 1 ulp and a product), underflow (every |w|, |b| counted as at least
-// 2^-125) and a factor 1.01 for the O(u^2) terms, the binary64 network's own
-// rounding (2^-29 of the bound) and the rounding of the bound itself.
+// 2^-125, and 2^-125 for each of a block's four sums) and a factor 1.01 for the
+// O(u^2) and 2^-8 terms, the binary64 network's own rounding (2^-28 of the bound)
+// and the rounding of the bound itself.
 // A row whose inputs leave [0, 2^100], or any of whose logits or whose bound
 // is not finite (a value outside the binary16 range makes it so), is never
 // certified.
@@ -117,26 +133,38 @@ __device__ __forceinline__ void split16(float x, float y, uint32_t& hi, uint32_t
 }
 // One block of 16 inputs (pairs p: rows g, g + 8 of inputs 2q.., then of 2q + 8..)
 // into NT tiles of 8 outputs of both row tiles: T points at the block's weights,
-// per tile and lane hi b0, b1, lo b0, b1.
+// per tile and lane hi b0, b1, lo b0, b1.  The block's sum starts at 0 and takes
+// the small terms first; see the bound above.
 template <int NT>
 __device__ __forceinline__ void block16(float (&acc)[2][NT][4], const uint32_t (&hi)[2][4], const uint32_t (&lo)[2][4],
                                         const float* T, int lane) {
   uint4 b[NT];
+  float s[NT][2][4];
 #pragma unroll
-  for (int nt = 0; nt < NT; ++nt) b[nt] = reinterpret_cast<const uint4*>(T)[32 * nt + lane];
-  // term by term: the instructions on one accumulator are 2 NT apart
+  for (int nt = 0; nt < NT; ++nt) {
+    b[nt] = reinterpret_cast<const uint4*>(T)[32 * nt + lane];
 #pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) mma16(acc[mt][nt], hi[mt], b[nt].x, b[nt].y);
-#pragma unroll
-  for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) mma16(acc[mt][nt], lo[mt], b[nt].x, b[nt].y);
+    for (int mt = 0; mt < 2; ++mt) s[nt][mt][0] = s[nt][mt][1] = s[nt][mt][2] = s[nt][mt][3] = 0.0f;
+  }
+  // term by term: the instructions on one sum are 2 NT apart
 #pragma unroll
   for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt) mma16(acc[mt][nt], hi[mt], b[nt].z, b[nt].w);
+    for (int mt = 0; mt < 2; ++mt) mma16(s[nt][mt], lo[mt], b[nt].x, b[nt].y);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) mma16(s[nt][mt], hi[mt], b[nt].z, b[nt].w);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) mma16(s[nt][mt], hi[mt], b[nt].x, b[nt].y);
+#pragma unroll
+  for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) acc[mt][nt][r] += s[nt][mt][r];
 }
 // Accumulators start at the biases of their outputs.
 template <int NT>
