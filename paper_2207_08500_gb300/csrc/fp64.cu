@@ -99,10 +99,12 @@ __device__ __forceinline__ void warp_umax(unsigned long long& x, unsigned long l
   }
 }
 
-// x / 2 for x = 0 or 2^-1021 <= |x| < inf, on the integer pipe.
+// x / 2 for x = 0 or |x| >= 2^-1021, infinities and NaN (rows of L where rounding
+// leaves a Roe state without a sound speed), on the integer pipe.
 __device__ __forceinline__ double half_exact(double x) {
   const int hi = __double2hiint(x);
-  return __hiloint2double((hi & 0x7ff00000) ? hi - 0x00100000 : hi, __double2loint(x));
+  const bool scale = (unsigned)(hi & 0x7ff00000) - 0x00100000u < 0x7fe00000u;
+  return __hiloint2double(scale ? hi - 0x00100000 : hi, __double2loint(x));
 }
 
 // Roe-averaged state of a face (Sec. 4.4).
