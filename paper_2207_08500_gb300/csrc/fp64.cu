@@ -202,9 +202,9 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
   // last warp, which has the fewest cells, into shared memory until step 3.
   double* sdt = smem + G::O_D;
   if (a.stage && warp == NT / 32 - 1) {
-    const double tm = *a.t_dev;
     double dt;
     if (a.stage == 1) {
+      const double tm = *a.t_dev;
       // maxima over the reduction's CTAs
       unsigned long long mx = 0, my = 0;
       for (int i = lane; i < a.nsmax; i += 32) {
@@ -216,13 +216,8 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
       if (NDIM == 2) s = __dadd_rn(s, __ddiv_rn(__longlong_as_double((long long)my), a.dy));
       dt = __ddiv_rn(a.cfl, s);
       if (a.t_end > 0.0 && __dadd_rn(tm, dt) > a.t_end) dt = __dsub_rn(a.t_end, tm);
-      if (blockIdx.x == 0 && lane == 0) {
-        *a.dt_dev = dt;
-        if (a.dt_user) *a.dt_user = dt;
-      }
     } else {
       dt = *a.dt_dev;
-      if (a.stage == 3 && blockIdx.x == 0 && lane == 0) *a.t_dev = __dadd_rn(tm, dt);
     }
     if (lane == 0) *sdt = dt;
   }
@@ -232,6 +227,16 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
   int tile = (int)blockIdx.x;
   do {
     const int i0 = tile % ntx * TX, j0 = tile / ntx * TY;
+    if (tile == 0 && a.stage && t == NT - 32) {
+      // by whichever CTA has the first tile (block 0 may be one that was handed
+      // out), the thread that formed dt
+      const double dt = *sdt;
+      if (a.stage == 1) {
+        *a.dt_dev = dt;
+        if (a.dt_user) *a.dt_user = dt;
+      }
+      if (a.stage == 3) *a.t_dev = __dadd_rn(*a.t_dev, dt);
+    }
     // ---- 1. tile + halo (without its corners) and per-cell quantities.
     // `odd`: some value is not 0 or in [2^-60, 2^60), or a cell is not
     // physical; the tile's faces then take every operation of the
