@@ -378,8 +378,8 @@ const char* neno6_last_error(const neno6_handle* h);
  *
  * Scratch: one file-scope static device array holding two stage states of at
  * most NENO6_NOALLOC_MAX_STATE_ELEMS float64 values each (4 MiB each) plus
- * the call's network (39 KB), wave-speed maxima (19 KB) and a few words; every GPU that loads the library holds it (8 MiB) until the
- * process exits.  Every call shares it and it keeps the previous call's
+ * the call's network (39 KB), wave-speed maxima (19 KB) and a few words; every
+ * GPU that loads the library holds it (8 MiB) until the process exits.  Every call shares it and it keeps the previous call's
  * contents; the call clears what must start at zero.  Calls whose work
  * overlaps on the GPU (different streams, or different host threads) race on
  * it and must be serialised by the caller.  The first call on a device looks
@@ -389,6 +389,9 @@ const char* neno6_last_error(const neno6_handle* h);
  * a device reset (or a release of the primary context) the next call sees a
  * new context id and looks the address up again, so that call too should
  * come before any stream capture.
+ * On the host every call with mask_mode NENO6_MASK_MLP lays its network out anew
+ * (about 60 us, on the stack: some 90 KB, no heap) and sends it with two small
+ * kernels; neno6_step does that once, in neno6_create.
  *
  *   cfg          host pointer: grid and scheme (precision must be NENO6_FP64);
  *                nv * nx * ny must not exceed NENO6_NOALLOC_MAX_STATE_ELEMS.

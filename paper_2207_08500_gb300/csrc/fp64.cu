@@ -28,7 +28,6 @@
 #include <cmath>
 #include <cstring>
 #include <utility>
-#include <vector>
 
 #include "fp64_ops.cuh"
 #include "internal.h"
@@ -697,14 +696,16 @@ float round16(float x, uint16_t& bits) {
   std::memcpy(&bits, &h, 2);
   return __half2float(h);
 }
-// v as two binary16 terms of its FP32 rounding: what they miss, |hi| + |lo|, |lo|
-struct Split {
+// The binary16 terms of v's FP32 rounding, and what they miss, |hi| + |lo|, |lo|
+struct Terms {
   uint16_t hi, lo;
+};
+struct Split {
   double error, size, low;
 };
-Split split_terms(double v) {
+Split split_terms(double v, Terms& t) {
   Split s;
-  const float f = (float)v, h = round16(f, s.hi), l = round16(f - h, s.lo);
+  const float f = (float)v, h = round16(f, t.hi), l = round16(f - h, t.lo);
   s.error = std::fabs(v - (double)h - (double)l);
   s.low = std::fabs((double)l);
   s.size = std::fabs((double)h) + s.low;
@@ -714,8 +715,8 @@ Split split_terms(double v) {
 }  // namespace
 
 // Coefficients of the filter's bound (mlp_filter.cuh).
-// `split`: the terms of the weights of layers 2 to 5 (layer 5 scaled), filled in.
-static void build_filter_kappa(const NetF64& net, FilterKappa& out, Split* split) {
+// `terms`: those of the weights of layers 2 to 5 (layer 5 scaled), filled in.
+static void build_filter_kappa(const NetF64& net, FilterKappa& out, Terms* terms) {
   constexpr int W[6] = {6, 64, 32, 16, 8, 4};
   constexpr int off[5] = {0, 448, 2528, 3056, 3192};
   const double u = 1.0 / 16777216.0, tiny = std::ldexp(1.0, -125), gap = std::ldexp(1.0, -25);
@@ -755,41 +756,44 @@ static void build_filter_kappa(const NetF64& net, FilterKappa& out, Split* split
     const int n = W[l], m = W[l + 1];
     const int blocks = (n + 15) / 16;  // of inputs (layers 2-5)
     const double c = 2.0 * ((n < 16 ? n : 16) + 2);  // units u an instruction may lose
-    double A[2048];  // |w|
-    for (int o = 0; o < m; ++o)
-      for (int i = 0; i < n; ++i) {
-        A[o * n + i] = aw(l, o, i);
-        if (l > 0) split[off[l] + o * n + i] = split_terms(net.p[off[l] + o * n + i] * (l == 4 ? out.scale[o] : 1.0));
-      }
-    double worst[64] = {};
-    for (int k = 0; k < 4; ++k) {
-      double own[64] = {};  // layers 2-5: the unit's coefficient
+    double own[4][64] = {};  // coefficients of the layer's inputs, per logit
+    for (int k = 0; k < 4; ++k)
       for (int i = 0; i < n; ++i) Gn[k][i] = 0.0;
-      for (int o = 0; o < m; ++o) {
-        const double g = G[k][o], gs = l == 4 ? g / out.scale[k] : g;  // G and layer 5's terms hold the scale already
-        for (int i = 0; i < n; ++i) {
-          Gn[k][i] += g * A[o * n + i];
-          if (l == 0) continue;
-          const Split& w = split[off[l] + o * n + i];
-          // the block's instruction, the additions from it on and the input's
-          // split, the weight's split, the dropped product
-          own[i] += gs * ((c + blocks - i / 16 + 2) * u * w.size + w.error + w.low / 2048.0);
-          k0[k] += gs * gap * (w.size + w.low);
-        }
-        if (l > 0) k0[k] += gs * 4 * blocks * tiny;
+    for (int o = 0; o < m; ++o) {
+      double gs[4];  // G, and layer 5's terms, hold the scale already
+      for (int k = 0; k < 4; ++k) {
+        gs[k] = l == 4 ? G[k][o] / out.scale[k] : G[k][o];
+        k0[k] += (l == 0 ? n + 1 : blocks + 1) * u * G[k][o] * ab(l, o);
+        if (l > 0) k0[k] += gs[k] * 4 * blocks * tiny;
       }
       for (int i = 0; i < n; ++i) {
-        double e = own[i];
+        const double a = aw(l, o, i);
+        for (int k = 0; k < 4; ++k) Gn[k][i] += G[k][o] * a;
+        if (l == 0) continue;
+        const double v = net.p[off[l] + o * n + i];
+        const Split w = split_terms(l == 4 ? v * out.scale[o] : v, terms[off[l] + o * n + i]);
+        // the block's instruction, the additions from it on and the input's
+        // split, the weight's split, the dropped product
+        const double e = (c + blocks - i / 16 + 2) * u * w.size + w.error + w.low / 2048.0;
+        const double abs = gap * (w.size + w.low);
+        for (int k = 0; k < 4; ++k) {
+          own[k][i] += gs[k] * e;
+          k0[k] += gs[k] * abs;
+        }
+      }
+    }
+    for (int i = 0; i < n; ++i) {
+      double worst = 0.0;
+      for (int k = 0; k < 4; ++k) {
+        double e = own[k][i];
         if (l == 0) {  // the i-th FMA of the chain and those after it, the weight's and the input's rounding
           e = (n - i + 1 + 8) * u * Gn[k][i];
           k0[k] += Gn[k][i] * tiny;
         }
-        worst[i] = std::fmax(worst[i], e == e ? e : INFINITY);  // a NaN weight: nothing is certified
+        worst = std::fmax(worst, e == e ? e : INFINITY);  // a NaN weight: nothing is certified
       }
+      dst[l][i] = up(worst);
     }
-    for (int i = 0; i < n; ++i) dst[l][i] = up(worst[i]);
-    for (int k = 0; k < 4; ++k)
-      for (int o = 0; o < m; ++o) k0[k] += (l == 0 ? n + 1 : blocks + 1) * u * G[k][o] * ab(l, o);
     for (int k = 0; k < 4; ++k)
       for (int i = 0; i < n; ++i) G[k][i] = Gn[k][i];
   }
@@ -798,12 +802,13 @@ static void build_filter_kappa(const NetF64& net, FilterKappa& out, Split* split
   out.k0 = up(worst);
 }
 
+// No heap: the allocation-free step calls it.
 void build_net_blob(const NetF64& net, void* blob) {
   constexpr int W[6] = {6, 64, 32, 16, 8, 4};
   constexpr int kW[5] = {0, kFiltW2, kFiltW3, kFiltW4, kFiltW5}, kB[5] = {0, kFiltB2, kFiltB3, kFiltB4, kFiltB5};
   FilterKappa k;
-  std::vector<Split> split(kNetParams);
-  build_filter_kappa(net, k, split.data());
+  Terms terms[kNetParams];
+  build_filter_kappa(net, k, terms);
   double* Wt = static_cast<double*>(blob);
   float* T = reinterpret_cast<float*>(Wt + kNetParams);
   for (int i = 0; i < kFiltFloats; ++i) T[i] = 0.0f;
@@ -824,8 +829,8 @@ void build_net_blob(const NetF64& net, void* blob) {
         const int tiles = (nout + 7) / 8, in = i % 16;
         uint16_t* at = reinterpret_cast<uint16_t*>(T + kW[l] + 128 * ((i / 16) * tiles + o / 8) +
                                                    4 * (4 * (o % 8) + in % 8 / 2) + in / 8) + in % 2;
-        at[0] = split[p + o * nin + i].hi;
-        at[4] = split[p + o * nin + i].lo;
+        at[0] = terms[p + o * nin + i].hi;
+        at[4] = terms[p + o * nin + i].lo;
       }
       const double b = net.p[p + nin * nout + o];
       Wt[p + nin * nout + o] = b;

@@ -152,14 +152,11 @@ extern "C" int neno6_step_noalloc(const neno6_config* cfg, const double* net_par
   if (c.mask_mode == NENO6_MASK_MLP) {
     NetF64 net;
     std::memcpy(net.p, net_params, sizeof net.p);
-    double img[kBlob];
-    build_net_blob(net, img);
-    for (size_t at = 0; at < kBlob; at += kChunk) {
-      Chunk ch;
-      const int n = (int)(kBlob - at < kChunk ? kBlob - at : kChunk);
-      std::memcpy(ch.v, img + at, n * sizeof(double));
-      put_chunk_kernel<<<1, 256, 0, s>>>(ch, blob + at, n);
-    }
+    Chunk ch[2];  // the blob in two pieces, one after the other
+    static_assert(sizeof ch >= kNetBlobBytes, "the blob's pieces");
+    build_net_blob(net, ch);
+    put_chunk_kernel<<<1, 256, 0, s>>>(ch[0], blob, (int)kChunk);
+    put_chunk_kernel<<<1, 256, 0, s>>>(ch[1], blob + kChunk, (int)(kBlob - kChunk));
     e = cudaGetLastError();
     if (e != cudaSuccess) return NENO6_ERR_CUDA;
   }
