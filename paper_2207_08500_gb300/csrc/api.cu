@@ -822,7 +822,7 @@ int neno6_rhs_vjp(neno6_handle* h, const double* U, const double* lambda, const 
     a.U = U;
     a.mask_out = h->d_mask;
     a.stage = 0;
-      e = launch_rhs_fp64(h->cfg.ndim, a, s);
+    e = launch_rhs_fp64(h->cfg.ndim, a, s);
     if (e != cudaSuccess) return cuda_fail(h, e, "rhs_vjp: forward");
     mask = h->d_mask;
   }

@@ -3,7 +3,6 @@
 #pragma once
 
 #include <cstdint>
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 namespace neno6 {
