@@ -522,9 +522,9 @@ PRECISION_NOTE = {
 # DRAM bytes (read + write) of one launch of the dominant kernel(s), from one
 # ncu capture of the current kernels at the grid named (dram__bytes_read.sum
 # + dram__bytes_write.sum, a single-pass capture); other grids: None
-TRAFFIC = {True: (2048, 135598080 + 107458304),
+TRAFFIC = {True: (2048, 135122944 + 106195200),
            False: (4096, 1077111296 + 1047517440 + 1074123776 + 507575552)}
-TRAFFIC_NOTE = {True: "rhs_fp64_kernel at 2048^2, one launch: 135.6 MB read + 107.5 MB written",
+TRAFFIC_NOTE = {True: "rhs_fp64_kernel at 2048^2, one launch: 135.1 MB read + 106.2 MB written",
                 False: "one RHS at 4096^2: faces_mixed_kernel 1077.1 MB read + 1047.5 MB written, "
                        "diff_mixed_kernel 1074.1 MB read + 507.6 MB written"}
 

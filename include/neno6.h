@@ -390,7 +390,7 @@ const char* neno6_last_error(const neno6_handle* h);
  * new context id and looks the address up again, so that call too should
  * come before any stream capture.
  * On the host every call with mask_mode NENO6_MASK_MLP lays its network out anew
- * (about 60 us, on the stack: some 90 KB, no heap) and sends it with two small
+ * (40 to 60 us, on the stack: some 90 KB, no heap) and sends it with two small
  * kernels; neno6_step does that once, in neno6_create.
  *
  *   cfg          host pointer: grid and scheme (precision must be NENO6_FP64);

@@ -20,7 +20,7 @@
 // wrap or zero-gradient copy done in the load) and the per-cell quantities are
 // staged in shared memory, the faces' fluxes written back there and
 // differenced, with no scratch in global memory.  Comparisons (ReLU, max, |x|)
-// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 11.4 ms,
+// run on the integer pipe on the bit patterns.  Measured, 2048^2 RHS: 11.7 ms,
 // against 437 ms with every classifier row in binary64 and four lanes per
 // face; the FP64 operations alone would take 7.9 ms of a full FP64 pipe.
 #include <cuda_fp16.h>
@@ -499,7 +499,8 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
     __syncthreads();
     // Tiles are handed out: a CTA takes over one that has not been launched yet.
     // Rows evaluated again in binary64 make tiles uneven, and an SM's two CTAs do
-    // not advance evenly (2048^2 11.69 ms dealt out beforehand, 11.42 handed out).
+    // not advance evenly (2048^2 11.69 ms dealt out beforehand, 11.42 handed out, both
+    // before the filter's blocks had sums of their own, 11.67 since).
     if (t == 0 && gridDim.x > G::kResident) tc::try_cancel(&s_next, &s_nbar);
     if (G::SPLIT && a.out) {
       const double* sG = smem + G::O_G;
@@ -674,8 +675,9 @@ cudaError_t dependent_launch(void (*kern)(P...), unsigned grid, unsigned block, 
 
 namespace {
 
-// Round x to binary16 (nearest even); returns its value.  The table takes
-// 60 us of a solver's creation so, 115 with the library's host conversions.
+// Round x to binary16 (nearest even); returns its value.  The table takes 41 us of
+// a solver's creation on the GPU's Arm host; the library's host conversions would
+// add some 55.
 float round16(float x, uint16_t& bits) {
   uint32_t b;
   std::memcpy(&b, &x, 4);
@@ -874,8 +876,9 @@ cudaError_t launch_rhs_fp64(int ndim, RhsArgs& a, cudaStream_t s) {
   // for 7 x 16.  The smaller the grid, the smaller the tile, so that every SM
   // has warps; the smallest grids give a warp a single field.  Measured in us
   // per RHS, periodic quadrants (threads x CTAs per SM; * taken; tiles dealt out
-  // beforehand, handed out the starred ones take 327 at 300^2, 807 at 512^2, 2951
-  // at 1024^2 and 11420 at 2048^2):
+  // beforehand and the filter's sums one per layer.  Handed out, and a sum per block,
+  // the starred ones take 327 at 300^2, 545 at 400^2, 824 at 512^2, 1474 at 700^2,
+  // 3018 at 1024^2 and 11670 at 2048^2):
   //                        24x16 64x64 100x100 200x136 300x300 400x400 512^2 700^2 1024^2 2048^2
   //   15 x 16       256x2   209   135    140     142     350     551    822* 1467*  3034*  11696*
   //   15 x 16       192x2   236   154            161                    848         3107   12058

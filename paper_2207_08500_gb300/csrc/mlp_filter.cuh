@@ -41,7 +41,7 @@
 //    loses at most 36 u (n inputs in a block below 16: 2 (n + 2) u) of the magnitudes
 //    it sums.  The first two work on magnitudes 2^-10 of the third's: only that one
 //    counts.  Were all three to work on the layer's whole sum, as they may, a layer
-//    of 64 inputs would lose 432 u: 2.5 times as many rows would stay undecided
+//    of 64 inputs would lose 432 u: about three times as many rows would stay undecided
 //    (200 x 136: 189 us, 153 as it is).
 //  * Of B blocks an addition rounds block k and those before it, B - k times.
 // Together the unit is off by at most
