@@ -757,7 +757,7 @@ static void build_filter_kappa(const NetF64& net, FilterKappa& out, Terms* terms
   for (int l = 4; l >= 0; --l) {
     const int n = W[l], m = W[l + 1];
     const int blocks = (n + 15) / 16;  // of inputs (layers 2-5)
-    const double c = 2.0 * ((n < 16 ? n : 16) + 2);  // units u an instruction may lose
+    const double c = 2.5 * (n < 16 ? n : 16);  // units u an instruction may lose
     double own[4][64] = {};  // coefficients of the layer's inputs, per logit
     for (int k = 0; k < 4; ++k)
       for (int i = 0; i < n; ++i) Gn[k][i] = 0.0;

@@ -32,20 +32,22 @@
 //    weight both are known, |lo| and dw; with s = |hi| + |lo| of the weight a product
 //    is off by 2 u s |h| for the input's split, dw |h| for the weight's, and
 //    2^-11 |lo| |h| for the dropped lo lo'; besides 2^-25 (s + |lo|).
-//  * An instruction sums the accumulator and at most 16 products, themselves exact.
-//    All that is promised is at least single precision, in any order and with any
-//    rounding.  Additions one after the other, cut off at 24 bits, lose 2 u each, 16
-//    of them; addends aligned to the largest and cut off at its 24 bits (Fasi,
-//    Higham, Mikaitis and Pranesh, "Numerical behavior of NVIDIA tensor cores",
-//    PeerJ CS 7:e330) lose 2 u of it each, 17 of them, and 2 u for the result.  So it
-//    loses at most 36 u (n inputs in a block below 16: 2 (n + 2) u) of the magnitudes
-//    it sums.  The first two work on magnitudes 2^-10 of the third's: only that one
-//    counts.  Were all three to work on the layer's whole sum, as they may, a layer
-//    of 64 inputs would lose 432 u: about three times as many rows would stay undecided
-//    (200 x 136: 189 us, 153 as it is).
+//  * An instruction sums the accumulator and at most n = 16 products (8 in layer 5),
+//    themselves exact.  All that is promised is at least single precision, in any
+//    order and with any rounding.  Additions one after the other, cut off at 24 bits,
+//    lose 2 u each, n of them.  Sums of a group of addends, aligned to the largest and
+//    cut off below its 24 bits, are what has been found (Fasi, Higham, Mikaitis and
+//    Pranesh, "Numerical behavior of NVIDIA tensor cores", PeerJ CS 7:e330), in groups
+//    of 4, 8 or 16 products and the sum before: the largest is kept whole, the others
+//    lose 2 u of it each, and 2 u for the group's result, (2 n + 2 n / 4) u at most.
+//    So an instruction loses at most 40 u (20 u) of the magnitudes it sums.  The first
+//    two work on magnitudes 2^-10 of the third's: only that one counts.  Were all
+//    three to work on the layer's whole sum, as they may, a layer of 64 inputs would
+//    lose twelve times as much: three times as many rows would stay undecided (200 x
+//    136 with 36 u each: 189 us, 153 with a sum per block).
 //  * Of B blocks an addition rounds block k and those before it, B - k times.
 // Together the unit is off by at most
-//   sum_j ((36 + B - k_j + 2) u s_j + dw_j + 2^-11 |lo_j|) |h_j|
+//   sum_j ((40 + B - k_j + 2) u s_j + dw_j + 2^-11 |lo_j|) |h_j|
 //     + 2^-25 sum_j (s_j + |lo_j|) + (B + 1) u |b|
 // up to O(u^2) and relative 2^-8.  ReLU does not enlarge a difference, and layers
 // l+1..5 carry one of layer l to logit k multiplied by at most

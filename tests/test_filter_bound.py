@@ -2,12 +2,13 @@
 sign, against an emulation of the filter on the CPU.
 
 The matrix instructions promise their sums in at least single precision, in any
-order and with any rounding.  The two weakest readings are emulated: addends
-aligned to the largest and cut off below its 24 bits, and additions one after
-the other, each cut off at 24 bits.  The distance to the binary64 network has to
-stay within the bound for either, on the trained network and on networks built
-for the worst: a large sum that many small addends are added to, and values just
-above powers of two, whose two binary16 terms leave the most behind.
+order and with any rounding.  The weakest readings are emulated: additions one
+after the other, each cut off at 24 bits, and sums of groups of 4, 8 or 16 products
+with the sum before, aligned to the largest addend and cut off below its 24 bits.
+The distance to the binary64 network has to stay within the bound for each, on the
+trained network and on networks built for the worst: a large addend that many small
+ones are added to, and values just above powers of two, whose two binary16 terms
+leave the most behind.
 """
 import ctypes
 
@@ -63,16 +64,18 @@ def cut(v, e=None):
     return np.trunc(v / unit) * unit
 
 
-def instruction(acc, a, b, model):
-    """acc [row][out] + sum over inputs of a [row][in] b [out][in]."""
-    add = np.concatenate([acc[:, :, None], a[:, None, :] * b[None]], axis=2)
-    if model == "aligned":
+def instruction(acc, a, b, group):
+    """acc [row][out] + sum over inputs of a [row][in] b [out][in], in groups of
+    products aligned with the sum before, or one after the other (group 1)."""
+    prod = a[:, None, :] * b[None]
+    for i in range(0, prod.shape[2], group):
+        if group == 1:
+            acc = cut(acc + prod[:, :, i])
+            continue
+        add = np.concatenate([acc[:, :, None], prod[:, :, i:i + group]], axis=2)
         e = np.frexp(add)[1].max(axis=2, where=add != 0.0, initial=-200)
-        return cut(cut(add, e[:, :, None]).sum(axis=2))
-    s = add[:, :, 0]
-    for i in range(1, add.shape[2]):
-        s = cut(s + add[:, :, i])
-    return s
+        acc = cut(cut(add, e[:, :, None]).sum(axis=2))
+    return acc
 
 
 def split(h):
@@ -85,7 +88,7 @@ def f32(v):
     return v.astype(np.float32).astype(np.float64)
 
 
-def filtered(net, X, model):
+def filtered(net, X, group):
     """Logits (scaled as the table scales them) and the bound, as the kernel
     forms them, and the scales."""
     T = table(net)
@@ -111,7 +114,7 @@ def filtered(net, X, model):
             s = slice(k, k + 16)
             block = np.zeros(acc.shape)
             for a, b in ((lo, whi), (hi, wlo), (hi, whi)):
-                block = instruction(block, a[:, s], b[:, s], model)
+                block = instruction(block, a[:, s], b[:, s], group)
             acc = f32(acc + block)
         if l < 4:
             h = np.maximum(acc, 0.0)
@@ -162,11 +165,11 @@ def networks():
             yield "%s %+d" % (kind, sign), worst_net(kind, sign)
 
 
-@pytest.mark.parametrize("model", ["aligned", "one after the other"])
-def test_no_error_beyond_the_bound(oracle_mod, model):
+@pytest.mark.parametrize("group", [1, 4, 8, 16])
+def test_no_error_beyond_the_bound(oracle_mod, group):
     X = np.concatenate([synth.mlp_stencils(500, seed=73), 1e-3 * synth.mlp_stencils(100, seed=74)])
     for name, net in networks():
-        z, bound, scale = filtered(net, X, model)
+        z, bound, scale = filtered(net, X, group)
         z64 = logits64(net, X) * scale
         ok = np.isfinite(z64)  # a scale that a bias of 0 hides is not compared
         # the scale is read off an FP32 bias: 2 u of the logit
