@@ -561,7 +561,11 @@ __global__ void __launch_bounds__(G::NT, G::OCC) rhs_fp64_kernel(const __grid_co
     tc::fence_async_smem();
     // the next tile's cells overwrite what the difference reads
     if (__syncthreads_or(lost)) {
-      if (t == 0) atomicOr(a.status, 4);
+      if (t == 0) {
+        atomicOr(a.status, 4);
+        // the answer may still be on its way into this CTA's memory
+        tc::mbar_wait(&s_nbar, nphase ^ 1u);
+      }
       break;
     }
   } while (tile >= 0);
