@@ -708,7 +708,11 @@ __global__ void __launch_bounds__(kMlpThreads, 8) faces_mixed_kernel(const __gri
   }
   if (*fail_flag && t == 0) {
     atomicOr(a.status, 4);
-    if (gridDim.x > kResident && blk >= 0) drain_blocks(smem + kOffNext, next_bar, nphase);
+    // (after a timeout the answer may still be on its way into this CTA's memory)
+    if (gridDim.x > kResident && mbar_wait(next_bar, nphase ^ 1u) && cancelled_block(smem + kOffNext) >= 0) {
+      fence_async_smem();
+      drain_blocks(smem + kOffNext, next_bar, nphase);
+    }
   }
   tc_fence_before();
   __syncthreads();
