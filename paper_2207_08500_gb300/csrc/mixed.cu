@@ -105,9 +105,10 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
     if (HANDOUT && t == 0) {
       if (!asked) try_cancel(&s_answer, &s_nbar);
       asked = true;
-      if (!mbar_wait(&s_nbar, nphase)) s_fail = 1;
+      s_next = -1;
+      if (mbar_wait(&s_nbar, nphase)) s_next = cancelled_block(&s_answer);
+      else s_fail = 1;
       nphase ^= 1u;
-      s_next = cancelled_block(&s_answer);
     }
     __syncthreads();
     // read between this barrier and the classifier's: thread 0 writes the word
@@ -126,9 +127,12 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
       if (t == 0) atomicOr(status, 4);
       // copies may still be in flight: wait for them (bounded) before leaving
       if (!HANDOUT || next >= 0) rows.get(tile, x);
-      if (HANDOUT && t == 0 && next >= 0 && mbar_wait(&s_nbar, nphase) && cancelled_block(&s_answer) >= 0) {
-        fence_async_smem();
-        drain_blocks(&s_answer, &s_nbar, nphase ^ 1u);
+      if (HANDOUT && t == 0) {
+        if (next < 0) nphase ^= 1u;  // nothing asked since the last answer
+        if (mbar_wait(&s_nbar, nphase) && cancelled_block(&s_answer) >= 0) {
+          fence_async_smem();
+          drain_blocks(&s_answer, &s_nbar, nphase ^ 1u);
+        }
       }
       break;
     }
