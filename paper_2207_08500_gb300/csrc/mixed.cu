@@ -95,7 +95,8 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
     const long long r = tile * 128 + t;
     float x[6];
     float m = 1.0f;
-    if (!rows.get(tile, x)) s_fail = 1;
+    const bool got = rows.get(tile, x);
+    if (!got) s_fail = 1;
 #pragma unroll
     for (int j = 0; j < 6; ++j) m = fmaxf(m, fabsf(x[j]));
 #pragma unroll
@@ -116,9 +117,9 @@ __global__ void __launch_bounds__(kMlpThreads) classify_mixed_kernel(const doubl
     // not have got to the end of this one
     if (HANDOUT) next = s_next;
     if (!HANDOUT) {
-      if (t == 0) rows.fetch(tile + gridDim.x);
+      if (t == 0 && got) rows.fetch(tile + gridDim.x);
     } else if (t == 0 && next >= 0) {
-      rows.fetch(next);
+      if (got) rows.fetch(next);
       fence_async_smem();
       try_cancel(&s_answer, &s_nbar);
     }

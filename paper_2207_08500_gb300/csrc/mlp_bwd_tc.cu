@@ -169,7 +169,8 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     // ---- Eq. (normalizainput) in FP32
     const unsigned lab = live ? y[s] : 0u;
     float x0[6], m = 1.0f;
-    if (!rows.get(tile, x0)) *fail = 1;
+    const bool got = rows.get(tile, x0);
+    if (!got) *fail = 1;
 #pragma unroll
     for (int j = 0; j < 6; ++j) m = fmaxf(m, fabsf(x0[j]));
 #pragma unroll
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kT, 2) mlp_bwd_tc_kernel(const double* __restr
     // ---- layer 1 (bias on the ones columns) -> H1
     if (t == 0) {
       issue_layer<BF16>(mc, smem + kOffX0, 16, kNetImageB1, 64, (int)kColD1);
-      rows.fetch(tile + gridDim.x);
+      if (got) rows.fetch(tile + gridDim.x);
     }
     wait_layer(mc);
     uint32_t mask1[2] = {0u, 0u};

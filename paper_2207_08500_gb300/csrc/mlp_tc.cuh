@@ -296,7 +296,8 @@ struct TileRows {
   uint64_t* bar;
   uint32_t phase;
   bool bulk;
-  // thread 0, once every thread has read the rows before
+  // thread 0, once every thread has read the rows before (not after a timeout: one
+  // copy at a time)
   __device__ __forceinline__ void fetch(long long tile) {
     const long long rows = n - tile * 128 < 128 ? n - tile * 128 : 128;
     if (!bulk || rows <= 0) return;
@@ -309,7 +310,7 @@ struct TileRows {
     bool ok = true;
     if (bulk) {
       ok = mbar_wait(bar, phase);
-      phase ^= 1u;
+      phase ^= ok ? 1u : 0u;  // a copy that has not come is waited for again
       const double2* b = reinterpret_cast<const double2*>(buf) + 3 * threadIdx.x;
 #pragma unroll
       for (int j = 0; j < 3; ++j) {
